@@ -164,6 +164,10 @@ __device__ __noinline__ void invert_sub32(const T* blk, int ld, int cw, T* out, 
   T x[32];
 #pragma unroll
   for (int i = 0; i < 32; i++) {
+    if (i >= cw) {   // (a root's last sub-block: rows past cw lie past the factor's storage)
+      x[i] = (i == lane) ? T(1) : T(0);
+      continue;
+    }
     T a0 = T(0), a1 = T(0);
 #pragma unroll
     for (int k = 0; k + 1 < i; k += 2) {
