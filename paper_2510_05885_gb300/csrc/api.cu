@@ -90,18 +90,22 @@ struct Level {
   int64_t tsyrk_tiles = 0;
   int64_t tsyrk_tp_off = 0;
   int tsyrk_stages = 1;
-  int64_t chain_off = 0;  // block-row items of the level (sweeps)
+  // triangular sweeps: the level's supernodes by role (sweep.cu)
+  int64_t narrow_off = 0, block_off = 0;
+  int narrow_cnt = 0, block_cnt = 0, block_below = 0;
+  // strips of the large ones: pivot rows and rows below (forward), columns
+  // of L21 and of the pivot block (backward); vec: most entries of a strip's
+  // vector
+  struct Strips {
+    int64_t off = 0;
+    int cnt = 0, vec = 0;
+  } prow, brow, bcol, pcol;
+  bool multi = false;        // some supernode of the level has more than CHAIN_ROWS pivots
+  int64_t chain_off = 0;     // FP64: block-rows of those supernodes
   int chain_cnt = 0;
-  int64_t chain_smem = 0; // dynamic shared memory of the chained sweep kernels
-  bool chain_multi = false;  // some supernode of the level has more than one block-row
-  int64_t below_off = 0;  // (s, a0) solve items
-  int below_cnt = 0;
-  int64_t bbelow_off = 0; // (s, a0, k0) backward solve items
-  int bbelow_cnt = 0;
-  int bbelow_narrow = 0;  //   the first ones: supernodes of at most 32 columns (one warp each)
   int64_t dag_off = 0;    // tasks of the persistent large-front launch
   int dag_cnt = 0;
-  Cost asm_cost, small_cost, syrk_cost, fdiag_cost, fbelow_cost, bdiag_cost, bbelow_cost, dag_cost;
+  Cost asm_cost, small_cost, syrk_cost, one_cost, diag_cost, below_cost, dag_cost;   // one: narrow and block supernodes
 };
 
 struct KStat {
@@ -118,16 +122,13 @@ struct Pending {
 std::atomic<int64_t> g_kernel_launches{0};
 
 struct HostSched {
-  std::vector<int2> asmv, belowv;
+  std::vector<int2> asmv;
   std::vector<int32_t> smallv;
-  std::vector<int4> chainv;               // (supernode, first block-row, first 32-row block, 0) per block-row (sweeps)
-  std::vector<int32_t> chain_pptr;        // per global 32-row pivot block: its run of child ranges
-  std::vector<int4> chain_pran;           // (child, alo, ahi, 0): child W entries landing on the block
-  int64_t nblocks = 0;                    // 32-row pivot blocks in all
-  int64_t nbrows = 0;                     // block-rows of the chained sweeps in all
-  std::vector<int4> bbelowv;              // (s, a0, k0, 0): backward below-rows items, 256 columns each
-  std::vector<int32_t> below_cptr;        // per below-rows solve item: its run of child ranges
-  std::vector<int4> below_cran;           // (child, lo, hi, 0)
+  // triangular sweeps (sweep.cu): supernodes by role, strips of the large ones
+  std::vector<int32_t> narrowv, blockv;
+  std::vector<int4> stripv;
+  std::vector<int2> chainv;               // (supernode, first block-row flag) per block-row of the wide ones
+  int64_t nbrows = 0;                     // block-row flags in all
   std::vector<int32_t> asm_cptr;          // per assembly item: its run of child row ranges
   std::vector<int4> asm_cran;             // (child, alo, ahi, 0)
   std::vector<int4> panelv;
@@ -141,7 +142,6 @@ struct HostSched {
   std::vector<int32_t> tc_fronts;
   int64_t split_max = 0;
   std::vector<int8_t> sn_flags;
-  std::vector<int64_t> sn_Ioff;
   // persistent large-front factorisation: tasks of every level, and the
   // counters they wait on (one queue head per level, then the fronts'
   // tile and row-task counters)
@@ -152,10 +152,22 @@ struct HostSched {
   // most 32 pivots all of whose descendants have at most 32 (one warp per
   // maximal subtree); the level launches skip them
   std::vector<int8_t> inreg;
-  std::vector<int32_t> regnodes;          // each subtree's supernodes in postorder
-  std::vector<int2> regitems;             // (first node, count) per subtree
+  std::vector<int32_t> regnodes;          // each subtree's supernodes level by level (children first)
+  std::vector<int4> regitems;             // (first node, nodes, first level bound, levels) per subtree
+  std::vector<int32_t> regbounds;         // per subtree: its levels' offsets into its nodes, and the end
   Cost reg_fwd_cost, reg_bwd_cost, reg_fac_cost;
-  std::vector<int2> invv;                 // (large front, 32-column sub-block): inverses after the factorisation
+  // inverses of the pivot blocks after the factorisation (invert.cu): diagonal
+  // blocks (supernode, first column) of at most 64 and at most 128 columns,
+  // and the tiles of the merges of wider blocks (FP32), width by width
+  std::vector<int2> inv64, inv128;
+  std::vector<int4> mergev;
+  struct Merge {
+    int h;
+    int64_t off;
+    int cnt;
+  };
+  std::vector<Merge> merges;
+  Cost inv_cost, merge_cost;
   int64_t reg_smem = 0;                   // dynamic shared memory of the subtree factorisation
 };
 
@@ -194,19 +206,15 @@ struct ncl_kkt_s {
   GemmProb* d_probs = nullptr;
   int32_t* d_tilep = nullptr;
   int32_t* d_tilep_tc = nullptr;
-  int4* d_chain = nullptr;
-  int32_t* d_chain_pptr = nullptr;
-  int4* d_chain_pran = nullptr;
-  int* d_chain_sync = nullptr;              // tickets (fwd, bwd) then flags (fwd, bwd) of the pivot blocks
-  int2* d_below = nullptr;
-  int4* d_bbelow = nullptr;
-  int32_t* d_below_cptr = nullptr;
-  int4* d_below_cran = nullptr;
+  int32_t* d_narrow = nullptr;
+  int32_t* d_block = nullptr;
+  int4* d_strips = nullptr;
+  int2* d_chain = nullptr;
+  int* d_chain_sync = nullptr;              // tickets (fwd, bwd) then flags (fwd, bwd) of the block-rows
   // solve workspace
   void* xp = nullptr;
   void* own_xp = nullptr;                  // the handle's own sweep workspace
   void* W = nullptr;
-  void* Pw = nullptr;
   double* R = nullptr;
   double* jx = nullptr;
   double* jg = nullptr;
@@ -227,8 +235,11 @@ struct ncl_kkt_s {
   CUtensorMap* d_maps = nullptr;           // 4 tensor maps per tensor-core front
   TcProb* d_tc = nullptr;
   int* d_err = nullptr;                    // device error flags (bounded waits)
-  int2* d_invv = nullptr;                  // sub-blocks whose inverses follow the factorisation
-  int2* d_regitems = nullptr;              // small-subtree sweep items and their nodes
+  int2* d_inv64 = nullptr;                 // pivot blocks inverted after the factorisation
+  int2* d_inv128 = nullptr;
+  int4* d_merge = nullptr;
+  int4* d_regitems = nullptr;              // small subtrees, their nodes and level bounds
+  int32_t* d_regbounds = nullptr;
   int32_t* d_regnodes = nullptr;
   DagTask* d_dag = nullptr;                // persistent large-front tasks
   int* d_dag_cnt = nullptr;                //   their queue heads and counters
@@ -326,7 +337,6 @@ void build_schedule(ncl_kkt_s* h) {
   const size_t esz = is_fp32(h) ? 4 : 8;
   HostSched& hs = h->hs;
   std::vector<int2>& asmv = hs.asmv;
-  std::vector<int2>& belowv = hs.belowv;
   std::vector<int32_t>& smallv = hs.smallv;
   std::vector<int4>& panelv = hs.panelv;
   std::vector<GemmProb>& probv = hs.probv;
@@ -335,7 +345,8 @@ void build_schedule(ncl_kkt_s* h) {
   const int PNB = MACRO_NB;   // pivot columns per panel step
   hs.dagv.clear();
   hs.dag_counters = (int64_t)P.nlevels;   // one queue head per level first
-  hs.invv.clear();
+  hs.inv64.clear();
+  hs.inv128.clear();
   hs.inreg.assign(P.ns, 0);
   hs.regnodes.clear();
   hs.regitems.clear();
@@ -364,10 +375,18 @@ void build_schedule(ncl_kkt_s* h) {
         pre.push_back(v);
         for (int32_t k = P.child_ptr[v]; k < P.child_ptr[v + 1]; k++) stack.push_back(P.child_list[k]);
       }
-      // reversed preorder (node after its children, children pushed in
-      // order) is a postorder
-      for (auto it = pre.rbegin(); it != pre.rend(); ++it) hs.regnodes.push_back(*it);
-      hs.regitems.push_back(make_int2(first, (int32_t)pre.size()));
+      // level by level (a supernode's level is its height, so children come
+      // first), reversed preorder within a level
+      std::reverse(pre.begin(), pre.end());
+      std::stable_sort(pre.begin(), pre.end(), [&](int32_t a, int32_t b) { return P.sn_level[a] < P.sn_level[b]; });
+      const int32_t lptr = (int32_t)hs.regbounds.size();
+      for (size_t q = 0; q < pre.size(); q++) {
+        if (q == 0 || P.sn_level[pre[q]] != P.sn_level[pre[q - 1]]) hs.regbounds.push_back((int32_t)q);
+        hs.regnodes.push_back(pre[q]);
+      }
+      const int32_t nlev = (int32_t)hs.regbounds.size() - lptr;
+      hs.regbounds.push_back((int32_t)pre.size());
+      hs.regitems.push_back(make_int4(first, (int32_t)pre.size(), lptr, nlev));
     }
     // largest subtrees first: the kernels hand subtrees out in item order
     // (a work counter), so the longest ones start early and the tail is short
@@ -381,7 +400,7 @@ void build_schedule(ncl_kkt_s* h) {
       std::vector<size_t> ord(hs.regitems.size());
       for (size_t i = 0; i < ord.size(); i++) ord[i] = i;
       std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b) { return wgt[a] > wgt[b]; });
-      std::vector<int2> sorted(ord.size());
+      std::vector<int4> sorted(ord.size());
       for (size_t i = 0; i < ord.size(); i++) sorted[i] = hs.regitems[ord[i]];
       hs.regitems.swap(sorted);
     }
@@ -412,12 +431,7 @@ void build_schedule(ncl_kkt_s* h) {
   }
   hs.sn_Soff.assign(P.ns, -1);
   hs.sn_flags.assign(P.ns, 0);
-  hs.sn_Ioff.assign(P.ns + 1, 0);
   hs.asm_cptr.assign(1, 0);
-  hs.chain_pptr.assign(1, 0);
-  hs.below_cptr.assign(1, 0);
-  for (int32_t s = 0; s < P.ns; s++)
-    hs.sn_Ioff[s + 1] = hs.sn_Ioff[s] + (int64_t)((P.sn_ncol[s] + 31) / 32) * 1024;
   // problems of one launch are pushed consecutively; each launch's tiles map
   // to its problems through a contiguous run of the per-tile index arrays
   auto push_gemm = [&](GemmProb g, int64_t prob_base, int64_t& tiles, Cost& c) {
@@ -451,9 +465,10 @@ void build_schedule(ncl_kkt_s* h) {
     Level& L = h->levels[l];
     L.asm_off = (int64_t)asmv.size();
     L.small_off = (int64_t)smallv.size();
+    L.narrow_off = (int64_t)hs.narrowv.size();
+    L.block_off = (int64_t)hs.blockv.size();
     L.chain_off = (int64_t)hs.chainv.size();
-    L.below_off = (int64_t)belowv.size();
-    L.bbelow_off = (int64_t)hs.bbelowv.size();
+    std::vector<int4> prow, brow, bcol, pcol;
     std::vector<int32_t> large, small;
     for (int32_t k = P.level_ptr[l]; k < P.level_ptr[l + 1]; k++) {
       const int32_t s = P.level_list[k];
@@ -474,45 +489,40 @@ void build_schedule(ncl_kkt_s* h) {
         }
         hs.asm_cptr.push_back((int32_t)hs.asm_cran.size());
       }
-      {
-        // block-rows of the chained sweeps (every item of the supernode
-        // carries its first block-row and first 32-row block) and, per
-        // 32-row block, the children's W entries that land on its rows
-        const int nblk = (ncol + 31) / 32, nbr = (ncol + CHAIN_ROWS - 1) / CHAIN_ROWS;
-        if (!hs.inreg[s]) {
-          for (int B = 0; B < nbr; B++) hs.chainv.push_back(make_int4(s, (int32_t)hs.nbrows, (int32_t)hs.nblocks, 0));
-          L.chain_smem = std::max<int64_t>(L.chain_smem, chain_smem(std::min(CHAIN_ROWS, ncol), (int)esz));
-          if (nbr > 1) L.chain_multi = true;
-        }
-        for (int b = 0; b < nblk; b++) {
-          const int lo = 32 * b, hi = std::min(32 * b + 32, ncol);
-          for (int32_t k2 = P.child_ptr[s]; k2 < P.child_ptr[s + 1]; k2++) {
-            const int32_t c = P.child_list[k2];
-            const int32_t* rel = P.relmap.data() + P.relmap_off[c];
-            const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
-            const int alo = (int)(std::lower_bound(rel, rel + nbc, lo) - rel);
-            const int ahi = (int)(std::lower_bound(rel, rel + nbc, hi) - rel);
-            if (ahi > alo) hs.chain_pran.push_back(make_int4(c, alo, ahi, 0));
+      if (!reg) {
+        // role in the sweeps: a warp, a CTA, or strips.  A warp streams up to
+        // 4096 entries below its pivots and a CTA 96 KB of front (2 to 3 us
+        // each, hidden by the level's other supernodes); larger fronts are
+        // spread over CTAs, 16 KB to 64 KB of factor to a strip.
+        const int nb = nrow - ncol;
+        if (ncol <= 32 && (int64_t)nb * ncp <= 4096) {
+          hs.narrowv.push_back(s);
+        } else if (ncol <= CHAIN_ROWS && (int64_t)nrow * ncp * (int64_t)esz <= SWEEP_BLOCK_BYTES &&
+                   nb <= SWEEP_BLOCK_BELOW) {
+          hs.blockv.push_back(s);
+          L.block_below = std::max(L.block_below, nb);
+        } else {
+          const int rows = std::max(16, std::min(128, 16384 / ncp / 16 * 16));
+          const bool chain = esz == 8 && ncol > CHAIN_ROWS;
+          for (int r0 = (ncol - 1) / rows * rows; r0 >= 0 && !chain; r0 -= rows) {   // longest rows first
+            prow.push_back(make_int4(s, r0, std::min(r0 + rows, ncol), 0));
+            L.prow.vec = std::max(L.prow.vec, std::min(r0 + rows, ncol));
           }
-          hs.chain_pptr.push_back((int32_t)hs.chain_pran.size());
+          for (int r0 = ncol; r0 < nrow; r0 += rows) brow.push_back(make_int4(s, r0, std::min(r0 + rows, nrow), 0));
+          for (int j0 = 0; j0 < ncol; j0 += 16) {
+            if (nb > 0) bcol.push_back(make_int4(s, j0, 0, 0));
+            if (!chain) pcol.push_back(make_int4(s, j0, 0, 0));
+          }
+          if (nb > 0) L.brow.vec = std::max(L.brow.vec, ncol);
+          L.bcol.vec = std::max(L.bcol.vec, nb);
+          if (!chain) L.pcol.vec = std::max(L.pcol.vec, ncol);
+          if (ncol > CHAIN_ROWS) {
+            const int nbr = (ncol + CHAIN_ROWS - 1) / CHAIN_ROWS;
+            for (int B = 0; B < nbr; B++) hs.chainv.push_back(make_int2(s, (int32_t)hs.nbrows));
+            hs.nbrows += nbr;
+            L.multi = true;
+          }
         }
-        hs.nblocks += nblk;
-        hs.nbrows += nbr;
-      }
-      for (int a0 = 0; a0 < nrow - ncol && !hs.inreg[s]; a0 += SOLVE_ROWS) {
-        belowv.push_back(make_int2(s, a0));
-        for (int k0 = 0; k0 < ncol; k0 += 256) hs.bbelowv.push_back(make_int4(s, a0, k0, 0));
-        // the children's W entries that land on the rows [a0, a1) below
-        const int a1 = std::min(a0 + SOLVE_ROWS, nrow - ncol);
-        for (int32_t k2 = P.child_ptr[s]; k2 < P.child_ptr[s + 1]; k2++) {
-          const int32_t c = P.child_list[k2];
-          const int32_t* rel = P.relmap.data() + P.relmap_off[c];
-          const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
-          const int lo = (int)(std::lower_bound(rel, rel + nbc, ncol + a0) - rel);
-          const int hi = (int)(std::lower_bound(rel, rel + nbc, ncol + a1) - rel);
-          if (hi > lo) hs.below_cran.push_back(make_int4(c, lo, hi, 0));
-        }
-        hs.below_cptr.push_back((int32_t)hs.below_cran.size());
       }
       const bool is_small = ncol <= 64 && nrow <= 512 && (int64_t)nrow * ncp * (int64_t)esz <= SMALL_SMEM;
       if (reg) {
@@ -538,28 +548,37 @@ void build_schedule(ncl_kkt_s* h) {
         L.small_cost.flops += 2.0 * (ncol * (double)ncol * ncol / 3.0 + nb * ncol * ncol);
         L.small_cost.bytes += esz * 2.0 * nrow * ncp;
       }
-      if (!hs.inreg[s]) {
-        L.fdiag_cost.bytes += esz * 0.5 * ncol * (ncol + 1.0);
-        L.fdiag_cost.flops += (double)ncol * ncol;
-        L.fbelow_cost.bytes += esz * nb * ncol;
-        L.fbelow_cost.flops += 2.0 * nb * ncol;
-        L.bdiag_cost = L.fdiag_cost;
-        L.bbelow_cost.bytes += esz * nb * ncol;
-        L.bbelow_cost.flops += 2.0 * nb * ncol;
+      if (!reg) {
+        const bool strips = !(hs.narrowv.size() && hs.narrowv.back() == s) && !(hs.blockv.size() && hs.blockv.back() == s);
+        Cost& cd = strips ? L.diag_cost : L.one_cost;
+        Cost& cb = strips ? L.below_cost : L.one_cost;
+        cd.bytes += esz * 0.5 * ncol * (ncol + 1.0);
+        cd.flops += (double)ncol * ncol;
+        cb.bytes += esz * nb * ncol;
+        cb.flops += 2.0 * nb * ncol;
+        // inverses: the fronts kept in shared memory with one sub-block have theirs
+        if (ncol > 1 && !(is_small && ncol <= 32)) {
+          for (int b = 0; b < ncol; b += CHAIN_ROWS) (ncol <= 64 ? hs.inv64 : hs.inv128).push_back(make_int2(s, b));
+          const double w = std::min(ncol, CHAIN_ROWS), q = (ncol + CHAIN_ROWS - 1) / CHAIN_ROWS;
+          hs.inv_cost.flops += q * w * w * w / 3.0;
+          hs.inv_cost.bytes += q * esz * w * w;
+        }
       }
     }
     L.asm_cnt = (int)(asmv.size() - L.asm_off);
     L.small_cnt = (int)(smallv.size() - L.small_off);
+    L.narrow_cnt = (int)(hs.narrowv.size() - L.narrow_off);
+    L.block_cnt = (int)(hs.blockv.size() - L.block_off);
     L.chain_cnt = (int)(hs.chainv.size() - L.chain_off);
-    L.below_cnt = (int)(belowv.size() - L.below_off);
-    L.bbelow_cnt = (int)(hs.bbelowv.size() - L.bbelow_off);
-    {
-      // the items of supernodes with at most 32 columns first (a warp each),
-      // then the others (a CTA each), each group in supernode order
-      auto b0 = hs.bbelowv.begin() + L.bbelow_off;
-      auto mid = std::stable_partition(b0, hs.bbelowv.end(), [&](const int4& it) { return P.sn_ncol[it.x] <= 32; });
-      L.bbelow_narrow = (int)(mid - b0);
-    }
+    auto put = [&](Level::Strips& S, const std::vector<int4>& v) {
+      S.off = (int64_t)hs.stripv.size();
+      S.cnt = (int)v.size();
+      hs.stripv.insert(hs.stripv.end(), v.begin(), v.end());
+    };
+    put(L.prow, prow);
+    put(L.brow, brow);
+    put(L.bcol, bcol);
+    put(L.pcol, pcol);
     if (hs.tc) {
       int64_t off = 0;
       for (int32_t s : large) {
@@ -573,7 +592,6 @@ void build_schedule(ncl_kkt_s* h) {
     }
     for (int32_t s : large) {
       hs.sn_flags[s] = 1;
-      for (int b = 0; b < (P.sn_ncol[s] + 31) / 32; b++) hs.invv.push_back(make_int2(s, b));
     }
     int maxm = 0;
     for (int32_t s : large) maxm = std::max(maxm, (P.sn_ncol[s] + PNB - 1) / PNB);
@@ -749,6 +767,24 @@ void build_schedule(ncl_kkt_s* h) {
     L.syrk_cnt = (int)(probv.size() - L.syrk_off);
     L.tsyrk_cnt = (int)(hs.tcv.size() - L.tsyrk_off);
   }
+  // FP32: merges of the inverted diagonal blocks of 128, 256, ... columns
+  hs.mergev.clear();
+  hs.merges.clear();
+  hs.inv_cost = hs.merge_cost = Cost{};
+  if (is_fp32(h))
+    for (int w = CHAIN_ROWS; w < P.max_pivots; w *= 2) {
+      HostSched::Merge M{w, (int64_t)hs.mergev.size(), 0};
+      for (int32_t s = 0; s < P.ns; s++)
+        for (int q0 = 0; q0 + w < P.sn_ncol[s]; q0 += 2 * w) {
+          const int m = std::min(w, P.sn_ncol[s] - q0 - w);
+          for (int i = 0; i < (m + 127) / 128; i++)
+            for (int n = 0; n < w / 64; n++) hs.mergev.push_back(make_int4(s, q0, i, n));
+          hs.merge_cost.flops += (double)m * w * w + (double)m * m * w;
+          hs.merge_cost.bytes += 4.0 * (3.0 * m * w + 0.5 * w * w + 0.5 * m * m);
+        }
+      M.cnt = (int)(hs.mergev.size() - M.off);
+      hs.merges.push_back(M);
+    }
   // bounds of every launch item against its buffers, checked on the host
   // before anything runs on the device
   {
@@ -776,13 +812,22 @@ void build_schedule(ncl_kkt_s* h) {
             bad("assembly map");
       }
     }
-    if (hs.chain_pptr.size() != (size_t)hs.nblocks + 1 || hs.chainv.size() > (size_t)hs.nbrows) bad("pivot blocks");
     // the small-subtree region: every node once, in a subtree of its own
     // region, children before parents within it, at most 32 pivots
     {
       std::vector<int> seen(P.ns, 0);
-      for (const int2& it : hs.regitems) {
+      for (const int4& it : hs.regitems) {
         if (it.x < 0 || it.y <= 0 || (size_t)(it.x + it.y) > hs.regnodes.size()) bad("subtree item");
+        if (it.z < 0 || it.w <= 0 || (size_t)(it.z + it.w) >= hs.regbounds.size() || hs.regbounds[it.z] != 0 ||
+            hs.regbounds[it.z + it.w] != it.y)
+          bad("subtree levels");
+        for (int l = 0; l < it.w; l++) {
+          const int q0 = hs.regbounds[it.z + l], q1 = hs.regbounds[it.z + l + 1];
+          if (q0 < 0 || q1 <= q0 || q1 > it.y) bad("subtree levels");
+          for (int q = q0; q < q1; q++)   // a level's parents lie in later levels
+            if (q + 1 < q1 && P.sn_level[hs.regnodes[it.x + q]] != P.sn_level[hs.regnodes[it.x + q + 1]])
+              bad("subtree levels");
+        }
         for (int q = 0; q < it.y; q++) {
           const int32_t v = hs.regnodes[it.x + q];
           if (v < 0 || v >= P.ns || !hs.inreg[v] || P.sn_ncol[v] > 32 || seen[v]++) bad("subtree node");
@@ -798,31 +843,67 @@ void build_schedule(ncl_kkt_s* h) {
                             small_front_smem(P.sn_nrow[v], P.sn_ncolp[v], (int)esz) > hs.reg_smem))
           bad("subtree front");
     }
-    for (size_t i = 0; i < hs.chainv.size(); i++) {
-      const int4 it = hs.chainv[i];
-      if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.y + (P.sn_ncol[it.x] + CHAIN_ROWS - 1) / CHAIN_ROWS > hs.nbrows ||
-          it.z < 0 || it.z + (P.sn_ncol[it.x] + 31) / 32 > hs.nblocks)
-        bad("pivot blocks");
-    }
-    for (const Level& L : h->levels)
-      if (L.chain_smem > chain_smem(CHAIN_ROWS, (int)esz)) bad("chain shared memory");
-    for (int64_t g = 0; g < hs.nblocks; g++) {
-      if (hs.chain_pptr[g] > hs.chain_pptr[g + 1] || hs.chain_pptr[g + 1] > (int32_t)hs.chain_pran.size())
-        bad("pivot block ranges");
-    }
-    for (size_t i = 0; i < hs.chainv.size(); i++) {
-      const int4 it = hs.chainv[i];
-      const int nblk = (P.sn_ncol[it.x] + 31) / 32;
-      for (int b = 0; b < nblk; b++)
-        for (int32_t e = hs.chain_pptr[it.z + b]; e < hs.chain_pptr[it.z + b + 1]; e++) {
-          const int4 cr = hs.chain_pran[e];
-          if (cr.x < 0 || cr.x >= P.ns || P.sn_parent[cr.x] != it.x || cr.y < 0 || cr.y >= cr.z ||
-              cr.z > P.sn_nrow[cr.x] - P.sn_ncol[cr.x])
-            bad("pivot block ranges");
-          const int32_t* rel = P.relmap.data() + P.relmap_off[cr.x];
-          if (rel[cr.y] < 32 * b || rel[cr.z - 1] >= std::min(32 * b + 32, (int)P.sn_ncol[it.x])) bad("pivot block ranges");
+    for (const int2& it : hs.chainv)
+      if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.y + (P.sn_ncol[it.x] + CHAIN_ROWS - 1) / CHAIN_ROWS > hs.nbrows)
+        bad("block-rows");
+    // sweeps: every supernode outside the region once, in a role that fits it
+    {
+      std::vector<int8_t> seen(P.ns, 0);
+      for (int32_t s : hs.narrowv)
+        if (s < 0 || s >= P.ns || hs.inreg[s] || seen[s]++ || P.sn_ncol[s] > 32) bad("narrow supernode");
+      for (const Level& L : h->levels)
+        for (int i = 0; i < L.block_cnt; i++) {
+          const int32_t s = hs.blockv[L.block_off + i];
+          if (s < 0 || s >= P.ns || hs.inreg[s] || seen[s]++ || P.sn_ncol[s] > CHAIN_ROWS ||
+              P.sn_nrow[s] - P.sn_ncol[s] > std::min(L.block_below, SWEEP_BLOCK_BELOW))
+            bad("block supernode");
         }
+      // strips: rows and columns of each large supernode covered exactly once
+      std::vector<int64_t> pr(P.ns, 0), br(P.ns, 0), bc(P.ns, 0), pc(P.ns, 0);
+      for (const Level& L : h->levels) {
+        auto each = [&](const Level::Strips& S, auto f) {
+          if (S.off < 0 || S.off + S.cnt > (int64_t)hs.stripv.size()) bad("strips");
+          for (int i = 0; i < S.cnt; i++) {
+            const int4 it = hs.stripv[S.off + i];
+            if (it.x < 0 || it.x >= P.ns || hs.inreg[it.x] || seen[it.x]) bad("strip");
+            f(it, P.sn_ncol[it.x], P.sn_nrow[it.x]);
+          }
+        };
+        each(L.prow, [&](int4 it, int nc, int) {
+          if (it.y < 0 || it.z <= it.y || it.z > nc || it.z > L.prow.vec) bad("pivot row strip");
+          pr[it.x] += it.z - it.y;
+        });
+        each(L.brow, [&](int4 it, int nc, int nr) {
+          if (it.y < nc || it.z <= it.y || it.z > nr || nc > L.brow.vec) bad("row strip");
+          br[it.x] += it.z - it.y;
+        });
+        each(L.bcol, [&](int4 it, int nc, int nr) {
+          if (it.y < 0 || it.y >= nc || it.y % 16 || nr - nc > L.bcol.vec) bad("column strip");
+          bc[it.x] += std::min(16, nc - it.y);
+        });
+        each(L.pcol, [&](int4 it, int nc, int) {
+          if (it.y < 0 || it.y >= nc || it.y % 16 || nc > L.pcol.vec) bad("pivot column strip");
+          pc[it.x] += std::min(16, nc - it.y);
+        });
+      }
+      for (int32_t s = 0; s < P.ns; s++) {
+        if (hs.inreg[s] || seen[s]) continue;
+        const int64_t nc = P.sn_ncol[s], nb = P.sn_nrow[s] - nc, piv = (esz == 8 && nc > CHAIN_ROWS) ? 0 : nc;
+        if (pr[s] != piv || pc[s] != piv || br[s] != nb || bc[s] != (nb > 0 ? nc : 0)) bad("strip coverage");
+      }
     }
+    for (const auto* v : {&hs.inv64, &hs.inv128})
+      for (const int2& it : *v)
+        if (it.x < 0 || it.x >= P.ns || hs.inreg[it.x] || it.y < 0 || it.y >= P.sn_ncol[it.x] || it.y % CHAIN_ROWS ||
+            (v == &hs.inv64 && P.sn_ncol[it.x] > 64))
+          bad("inverse item");
+    for (const HostSched::Merge& M : hs.merges)
+      for (int i = 0; i < M.cnt; i++) {
+        const int4 it = hs.mergev[M.off + i];
+        if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.y % (2 * M.h) || it.y + M.h >= P.sn_ncol[it.x] || it.z < 0 ||
+            128 * it.z >= std::min(M.h, P.sn_ncol[it.x] - it.y - M.h) || it.w < 0 || 64 * it.w >= M.h)
+          bad("inverse merge");
+      }
     if (hs.asm_cptr.size() != asmv.size() + 1) bad("assembly child ranges");
     for (size_t i = 0; i < asmv.size(); i++) {
       const int2 it = asmv[i];
@@ -834,29 +915,6 @@ void build_schedule(ncl_kkt_s* h) {
         if (cr.x < 0 || cr.x >= P.ns || P.sn_parent[cr.x] != it.x || cr.y < 0 || cr.y >= cr.z ||
             cr.z > P.sn_nrow[cr.x] - P.sn_ncol[cr.x])
           bad("assembly child ranges");
-      }
-    }
-    for (const int4& it : hs.bbelowv)
-      if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.y >= P.sn_nrow[it.x] - P.sn_ncol[it.x] || it.y % SOLVE_ROWS ||
-          it.z < 0 || it.z >= P.sn_ncol[it.x] || it.z % 256)
-        bad("solve item");
-    for (const Level& L : h->levels)
-      for (int i = 0; i < L.bbelow_cnt; i++)
-        if ((i < L.bbelow_narrow) != (P.sn_ncol[hs.bbelowv[L.bbelow_off + i].x] <= 32)) bad("narrow solve items");
-    if (hs.below_cptr.size() != belowv.size() + 1) bad("solve child ranges");
-    for (size_t i = 0; i < belowv.size(); i++) {
-      const int2 it = belowv[i];
-      if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.y >= P.sn_nrow[it.x] - P.sn_ncol[it.x]) bad("solve item");
-      if (hs.below_cptr[i] > hs.below_cptr[i + 1] || hs.below_cptr[i + 1] > (int32_t)hs.below_cran.size())
-        bad("solve child ranges");
-      const int a1 = std::min(it.y + SOLVE_ROWS, P.sn_nrow[it.x] - P.sn_ncol[it.x]);
-      for (int32_t e = hs.below_cptr[i]; e < hs.below_cptr[i + 1]; e++) {
-        const int4 cr = hs.below_cran[e];
-        if (cr.x < 0 || cr.x >= P.ns || P.sn_parent[cr.x] != it.x || cr.y < 0 || cr.y >= cr.z ||
-            cr.z > P.sn_nrow[cr.x] - P.sn_ncol[cr.x])
-          bad("solve child ranges");
-        const int32_t* rel = P.relmap.data() + P.relmap_off[cr.x];
-        if (rel[cr.y] < P.sn_ncol[it.x] + it.y || rel[cr.z - 1] >= P.sn_ncol[it.x] + a1) bad("solve child ranges");
       }
     }
     for (int32_t s : smallv)
@@ -937,10 +995,6 @@ void build_schedule(ncl_kkt_s* h) {
               if (tc[ti * t.Ct + tj] != std::min(tj, ti)) bad("front task coverage");
         }
     }
-    for (const int2& it : hs.invv)
-      if (it.x < 0 || it.x >= P.ns || it.y < 0 || 32 * it.y >= P.sn_ncol[it.x] || !hs.sn_flags[it.x] ||
-          hs.sn_Ioff[it.x] + (int64_t)(it.y + 1) * 1024 > hs.sn_Ioff[it.x + 1])
-        bad("inverse item");
     for (const TcProb& q : hs.tcv) {
       const int64_t csz = q.c_in_u ? Usz : Lsz;
       if (q.map < 0 || q.map >= (int)hs.tc_fronts.size()) bad("tc map");
@@ -1007,13 +1061,65 @@ void build_device(ncl_kkt_s* h) {
   d.sn_rows = h->upload(P.sn_rows);
   d.sn_Loff = h->upload(P.sn_Loff);
   d.sn_Uoff = h->upload(P.sn_Uoff);
-  d.sn_Woff = h->upload(P.sn_Woff);
-  std::vector<int64_t> Poff(P.ns + 1, 0);
-  for (int32_t s = 0; s < P.ns; s++) {
-    int64_t nb = P.sn_nrow[s] - P.sn_ncol[s];
-    Poff[s + 1] = Poff[s] + ((nb + SOLVE_ROWS - 1) / SOLVE_ROWS) * P.sn_ncol[s];
+  {
+    std::vector<SnMeta> meta((size_t)std::max<int32_t>(P.ns, 1));
+    for (int32_t q = 0; q < P.ns; q++) {
+      SnMeta& m = meta[q];
+      m = SnMeta{};
+      m.L = P.sn_Loff[q];
+      m.rows = P.sn_rows_off[q];
+      m.W = (uint32_t)P.sn_Woff[q];
+      m.col0 = P.sn_col0[q];
+      m.ncol = P.sn_ncol[q];
+      m.ncp = P.sn_ncolp[q];
+      m.nrow = P.sn_nrow[q];
+    }
+    d.sn_meta = h->upload(meta);
+    // by front row, the entries of the children's update vectors that land on
+    // it (children in order): the first two in the row's record; where there
+    // are more, the second and later ones in a list (count, entries)
+    const int64_t totrows = P.sn_rows_off[P.ns], wtot = P.sn_Woff[P.ns];
+    if (wtot >= (int64_t)0x7fffffff) throw std::bad_alloc();   // (the vectors alone would take over 64 GB)
+    constexpr uint32_t none = 0x7fffffffu;
+    std::vector<uint2> wm((size_t)std::max<int64_t>(totrows, 1), make_uint2(none, none));
+    std::vector<uint32_t> list;
+    std::vector<std::pair<uint32_t, uint32_t>> more;   // (row within its front, entry), by child
+    for (int32_t q = 0; q < P.ns; q++) {
+      uint2* w = wm.data() + P.sn_rows_off[q];
+      more.clear();
+      for (int32_t k = P.child_ptr[q]; k < P.child_ptr[q + 1]; k++) {
+        const int32_t c = P.child_list[k];
+        const int32_t* rel = P.relmap.data() + P.relmap_off[c];
+        const int64_t nb = P.relmap_off[c + 1] - P.relmap_off[c];
+        for (int64_t a = 0; a < nb; a++) {
+          const uint32_t e = (uint32_t)(P.sn_Woff[c] + a);
+          uint2& x = w[rel[a]];
+          if (x.x == none) x.x = e;
+          else if (x.y == none) x.y = e;
+          else more.emplace_back((uint32_t)rel[a], e);
+        }
+      }
+      std::stable_sort(more.begin(), more.end(), [](auto& a, auto& b) { return a.first < b.first; });
+      for (size_t i = 0; i < more.size();) {
+        size_t j = i;
+        while (j < more.size() && more[j].first == more[i].first) j++;
+        uint2& x = w[more[i].first];
+        const uint32_t at = (uint32_t)list.size();
+        list.push_back((uint32_t)(j - i + 1));
+        list.push_back(x.y);
+        for (size_t l = i; l < j; l++) list.push_back(more[l].second);
+        x.y = 0x80000000u | at;
+        i = j;
+      }
+    }
+    if (list.size() >= 0x7fffffffu) throw std::bad_alloc();
+    d.wm = h->upload(wm);
+    d.wm_list = h->upload(list);
   }
-  d.sn_Poff = h->upload(Poff);
+  // (the no-alloc entry point's size rule counts partial sums per 64 rows below)
+  d.Ptot = 0;
+  for (int32_t s = 0; s < P.ns; s++)
+    d.Ptot += (int64_t)((P.sn_nrow[s] - P.sn_ncol[s] + SOLVE_ROWS - 1) / SOLVE_ROWS) * P.sn_ncol[s];
   d.child_ptr = h->upload(P.child_ptr);
   d.child_list = h->upload(P.child_list);
   d.relmap_off = h->upload(P.relmap_off);
@@ -1032,7 +1138,6 @@ void build_device(ncl_kkt_s* h) {
   d.col_inst = h->upload(P.col_inst);
   d.col_sign = h->upload(P.col_sign);
   d.Wtot = P.sn_Woff[P.ns];
-  d.Ptot = Poff[P.ns];
   d.H_row = h->upload(P.H_row);
   d.H_col = h->upload(P.H_col);
   d.J_con = h->upload(P.J_row);
@@ -1096,7 +1201,6 @@ void build_device(ncl_kkt_s* h) {
     N.U = h->alloc<T>(P.U_stored);
     N.D = h->alloc<T>(P.dim);
     N.piv = h->alloc<int8_t>(P.dim);
-    N.Linv = h->alloc<T>(h->hs.sn_Ioff[P.ns]);
     N.Klow = h->Klow;
   };
   if (is_fp32(h)) alloc_num(h->nf, float{});
@@ -1104,7 +1208,6 @@ void build_device(ncl_kkt_s* h) {
   h->xp = h->alloc<char>((int64_t)P.dim * MAX_RHS_SWEEP * esz);
   h->own_xp = h->xp;
   h->W = h->alloc<char>(std::max<int64_t>(d.Wtot, 1) * MAX_RHS_SWEEP * esz);
-  h->Pw = h->alloc<char>(std::max<int64_t>(d.Ptot, 1) * MAX_RHS_SWEEP * esz);
   h->R = h->alloc<double>((int64_t)P.dim * MAX_RHS_SWEEP);
   h->GBtmp = h->alloc<double>((int64_t)P.dim * MAX_RHS_SWEEP);
   h->jx = h->alloc<double>(std::max<int64_t>(d.ncon, 1) * MAX_RHS_SWEEP);
@@ -1135,10 +1238,13 @@ void build_device(ncl_kkt_s* h) {
   }
   h->d_err = h->alloc<int>(4);
   if (!h->hs.dagv.empty()) h->d_dag = h->upload(h->hs.dagv);
-  if (!h->hs.invv.empty()) h->d_invv = h->upload(h->hs.invv);
+  h->d_inv64 = h->upload(h->hs.inv64);
+  h->d_inv128 = h->upload(h->hs.inv128);
+  h->d_merge = h->upload(h->hs.mergev);
   if (!h->hs.regitems.empty()) {
     h->d_regitems = h->upload(h->hs.regitems);
     h->d_regnodes = h->upload(h->hs.regnodes);
+    h->d_regbounds = h->upload(h->hs.regbounds);
   }
   h->d_dag_cnt = h->alloc<int>(h->hs.dag_counters + 1);   // + the subtree factorisation's counter
   {
@@ -1148,7 +1254,6 @@ void build_device(ncl_kkt_s* h) {
     h->n_sm = std::max(1, nsm);
   }
   d.sn_flags = h->upload(h->hs.sn_flags);
-  d.sn_Ioff = h->upload(h->hs.sn_Ioff);
   CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
 
   HostSched& hs = h->hs;
@@ -1160,14 +1265,11 @@ void build_device(ncl_kkt_s* h) {
   h->d_panel_sync = h->alloc<int>(std::max<int64_t>(hs.panel_sync, 8));
   h->d_probs = h->upload(hs.probv);
   h->d_tilep = h->upload(hs.tilep);
+  h->d_narrow = h->upload(hs.narrowv);
+  h->d_block = h->upload(hs.blockv);
+  h->d_strips = h->upload(hs.stripv);
   h->d_chain = h->upload(hs.chainv);
-  h->d_chain_pptr = h->upload(hs.chain_pptr);
-  h->d_chain_pran = h->upload(hs.chain_pran);
-  h->d_chain_sync = h->alloc<int>(2 * (int64_t)P.ns + 2 * hs.nbrows + 2);   // + the two subtree-sweep counters
-  h->d_below = h->upload(hs.belowv);
-  h->d_bbelow = h->upload(hs.bbelowv);
-  h->d_below_cptr = h->upload(hs.below_cptr);
-  h->d_below_cran = h->upload(hs.below_cran);
+  h->d_chain_sync = h->alloc<int>(2 * (int64_t)P.ns + 2 * hs.nbrows);
   CK(cudaMallocHost(&h->h_pinned, sizeof(double) * (size_t)(7 * ni + 64 + 3 * ni * MAX_RHS_SWEEP)));
   CK(cudaEventCreate(&h->ev0));
   CK(cudaEventCreate(&h->ev1));
@@ -1309,10 +1411,20 @@ void run_factor(ncl_kkt_s* h, DevNum<T>& N, cudaStream_t st) {
                          L.tsyrk_stages, h->d_maps, h->d_err, h->opt.wait_cycles, st);
       });
   }
-  const int ninv = (int)h->hs.invv.size();
-  klaunch(h, st, f32 ? "invert_blocks_f32" : "invert_blocks_f64", ninv,
-          Cost{ninv * 32.0 * 32 * 32 / 3.0, ninv * 2.0 * 1024 * sizeof(T)},
-          [&] { launch_invert_blocks<T>(P, N, h->d_invv, ninv, st); });
+  // the pivot blocks' inverses for the sweeps
+  const HostSched& hs = h->hs;
+  const double inv_n = std::max<double>(1.0, (double)(hs.inv64.size() + hs.inv128.size()));
+  klaunch(h, st, f32 ? "invert_blocks_f32" : "invert_blocks_f64", (int64_t)hs.inv64.size(),
+          scaled(hs.inv_cost, hs.inv64.size() / inv_n),
+          [&] { launch_invert_diag<T>(P, N, h->d_inv64, (int)hs.inv64.size(), 64, st); });
+  klaunch(h, st, f32 ? "invert_blocks_f32" : "invert_blocks_f64", (int64_t)hs.inv128.size(),
+          scaled(hs.inv_cost, hs.inv128.size() / inv_n),
+          [&] { launch_invert_diag<T>(P, N, h->d_inv128, (int)hs.inv128.size(), 128, st); });
+  if constexpr (sizeof(T) == 4)
+    for (const HostSched::Merge& M : hs.merges)
+      for (int second = 0; second < 2; second++)
+        klaunch(h, st, "invert_merge_f32", M.cnt, scaled(hs.merge_cost, 0.5 / hs.merges.size()),
+                [&] { launch_invert_merge(P, N, h->d_merge + M.off, M.cnt, M.h, second != 0, st); });
   CK(cudaGetLastError());
 }
 
@@ -1321,54 +1433,75 @@ void run_sweeps(ncl_kkt_s* h, DevNum<T>& N, int nrhs, cudaStream_t st) {
   const DevPlan& P = h->dp;
   T* xp = (T*)h->xp;
   T* W = (T*)h->W;
-  T* Pw = (T*)h->Pw;
-  const bool f32 = sizeof(T) == 4;
-  const int64_t ns = P.ns, nb = h->hs.nbrows;
+  // y and z live in the residual vector, which a sweep's caller has read into
+  // xp (or does not use) and computes anew afterwards
+  T* yv = (T*)h->R;
+  constexpr bool f32 = sizeof(T) == 4;
+  const HostSched& hs = h->hs;
+  const int64_t ns = P.ns, nb = hs.nbrows;
   int* tk_f = h->d_chain_sync;
   int* tk_b = tk_f + ns;
   int* fl_f = tk_b + ns;
   int* fl_b = fl_f + nb;
   int* serr = h->d_err + 1;
-  int* reg_ctr = h->d_chain_sync + 2 * ns + 2 * nb;
-  const HostSched& hs = h->hs;
-  CK(cudaMemsetAsync(h->d_chain_sync, 0, (2 * ns + 2 * nb + 2) * sizeof(int), st));
+  if (!f32 && nb > 0) CK(cudaMemsetAsync(h->d_chain_sync, 0, (2 * ns + 2 * nb) * sizeof(int), st));
   klaunch(h, st, f32 ? "subtree_fwd_f32" : "subtree_fwd_f64", (int64_t)hs.regitems.size(),
           scaled(hs.reg_fwd_cost, nrhs), [&] {
-            launch_region_fwd<T>(P, N, h->d_regitems, (int)hs.regitems.size(), h->d_regnodes, xp, W, nrhs, reg_ctr,
-                                 h->n_sm, st);
+            launch_region_fwd<T>(P, N, h->d_regitems, (int)hs.regitems.size(), h->d_regnodes, h->d_regbounds, xp, yv, W,
+                                 nrhs, st);
           });
+  auto sum = [](Cost a, const Cost& b) {
+    a.flops += b.flops;
+    a.bytes += b.bytes;
+    return a;
+  };
+  // one: the level's narrow and block supernodes take part in the launch
+  auto items = [&](const Level& L, const Level::Strips& S, bool one) {
+    SweepItems I{};
+    if (one) {
+      I.narrow = h->d_narrow + L.narrow_off;
+      I.nnarrow = L.narrow_cnt;
+      I.block = h->d_block + L.block_off;
+      I.nblock = L.block_cnt;
+      I.block_below = L.block_below;
+    }
+    I.strips = h->d_strips + S.off;
+    I.nstrips = S.cnt;
+    I.vec = S.vec;
+    return I;
+  };
+  // (the profile names the pivot blocks' launches of levels with a supernode
+  // wider than one block-row apart)
   for (const Level& L : h->levels) {
-    // levels with a supernode of more than one block-row run the chained
-    // instantiation (named apart in the profile)
-    const char* fname = L.chain_multi ? (f32 ? "fwd_chain_multi_f32" : "fwd_chain_multi_f64")
-                                      : (f32 ? "fwd_chain_f32" : "fwd_chain_f64");
-    klaunch(h, st, fname, L.chain_cnt, scaled(L.fdiag_cost, nrhs), [&] {
-      launch_fwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, (int)L.chain_smem, L.chain_multi,
-                          h->d_chain_pptr, h->d_chain_pran, xp, W, nrhs, tk_f, fl_f, serr, h->opt.wait_cycles, st);
-    });
-    klaunch(h, st, f32 ? "fwd_below_f32" : "fwd_below_f64", L.below_cnt, scaled(L.fbelow_cost, nrhs),
-            [&] {
-              launch_fwd_below<T>(P, N, h->d_below + L.below_off, h->d_below_cptr + L.below_off, h->d_below_cran,
-                                  L.below_cnt, xp, W, nrhs, st);
-            });
+    klaunch(h, st, f32 ? (L.multi ? "fwd_chain_multi_f32" : "fwd_chain_f32") : "fwd_chain_f64",
+            L.narrow_cnt + L.block_cnt + L.prow.cnt, scaled(sum(L.one_cost, L.diag_cost), nrhs),
+            [&] { launch_fwd_level<T>(P, N, items(L, L.prow, true), xp, yv, W, nrhs, f32 || nb == 0, st); });
+    if (!f32)
+      klaunch(h, st, "fwd_chain_multi_f64", L.chain_cnt, scaled(L.diag_cost, nrhs), [&] {
+        launch_fwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, W, nrhs, tk_f, fl_f, serr,
+                            h->opt.wait_cycles, st);
+      });
+    klaunch(h, st, f32 ? "fwd_below_f32" : "fwd_below_f64", L.brow.cnt, scaled(L.below_cost, nrhs),
+            [&] { launch_fwd_level<T>(P, N, items(L, L.brow, false), xp, yv, W, nrhs, f32 || nb == 0, st); });
   }
   for (int l = (int)h->levels.size() - 1; l >= 0; l--) {
     const Level& L = h->levels[l];
-    klaunch(h, st, f32 ? "bwd_below_f32" : "bwd_below_f64", L.bbelow_cnt, scaled(L.bbelow_cost, nrhs),
-            [&] {
-              launch_bwd_below<T>(P, N, h->d_bbelow + L.bbelow_off, L.bbelow_cnt, L.bbelow_narrow, xp, Pw, nrhs, st);
-            });
-    const char* bname = L.chain_multi ? (f32 ? "bwd_chain_multi_f32" : "bwd_chain_multi_f64")
-                                      : (f32 ? "bwd_chain_f32" : "bwd_chain_f64");
-    klaunch(h, st, bname, L.chain_cnt, scaled(L.bdiag_cost, nrhs), [&] {
-      launch_bwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, (int)L.chain_smem, L.chain_multi, xp, Pw,
-                          nrhs, tk_b, fl_b, serr, h->opt.wait_cycles, st);
-    });
+    klaunch(h, st, f32 ? "bwd_below_f32" : "bwd_below_f64", L.narrow_cnt + L.block_cnt + L.bcol.cnt,
+            scaled(sum(L.one_cost, L.below_cost), nrhs),
+            [&] { launch_bwd_level<T>(P, N, items(L, L.bcol, true), false, xp, yv, nrhs, st); });
+    klaunch(h, st, f32 ? (L.multi ? "bwd_chain_multi_f32" : "bwd_chain_f32") : "bwd_chain_f64", L.pcol.cnt,
+            scaled(L.diag_cost, nrhs),
+            [&] { launch_bwd_level<T>(P, N, items(L, L.pcol, false), true, xp, yv, nrhs, st); });
+    if (!f32)
+      klaunch(h, st, "bwd_chain_multi_f64", L.chain_cnt, scaled(L.diag_cost, nrhs), [&] {
+        launch_bwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, nrhs, tk_b, fl_b, serr,
+                            h->opt.wait_cycles, st);
+      });
   }
   klaunch(h, st, f32 ? "subtree_bwd_f32" : "subtree_bwd_f64", (int64_t)hs.regitems.size(),
           scaled(hs.reg_bwd_cost, nrhs), [&] {
-            launch_region_bwd<T>(P, N, h->d_regitems, (int)hs.regitems.size(), h->d_regnodes, xp, nrhs, reg_ctr + 1,
-                                 h->n_sm, st);
+            launch_region_bwd<T>(P, N, h->d_regitems, (int)hs.regitems.size(), h->d_regnodes, h->d_regbounds, xp, yv,
+                                 nrhs, st);
           });
   CK(cudaGetLastError());
 }
@@ -2599,7 +2732,7 @@ extern "C" ncl_status ncl_kkt_solve_noalloc(ncl_kkt_t h, int32_t nrhs, const dou
     // its own workspace back
     struct Swap {
       ncl_kkt_s* h;
-      void *xp, *W, *Pw;
+      void *xp, *W;
       double* R;
       unsigned long long* norms;
       double *gV, *gZ, *gw, *gpart, *gcoef, *ghost;
@@ -2607,7 +2740,6 @@ extern "C" ncl_status ncl_kkt_solve_noalloc(ncl_kkt_t h, int32_t nrhs, const dou
       ~Swap() {
         h->xp = xp;
         h->W = W;
-        h->Pw = Pw;
         h->R = R;
         h->d_norms = norms;
         h->gm_V = gV;
@@ -2618,11 +2750,10 @@ extern "C" ncl_status ncl_kkt_solve_noalloc(ncl_kkt_t h, int32_t nrhs, const dou
         h->gm_host = ghost;
         h->opt.use_fgmres = use_fgmres;
       }
-    } keep{h, h->xp, h->W, h->Pw, h->R, h->d_norms, h->gm_V, h->gm_Z, h->gm_w, h->gm_part, h->gm_coef,
+    } keep{h, h->xp, h->W, h->R, h->d_norms, h->gm_V, h->gm_Z, h->gm_w, h->gm_part, h->gm_coef,
            h->gm_host, h->opt.use_fgmres};
     h->xp = p;
     h->W = p + b_xp;
-    h->Pw = p + b_xp + b_w;
     h->R = (double*)(p + b_xp + b_w + b_pw);
     h->d_norms = (unsigned long long*)(p + b_xp + b_w + b_pw + b_r);
     if (gm_fits) {
@@ -2658,22 +2789,9 @@ ncl_status selftest_timeout(ncl_kkt_s* h, DevNum<T>& N, int which, long long wai
     // than one: its ticket counter starts at 1 and only nbr - 1 CTAs run, so
     // block-row 0 is never solved and its flag never published; the CTA of
     // block-row 1 waits for it until the limit
-    int64_t i0 = -1;
-    int nbr = 0, smem = 0;
-    for (const Level& L : h->levels) {
-      for (int64_t i = L.chain_off; i < L.chain_off + L.chain_cnt; i++) {
-        const int s = hs.chainv[i].x;
-        if (P.sn_ncol[s] > CHAIN_ROWS && (i == L.chain_off || hs.chainv[i - 1].x != s)) {
-          i0 = i;
-          nbr = (P.sn_ncol[s] + CHAIN_ROWS - 1) / CHAIN_ROWS;
-          smem = (int)L.chain_smem;
-          break;
-        }
-      }
-      if (i0 >= 0) break;
-    }
-    if (i0 < 0) return fail(NCL_ERR_INVALID_ARG, "no supernode with more than one block-row");
-    const int s = hs.chainv[i0].x;
+    if (hs.chainv.empty()) return fail(NCL_ERR_INVALID_ARG, "no supernode with more than one block-row");
+    const int s = hs.chainv[0].x;
+    const int nbr = (P.sn_ncol[s] + CHAIN_ROWS - 1) / CHAIN_ROWS;
     const int64_t ns = P.ns, nb = hs.nbrows;
     int* tk_f = h->d_chain_sync;
     int* fl_f = tk_f + 2 * ns;
@@ -2681,8 +2799,8 @@ ncl_status selftest_timeout(ncl_kkt_s* h, DevNum<T>& N, int which, long long wai
     CK(cudaMemcpyAsync(tk_f + s, &one, sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(h->d_err + 1, 0, sizeof(int), st));
     g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-    launch_fwd_chain<T>(h->dp, N, h->d_chain + i0, nbr - 1, smem, true, h->d_chain_pptr, h->d_chain_pran,
-                        (T*)h->own_xp, (const T*)h->W, 1, tk_f, fl_f, h->d_err + 1, wait, st);
+    launch_fwd_chain<T>(h->dp, N, h->d_chain, nbr - 1, (const T*)h->own_xp, (T*)h->R, (const T*)h->W, 1, tk_f, fl_f,
+                        h->d_err + 1, wait, st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&herr, h->d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));

@@ -36,13 +36,24 @@ __global__ void __launch_bounds__(256, 1) k_macro_panel(DevPlan P, DevNum<T> N, 
 
 // Small fronts (ncol <= 64): one CTA factors the pivot columns of the whole
 // front in shared memory by 32-column sub-blocks, as the diagonal-block
-// kernel does: one warp factors the sub-block (factor_sub32) and inverts it
-// (for the triangular sweeps), the rows below it are solved by the blocked
+// kernel does: one warp factors the sub-block (factor_sub32; a front's only
+// sub-block is inverted too, for the triangular sweeps), the rows below it are solved by the blocked
 // forward substitution, L21 = F21 L_jj^-T D^-1, and, when a second
 // sub-block follows, the warps update its columns.  The update
 // block F22 -= L21 D1 L21^T is left to the SIMT update kernel, which spreads
 // it over many CTAs.
-int small_front_smem(int nrow, int ncp, int esz) { return (nrow * (ncp + 1) + 32 * LDS + 64) * esz; }
+int small_front_smem(int nrow, int ncp, int esz) { return (nrow * (ncp + 1) + 2 * 32 * LDS + 64) * esz; }
+
+// Write a shared-memory front back.  A pivot block of one sub-block (at most 32
+// columns) is written as its inverse Iv, which the sweeps apply; wider ones
+// are inverted after the factorisation (invert.cu).
+template <typename T>
+__device__ __forceinline__ void store_front(T* Lg, const T* F, const T* Iv, int nrow, int ncol, int ncp, int ldf) {
+  for (int idx = threadIdx.x; idx < nrow * ncp; idx += blockDim.x) {
+    const int r = idx / ncp, c = idx - r * ncp;
+    Lg[idx] = (r < ncol && c < r && ncol <= 32) ? Iv[r * LDS + c] : F[r * ldf + c];
+  }
+}
 
 // 256 threads per CTA (128 was measured slower on the 20 x 25, 300 x 300 and
 // 700 x 700 systems: the rows below the sub-block take twice the passes)
@@ -58,7 +69,8 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_factor_small(DevPlan P, DevNu
   const int ldf = ncp + 1;   // odd: column accesses by lanes are conflict-free
   T* F = reinterpret_cast<T*>(smem_raw);
   T* Ls = F + nrow * ldf;     // the sub-block's unit lower factor, zero padded
-  T* dsh = Ls + 32 * LDS;     // pivots
+  T* Iv = Ls + 32 * LDS;      // its inverse (fronts of one sub-block)
+  T* dsh = Iv + 32 * LDS;     // pivots
   T* Lg = N.L + P.sn_Loff[s];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   load_tile(F, ldf, Lg, ncp, nrow, ncp, [](int, int) { return true; });
@@ -79,7 +91,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_factor_small(DevPlan P, DevNu
 #pragma unroll 4
       for (int u = 0; u < 32; u++) Ls[lane * LDS + u] = (u < lane && lane < cw) ? F[(c0 + lane) * ldf + c0 + u] : T(0);
       __syncwarp();
-      invert_sub32<T>(Ls, LDS, cw, N.Linv + P.sn_Ioff[s] + (int64_t)(c0 >> 5) * 1024, lane);
+      if (ncol <= 32) invert_sub32<T>(Ls, Iv, cw, lane);
     }
     __syncthreads();
     // rows below the sub-block: L21 = F21 L_jj^-T D^-1 (blocked forward
@@ -113,7 +125,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_factor_small(DevPlan P, DevNu
       __syncthreads();
     }
   }
-  for (int idx = tid; idx < nrow * ncp; idx += blockDim.x) Lg[idx] = F[(idx / ncp) * ldf + idx % ncp];
+  store_front<T>(Lg, F, Iv, nrow, ncol, ncp, ldf);
 }
 
 template <typename T>
@@ -154,7 +166,8 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
   const int ldf = ncp + 1;
   T* F = reinterpret_cast<T*>(smem_raw);
   T* Ls = F + nrow * ldf;
-  T* dsh = Ls + 32 * LDS;
+  T* Iv = Ls + 32 * LDS;
+  T* dsh = Iv + 32 * LDS;
   T* Lg = N.L + P.sn_Loff[s];
   T* Ub = N.U + P.sn_Uoff[s];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
@@ -205,7 +218,7 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
 #pragma unroll 4
     for (int u = 0; u < 32; u++) Ls[lane * LDS + u] = (u < lane && lane < ncol) ? F[lane * ldf + u] : T(0);
     __syncwarp();
-    invert_sub32<T>(Ls, LDS, ncol, N.Linv + P.sn_Ioff[s], lane);
+    invert_sub32<T>(Ls, Iv, ncol, lane);
   }
   __syncthreads();
   // rows below: L21 = F21 L11^-T D1^-1
@@ -219,7 +232,7 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
   // write the factor block back, and form the update block from it:
   // 4 x 4 register tiles of its lower triangle spread over all threads
   // (9 shared loads per 16 products), F22[a][b] -= sum_k (L[a][k] d_k) L[b][k]
-  for (int idx = tid; idx < nrow * ncp; idx += blockDim.x) Lg[idx] = F[(idx / ncp) * ldf + idx % ncp];
+  store_front<T>(Lg, F, Iv, nrow, ncol, ncp, ldf);
   const int T4 = (nb + 3) / 4;
   const int ntl = T4 * (T4 + 1) / 2;
   for (int e = tid; e < ntl; e += blockDim.x) {
@@ -259,7 +272,7 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_subtree_factor(DevPlan P, DevNum<T> N, const int2* __restrict__ items,
+__global__ void __launch_bounds__(256) k_subtree_factor(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
                                                         int count, const int32_t* __restrict__ nodes, int* counter,
                                                         double eps, int policy) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -270,7 +283,7 @@ __global__ void __launch_bounds__(256) k_subtree_factor(DevPlan P, DevNum<T> N, 
     __syncthreads();
     const int it = s_item;
     if (it >= count) break;
-    const int2 item = items[it];
+    const int4 item = items[it];
     for (int q = 0; q < item.y; q++) {
       subtree_front<T>(P, N, nodes[item.x + q], eps, policy, smem_raw);
       __syncthreads();
@@ -279,7 +292,7 @@ __global__ void __launch_bounds__(256) k_subtree_factor(DevPlan P, DevNum<T> N, 
 }
 
 template <typename T>
-void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const int32_t* nodes,
+void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
                            int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st) {
   if (count <= 0) return;
   static bool attr = false;
@@ -295,35 +308,10 @@ void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int2* ite
   k_subtree_factor<T><<<grid, 256, smem, st>>>(P, N, items, count, nodes, counter, eps, policy);
 }
 
-template void launch_subtree_factor<float>(const DevPlan&, const DevNum<float>&, const int2*, int, const int32_t*,
+template void launch_subtree_factor<float>(const DevPlan&, const DevNum<float>&, const int4*, int, const int32_t*,
                                            int*, int, int, double, int, cudaStream_t);
-template void launch_subtree_factor<double>(const DevPlan&, const DevNum<double>&, const int2*, int, const int32_t*,
+template void launch_subtree_factor<double>(const DevPlan&, const DevNum<double>&, const int4*, int, const int32_t*,
                                             int*, int, int, double, int, cudaStream_t);
-
-// ---------------------------------------------------------------------------
-// Inverses of the unit lower 32 x 32 diagonal sub-blocks of the large
-// fronts' pivot blocks (used by the triangular sweeps), one warp per
-// sub-block, after the factorisation: items (supernode, sub-block).
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) k_invert_blocks(DevPlan P, DevNum<T> N, const int2* __restrict__ items,
-                                                       int count) {
-  const int it = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (it >= count) return;
-  const int s = items[it].x, b = items[it].y;
-  const int ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s];
-  const T* blk = N.L + P.sn_Loff[s] + (int64_t)(32 * b) * ncp + 32 * b;
-  invert_sub32<T>(blk, ncp, min(32, ncol - 32 * b), N.Linv + P.sn_Ioff[s] + (int64_t)b * 1024, lane);
-}
-
-template <typename T>
-void launch_invert_blocks(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, cudaStream_t st) {
-  if (count <= 0) return;
-  k_invert_blocks<T><<<(count + 7) / 8, 256, 0, st>>>(P, N, items, count);
-}
-
-template void launch_invert_blocks<float>(const DevPlan&, const DevNum<float>&, const int2*, int, cudaStream_t);
-template void launch_invert_blocks<double>(const DevPlan&, const DevNum<double>&, const int2*, int, cudaStream_t);
 
 template void launch_factor_small<float>(const DevPlan&, const DevNum<float>&, const int32_t*, int, int, double,
                                          int, cudaStream_t);

@@ -155,30 +155,26 @@ __device__ __noinline__ T factor_sub32(T* blk, int ld, int cw, int my_sign, doub
   return my_d;
 }
 
-// Inverse of the unit lower 32 x 32 block blk (row stride ld, cw valid
-// rows; identity on the padding) by one warp, written row-major to out:
-// lane j forms column j by forward substitution in registers,
+// Inverse of the unit lower 32 x 32 block blk (shared, stride LDS, zero padded;
+// identity past cw) by one warp, to out (shared, stride LDS): lane j forms
+// column j by forward substitution in registers,
 // x_i = -sum_{k<i} L[i][k] x_k, x_j = 1, x_i = 0 for i < j.
 template <typename T>
-__device__ __noinline__ void invert_sub32(const T* blk, int ld, int cw, T* out, int lane) {
+__device__ __noinline__ void invert_sub32(const T* blk, T* out, int cw, int lane) {
   T x[32];
 #pragma unroll
   for (int i = 0; i < 32; i++) {
-    if (i >= cw) {   // (a root's last sub-block: rows past cw lie past the factor's storage)
-      x[i] = (i == lane) ? T(1) : T(0);
-      continue;
-    }
     T a0 = T(0), a1 = T(0);
 #pragma unroll
     for (int k = 0; k + 1 < i; k += 2) {
-      a0 += blk[i * ld + k] * x[k];
-      a1 += blk[i * ld + k + 1] * x[k + 1];
+      a0 += blk[i * LDS + k] * x[k];
+      a1 += blk[i * LDS + k + 1] * x[k + 1];
     }
-    if (i & 1) a0 += blk[i * ld + i - 1] * x[i - 1];
+    if (i & 1) a0 += blk[i * LDS + i - 1] * x[i - 1];
     x[i] = (i == lane) ? T(1) : ((i > lane && i < cw) ? -(a0 + a1) : T(0));
   }
 #pragma unroll
-  for (int i = 0; i < 32; i++) out[i * 32 + lane] = x[i];
+  for (int i = 0; i < 32; i++) out[i * LDS + lane] = x[i];
 }
 
 // X = R L^-T for the rows [0, nrows) of R (shared, row stride ldr, ncols <=
@@ -316,8 +312,7 @@ __device__ __forceinline__ void block_update(T* A, int LDM, const T* Xs, int c0,
 // next sub-block (factor_sub32) while warps 1..7 publish sub-block j (its
 // columns and pivots to global memory, fence, release flag j, for the row
 // CTAs) and update the columns beyond the next sub-block.  The rows below
-// the first sub-block are loaded while warp 0 factors it.  At the end four
-// warps invert the four unit lower sub-blocks (for the triangular sweeps).
+// the first sub-block are loaded while warp 0 factors it.
 template <typename T, int MNB>
 __device__ __forceinline__ void panel_diag_role(const DevPlan& P, const DevNum<T>& N, int s, int q0, int* flags,
                                                 double eps, int policy, unsigned char* smem_raw) {

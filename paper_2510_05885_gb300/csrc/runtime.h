@@ -13,11 +13,22 @@ constexpr int PANEL_NB = 32;      // pivot columns of a diagonal sub-block
 constexpr int MACRO_NB = 128;     // pivot columns per panel of a large front
 constexpr int MACRO_ROWS = 64;    // rows below the macro panel per CTA
 constexpr int GEMM_TILE = 64;     // SIMT update tile (rows x cols)
-constexpr int SOLVE_ROWS = 64;     // below rows per solve CTA
+constexpr int SOLVE_ROWS = 64;     // rows per partial sum in the no-alloc workspace's size
 constexpr int MAX_RHS_SWEEP = 8;   // right-hand sides per triangular sweep
-constexpr int CHAIN_ROWS = 128;    // pivot rows per CTA of the chained sweeps
+constexpr int CHAIN_ROWS = 128;    // pivot rows per CTA of the chained sweeps (FP64), and of an inverted diagonal block
+constexpr int SWEEP_CHUNK_BYTES = 64 * 1024;   // staged vector of a sweep's strip
+constexpr int SWEEP_BLOCK_BELOW = 1024;        // rows below its pivots, at most
+constexpr int SWEEP_BLOCK_BYTES = 96 * 1024;   // front of a supernode swept by one CTA, at most
 constexpr int SMALL_SMEM = 64 * 1024;      // front bytes (nrow x ncolp) of a small front, at most
 constexpr int SMALL_SMEM_MAX = 96 * 1024;  // dynamic smem limit of the small-front kernel
+
+// What the sweeps need of a supernode, in one 48-byte record: factor block and
+// row offsets, first entry of W, first pivot, sizes.
+struct __align__(16) SnMeta {
+  int64_t L, rows;
+  uint32_t W;
+  int32_t col0, ncol, ncp, nrow, pad[3];
+};
 
 // Pointers into device copies of the symbolic plan.
 struct DevPlan {
@@ -47,8 +58,10 @@ struct DevPlan {
   const int32_t* sn_rows;
   const int64_t* sn_Loff;
   const int64_t* sn_Uoff;
-  const int64_t* sn_Woff;
-  const int64_t* sn_Poff;
+  const SnMeta* sn_meta;
+  const uint2* wm;           // per front row: the first two entries of W that land on it (children's
+                             // updates, by child); more are in wm_list (sweep.cu, Pulls)
+  const uint32_t* wm_list;
   const int32_t* child_ptr;
   const int32_t* child_list;
   const int64_t* relmap_off;
@@ -75,7 +88,6 @@ struct DevPlan {
   const int64_t* inst_row_off;  // ninst+1
   const int64_t* sn_Soff;       // split-operand offset of a tensor-core front, -1 otherwise
   const int8_t* sn_flags;       // bit 0: front factored by panels (large front)
-  const int64_t* sn_Ioff;       // offset of the inverted 32 x 32 diagonal blocks of L11
   // the J values of each variable (by its KKT row), in constraint order
   const int64_t* JT_ptr;        // dim+1
   const int32_t* JT_idx;        // J value indices
@@ -93,13 +105,12 @@ struct NewtonDev {
 // Numeric state for one precision T (float or double).
 template <typename T>
 struct DevNum {
-  T* L;            // supernodal factor blocks (row-major, ld = ncolp)
+  T* L;            // supernodal factor blocks (row-major, ld = ncolp); L11 holds its inverse after the factorisation
   T* U;            // multifrontal update blocks (row-major lower, ld = nbelow)
   T* D;            // pivots, permuted order
   int8_t* piv;     // pivot status: 0 ok, 1 perturbed, 2 zero (stop policy), 3 non-finite
   const double* Klow;  // FP64 lower KKT values (natural numbering)
   float* S;        // split TF32 operands (L_hi, L_lo, W_hi, W_lo planes) of tensor-core fronts
-  T* Linv;         // inverses of the unit lower 32 x 32 diagonal blocks of every L11 (row-major)
 };
 
 // A dense update C -= A diag(d) B^T restricted to the lower part, over a
@@ -182,9 +193,7 @@ void launch_gemm_simt(const DevPlan& P, const DevNum<T>& N, const GemmProb* prob
 // launchers (panel.cu)
 int small_front_smem(int nrow, int ncp, int esz);
 template <typename T>
-void launch_invert_blocks(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, cudaStream_t st);
-template <typename T>
-void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const int32_t* nodes,
+void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
                            int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st);
 template <typename T>
 void launch_macro_panel(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int* sync, int* err,
@@ -193,33 +202,50 @@ template <typename T>
 void launch_inertia(const DevPlan& P, const DevNum<T>& N, long long* counts, cudaStream_t st);
 
 
-// launchers (solve.cu)
+// launchers (invert.cu)
+template <typename T>
+void launch_invert_diag(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, int width,
+                        cudaStream_t st);
+void launch_invert_merge(const DevPlan& P, const DevNum<float>& N, const int4* items, int count, int h, bool second,
+                         cudaStream_t st);
+
+// The supernodes of one level launch of a sweep, by role (sweep.cu).
+struct SweepItems {
+  const int32_t* narrow;
+  const int32_t* block;
+  const int4* strips;     // (supernode, first row, end row) forward; (supernode, first column) backward
+  int nnarrow, nblock, nstrips;
+  int block_below;        // most rows below a block supernode
+  int vec;                // most entries of a strip's staged vector
+};
+
+// launchers (sweep.cu)
 template <typename T>
 void launch_perm_in(const DevPlan& P, T* xp, const double* B, int64_t ldb, int nrhs, cudaStream_t st);
 template <typename T>
 void launch_perm_out(const DevPlan& P, const T* xp, double* X, int64_t ldx, int nrhs, int accumulate,
                      cudaStream_t st);
-int chain_smem(int rows, int esz);
 template <typename T>
-void launch_fwd_chain(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int smem, bool multi,
-                      const int32_t* pptr, const int4* pran, T* xp, const T* W, int nrhs, int* tickets, int* flags,
-                      int* err, long long wait, cudaStream_t st);
+void launch_fwd_level(const DevPlan& P, const DevNum<T>& N, const SweepItems& I, const T* xp, T* yv, T* W, int nrhs,
+                      bool overlap, cudaStream_t st);
+// piv: the strips are columns of L11^-1 (else of L21)
 template <typename T>
-void launch_fwd_below(const DevPlan& P, const DevNum<T>& N, const int2* items, const int32_t* cptr, const int4* cran,
-                      int count, T* xp, T* W, int nrhs, cudaStream_t st);
+void launch_bwd_level(const DevPlan& P, const DevNum<T>& N, const SweepItems& I, bool piv, T* xp, T* yv, int nrhs,
+                      cudaStream_t st);
 template <typename T>
-void launch_bwd_below(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int narrow, const T* xp,
-                      T* Pw, int nrhs, cudaStream_t st);
+void launch_region_fwd(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
+                       const int32_t* bounds, const T* xp, T* yv, T* W, int nrhs, cudaStream_t st);
 template <typename T>
-void launch_bwd_chain(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int smem, bool multi, T* xp,
-                      const T* Pw, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st);
-int region_smem(int esz);
+void launch_region_bwd(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
+                       const int32_t* bounds, T* xp, const T* yv, int nrhs, cudaStream_t st);
 template <typename T>
-void launch_region_fwd(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const int32_t* nodes, T* xp,
-                       T* W, int nrhs, int* counter, int nsm, cudaStream_t st);
+void launch_fwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const T* xp, T* yv,
+                      const T* W, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st);
 template <typename T>
-void launch_region_bwd(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const int32_t* nodes, T* xp,
-                       int nrhs, int* counter, int nsm, cudaStream_t st);
+void launch_bwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, T* xp, const T* yv, int nrhs,
+                      int* tickets, int* flags, int* err, long long wait, cudaStream_t st);
+
+// launchers (solve.cu)
 void launch_residual(const DevPlan& P, const double* Kf, const double* B, int64_t ldb, const double* X,
                      int64_t ldx, double* R, int64_t ldr, int nrhs, unsigned long long* rnorm,
                      unsigned long long* xnorm, cudaStream_t st);

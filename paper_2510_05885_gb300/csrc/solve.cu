@@ -1,13 +1,6 @@
-// Triangular solves, FP64 residual and adjoint kernels (sm_103a).
-//
-// Solve with the supernodal factors of P K P^T = L D L^T:
-//   forward  L y = P b   leaves to root, level by level,
-//   diagonal z = D^-1 y,
-//   backward L^T w = z   root to leaves,   x = P^T w.
-// Forward updates flow to ancestors through per-supernode update vectors
-// W_s = (rows below s) - L21 y_s, pulled by the parent in a fixed order
-// (no atomics, bitwise reproducible).  The FP64 residual r = b - K x is
-// computed on the FP64 KKT values for iterative refinement (Section 4.3).
+// FP64 residual, refinement vectors, adjoint, slack-form and Newton-step
+// kernels (sm_103a).  The residual r = b - K x is computed on the FP64 KKT
+// values for iterative refinement (Section 4.3).
 #include "runtime.h"
 #include "reduce.cuh"
 
@@ -15,889 +8,11 @@
 
 namespace ncl {
 
-// ---------------------------------------------------------------------------
-// permutations
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void k_perm_in(DevPlan P, T* __restrict__ xp, const double* __restrict__ B, int64_t ldb, int nrhs) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P.dim; k += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t src = P.perm[k];
-    for (int r = 0; r < nrhs; r++) xp[r * P.dim + k] = (T)B[r * ldb + src];
-  }
-}
-
-template <typename T>
-__global__ void k_perm_out(DevPlan P, const T* __restrict__ xp, double* __restrict__ X, int64_t ldx, int nrhs,
-                           int accumulate) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P.dim; k += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t dst = P.perm[k];
-    for (int r = 0; r < nrhs; r++) {
-      const double v = (double)xp[r * P.dim + k];
-      if (accumulate) X[r * ldx + dst] += v;
-      else X[r * ldx + dst] = v;
-    }
-  }
-}
-
 static unsigned grid_for(int64_t n, int per = 256) {
   int64_t b = (n + per - 1) / per;
   if (b > 152 * 16) b = 152 * 16;
   if (b < 1) b = 1;
   return (unsigned)b;
-}
-
-template <typename T>
-void launch_perm_in(const DevPlan& P, T* xp, const double* B, int64_t ldb, int nrhs, cudaStream_t st) {
-  if (P.dim) k_perm_in<T><<<grid_for(P.dim), 256, 0, st>>>(P, xp, B, ldb, nrhs);
-}
-template <typename T>
-void launch_perm_out(const DevPlan& P, const T* xp, double* X, int64_t ldx, int nrhs, int acc, cudaStream_t st) {
-  if (P.dim) k_perm_out<T><<<grid_for(P.dim), 256, 0, st>>>(P, xp, X, ldx, nrhs, acc);
-}
-
-// ---------------------------------------------------------------------------
-// Pivot blocks of the sweeps, chained over 128-row block-rows.
-//
-// Every supernode's pivot block L11 is cut into block-rows of CHAIN_ROWS =
-// 128 rows, one CTA (4 warps) each; warp w owns the block-row's 32-row
-// sub-block w.  A CTA takes its block-row from the supernode's ticket
-// counter, in order, so every block-row it waits for belongs to a CTA that is
-// already running: the waits cannot deadlock, whatever the order in which
-// CTAs are scheduled.  Waits are bounded: past the limit the CTA sets the
-// sweep's error flag, goes on with what it has and still publishes, so that
-// nobody waits on it; the host then reports the sweep as failed.
-//   forward:  y_B = L_BB^-1 (t_B - sum_{J<B} L_BJ y_J),
-//             t_B = the block-row's right-hand side plus the children's updates;
-//   backward: x_B = L_BB^-T (z_B - sum_{I>B} L_IB^T x_I),
-//             z_B = D^-1 y_B - the partial sums of L21^T x of the rows below.
-// The sums over published block-rows are formed by every warp for its rows
-// (lane = row, the published values by shuffles); the diagonal block-row
-// L_BB is then solved inside the CTA sub-block by sub-block with the
-// inverted 32 x 32 diagonal blocks, its strictly lower part staged in shared
-// memory while the CTA waits (only when it has more than one sub-block).
-// Levels whose supernodes all have a single block-row launch the
-// instantiation without the cross-block-row part (MULTI = false), which
-// needs far fewer registers.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release(int* p, int v) {
-  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// lane 0 waits (bounded by `limit` clock cycles) for the flag; the warp then
-// proceeds together.  err is the sweep's error flag: once set, nobody waits
-// any more.
-__device__ __forceinline__ void chain_wait(const int* flag, int* err, long long limit) {
-  if ((threadIdx.x & 31) == 0 && !ld_acquire(flag) && !ld_acquire(err)) {
-    const long long t0 = clock64();
-    while (!ld_acquire(flag)) {
-      if (clock64() - t0 > limit || ld_acquire(err)) {
-        atomicExch(err, 1);
-        break;
-      }
-      __nanosleep(32);
-    }
-  }
-  __syncwarp();
-}
-
-// after a CTA barrier: thread 0 publishes the CTA's results (the release
-// store orders every write the barrier made visible to thread 0 before the
-// flag, so no separate fence is needed)
-__device__ __forceinline__ void chain_publish(int* flag) {
-  if (threadIdx.x == 0) st_release(flag, 1);
-}
-
-int chain_smem(int rows, int esz) {
-  return (rows * (rows + 1) + 2 * MAX_RHS_SWEEP * (CHAIN_ROWS + 1) + ((rows + 31) / 32) * 32 * 33) * esz;
-}
-
-// strictly lower part of the diagonal block-row tile (rows and columns
-// [R0, R0 + nr)) into shared memory, row stride nr + 1
-template <typename T>
-__device__ __forceinline__ void chain_stage_tile(T* Ls, const T* Lb, int64_t ncp, int R0, int nr) {
-  const int n = nr * nr, ld = nr + 1;
-  for (int base = threadIdx.x; base < n; base += 8 * blockDim.x) {
-    T v[8];
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const int idx = base + k * blockDim.x;
-      const int i = idx / nr, c = idx - i * nr;
-      v[k] = (idx < n && c < i) ? Lb[(int64_t)(R0 + i) * ncp + R0 + c] : T(0);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const int idx = base + k * blockDim.x;
-      const int i = idx / nr, c = idx - i * nr;
-      if (idx < n) Ls[i * ld + c] = v[k];
-    }
-  }
-}
-
-template <typename T, bool MULTI>
-__global__ void __launch_bounds__(128) k_fwd_chain(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
-                                                   const int32_t* __restrict__ pptr, const int4* __restrict__ pran,
-                                                   T* __restrict__ xp, const T* __restrict__ W, int nrhs,
-                                                   int* tickets, int* flags, int* err, long long wait) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int sb;
-  const int4 it = items[blockIdx.x];
-  const int s = it.x, broff = it.y, boff = it.z;
-  if (threadIdx.x == 0) sb = atomicAdd(&tickets[s], 1);
-  __syncthreads();
-  const int B = sb;
-  const int ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
-  const int R0 = CHAIN_ROWS * B, nr = min(CHAIN_ROWS, ncol - R0), nsub = (nr + 31) / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ldt = nr + 1;
-  T* Ls = reinterpret_cast<T*>(smem_raw);              // nr x nr, strictly lower
-  T* tb = Ls + nr * ldt;                               // [MAX_RHS_SWEEP][CHAIN_ROWS + 1]
-  T* ys = tb + MAX_RHS_SWEEP * (CHAIN_ROWS + 1);
-  T* Iv = ys + MAX_RHS_SWEEP * (CHAIN_ROWS + 1);      // the inverted 32 x 32 diagonal blocks, stride 33
-  const T* Lb = N.L + P.sn_Loff[s];
-  if (nsub > 1) chain_stage_tile(Ls, Lb, ncp, R0, nr);
-  const int rw = 32 * warp + lane;                     // this lane's row in the block-row
-  const bool mine = warp < nsub;
-  const bool valid = rw < nr;
-  if (mine) {
-    // the inverted diagonal block of this warp's sub-block (for the end)
-    const T* ip = N.Linv + P.sn_Ioff[s] + (int64_t)(4 * B + warp) * 1024;
-    T* iw = Iv + warp * 32 * 33;
-#pragma unroll 8
-    for (int i = 0; i < 32; i++) iw[i * 33 + lane] = ip[i * 32 + lane];
-    // t: the rows' entries plus the children's updates, child by child
-#pragma unroll
-    for (int r = 0; r < MAX_RHS_SWEEP; r++)
-      tb[r * (CHAIN_ROWS + 1) + rw] = (r < nrhs && valid) ? xp[(int64_t)r * P.dim + col0 + R0 + rw] : T(0);
-    __syncwarp();
-    const int k = 4 * B + warp;
-    for (int e = pptr[boff + k]; e < pptr[boff + k + 1]; e++) {
-      const int4 pr = pran[e];
-      const int c = pr.x;
-      const int32_t* rel = P.relmap + P.relmap_off[c];
-      for (int a = pr.y + lane; a < pr.z; a += 32)
-        for (int r = 0; r < nrhs; r++) tb[r * (CHAIN_ROWS + 1) + rel[a] - R0] += W[r * P.Wtot + P.sn_Woff[c] + a];
-      __syncwarp();
-    }
-  }
-  // sum over the published block-rows J < B (all 128 columns of J exist):
-  // the warp reads its 32 rows 32 columns at a time (one coalesced segment
-  // per row; the next segment is loaded before the current one is used and
-  // before waiting for its block-row), and a butterfly reduce-scatter leaves
-  // row rr's sum in lane rr.  Once J is published, its 128 values are loaded
-  // together.  (Levels whose supernodes all have one block-row compile
-  // without this part.)
-  T acc[MAX_RHS_SWEEP];
-#pragma unroll
-  for (int r = 0; r < MAX_RHS_SWEEP; r++) acc[r] = T(0);
-  if (MULTI && mine && B > 0) {
-    const T* wrow = Lb + (int64_t)(R0 + 32 * warp) * ncp + lane;
-    const int nrw = min(32, nr - 32 * warp);
-    // FP32: two chunks in flight ahead of the one in use, so that after the
-    // wait for a block-row its first two chunks are already in registers
-    // (FP64: one, for registers)
-    constexpr bool PF2 = sizeof(T) == 4;
-    T lv[32], ln[32], ln2[32];
-    const int nchunk = 4 * B;
-#pragma unroll
-    for (int rr = 0; rr < 32; rr++) ln[rr] = rr < nrw ? wrow[(int64_t)rr * ncp] : T(0);
-    if (PF2) {
-#pragma unroll
-      for (int rr = 0; rr < 32; rr++) ln2[rr] = rr < nrw ? wrow[(int64_t)rr * ncp + 32] : T(0);
-    }
-    // the right-hand sides of the four chunks of a block-row, loaded
-    // together once it is published and rotated chunk by chunk (FP64: the
-    // first right-hand side only, for registers)
-    constexpr int YQ = sizeof(T) == 4 ? MAX_RHS_SWEEP : 1;
-    T yq[4][YQ];
-    for (int q = 0; q < nchunk; q++) {
-      const int c0 = 32 * q;
-      if (PF2) {
-#pragma unroll
-        for (int rr = 0; rr < 32; rr++) {
-          lv[rr] = ln[rr];
-          ln[rr] = ln2[rr];
-        }
-        if (q + 2 < nchunk) {
-#pragma unroll
-          for (int rr = 0; rr < 32; rr++) ln2[rr] = rr < nrw ? wrow[(int64_t)rr * ncp + c0 + 64] : T(0);
-        }
-      } else {
-#pragma unroll
-        for (int rr = 0; rr < 32; rr++) lv[rr] = ln[rr];
-        if (q + 1 < nchunk) {
-#pragma unroll
-          for (int rr = 0; rr < 32; rr++) ln[rr] = rr < nrw ? wrow[(int64_t)rr * ncp + c0 + 32] : T(0);
-        }
-      }
-      if ((q & 3) == 0) {
-        chain_wait(flags + broff + (q >> 2), err, wait);
-#pragma unroll
-        for (int c = 0; c < 4; c++)
-#pragma unroll
-          for (int r = 0; r < YQ; r++)
-            yq[c][r] = r < nrhs ? __ldcg(xp + (int64_t)r * P.dim + col0 + c0 + 32 * c + lane) : T(0);
-      }
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-        if (r >= nrhs) break;
-        const T yu = r < YQ ? yq[0][r] : __ldcg(xp + (int64_t)r * P.dim + col0 + c0 + lane);
-        T v[32];
-#pragma unroll
-        for (int rr = 0; rr < 32; rr++) v[rr] = lv[rr] * yu;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-          const bool upper = (lane & o) != 0;
-#pragma unroll
-          for (int k = 0; k < o; k++) {
-            const T send = upper ? v[k] : v[k + o];
-            const T recv = __shfl_xor_sync(0xffffffffu, send, o);
-            v[k] = (upper ? v[k + o] : v[k]) + recv;
-          }
-        }
-        acc[r] += v[0];
-      }
-#pragma unroll
-      for (int c = 0; c < 3; c++)
-#pragma unroll
-        for (int r = 0; r < YQ; r++) yq[c][r] = yq[c + 1][r];
-    }
-  }
-  __syncthreads();
-  // the diagonal block-row, sub-block by sub-block
-  for (int w2 = 0; w2 < nsub; w2++) {
-    if (warp == w2) {
-      const T* iw = Iv + warp * 32 * 33 + lane * 33;   // row lane of the inverted block
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-        if (r >= nrhs) break;
-        const T z = valid ? tb[r * (CHAIN_ROWS + 1) + rw] - acc[r] : T(0);
-        T v = T(0);
-#pragma unroll
-        for (int u = 0; u < 32; u++) v += iw[u] * __shfl_sync(0xffffffffu, z, u);
-        ys[r * (CHAIN_ROWS + 1) + rw] = valid ? v : T(0);
-        if (valid) xp[(int64_t)r * P.dim + col0 + R0 + rw] = v;
-      }
-    }
-    __syncthreads();
-    if (warp > w2 && mine) {
-      const T* lr = Ls + min(rw, nr - 1) * ldt + 32 * w2;
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-        if (r >= nrhs) break;
-        const T* y = ys + r * (CHAIN_ROWS + 1) + 32 * w2;
-        T a = T(0);
-#pragma unroll 8
-        for (int u = 0; u < 32; u++) a += lr[u] * y[u];
-        acc[r] += a;
-      }
-    }
-  }
-  chain_publish(flags + broff + B);
-}
-
-template <typename T, bool MULTI>
-__global__ void __launch_bounds__(128) k_bwd_chain(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
-                                                   T* __restrict__ xp, const T* __restrict__ Pw, int nrhs,
-                                                   int* tickets, int* flags, int* err, long long wait) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int sb;
-  const int4 it = items[blockIdx.x];
-  const int s = it.x, broff = it.y;
-  const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
-  const int nbr = (ncol + CHAIN_ROWS - 1) / CHAIN_ROWS;
-  if (threadIdx.x == 0) sb = nbr - 1 - atomicAdd(&tickets[s], 1);
-  __syncthreads();
-  const int B = sb;
-  const int R0 = CHAIN_ROWS * B, nr = min(CHAIN_ROWS, ncol - R0), nsub = (nr + 31) / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ldt = nr + 1;
-  T* Ls = reinterpret_cast<T*>(smem_raw);
-  T* zb = Ls + nr * ldt;
-  T* xs = zb + MAX_RHS_SWEEP * (CHAIN_ROWS + 1);
-  T* Iv = xs + MAX_RHS_SWEEP * (CHAIN_ROWS + 1);      // the inverted 32 x 32 diagonal blocks, stride 33
-  const T* Lb = N.L + P.sn_Loff[s];
-  if (nsub > 1) chain_stage_tile(Ls, Lb, ncp, R0, nr);
-  const int rw = 32 * warp + lane;                     // this lane's column (unknown) in the block-row
-  const bool mine = warp < nsub;
-  const bool valid = rw < nr;
-  if (mine) {
-    // the inverted diagonal block of this warp's sub-block (for the end)
-    const T* ip = N.Linv + P.sn_Ioff[s] + (int64_t)(4 * B + warp) * 1024;
-    T* iw = Iv + warp * 32 * 33;
-#pragma unroll 8
-    for (int i = 0; i < 32; i++) iw[i * 33 + lane] = ip[i * 32 + lane];
-    // z = D^-1 y - the partial sums of the rows below
-    const int nb = nrow - ncol, nch = (nb + SOLVE_ROWS - 1) / SOLVE_ROWS;
-    const T dk = valid ? N.D[col0 + R0 + rw] : T(1);
-    for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-      T z = T(0);
-      if (r < nrhs && valid) {
-        z = xp[(int64_t)r * P.dim + col0 + R0 + rw] / dk;
-        for (int ch = 0; ch < nch; ch++) z -= Pw[r * P.Ptot + P.sn_Poff[s] + (int64_t)ch * ncol + R0 + rw];
-      }
-      zb[r * (CHAIN_ROWS + 1) + rw] = z;
-    }
-  }
-  // sum over the published block-rows I > B: L_IB^T x_I (lane = column);
-  // once I is published, its values are loaded together.  (Levels whose
-  // supernodes all have one block-row compile without this part.)
-  T acc[MAX_RHS_SWEEP];
-#pragma unroll
-  for (int r = 0; r < MAX_RHS_SWEEP; r++) acc[r] = T(0);
-  if (MULTI && mine && B < nbr - 1) {
-    // chunks q = 0, 1, ...: 32 rows of block-row I = nbr - 1 - q / 4, the
-    // next chunk loaded before the current one is used and before waiting
-    const T* lcol = Lb + R0 + min(rw, nr - 1);
-    const int nchunk = 4 * (nbr - 1 - B);
-    auto rows_of = [&](int q, int& q0, int& bwi) {
-      const int I = nbr - 1 - (q >> 2);
-      q0 = CHAIN_ROWS * I + 32 * (q & 3);
-      bwi = max(0, min(32, ncol - q0));
-    };
-    // FP32: two chunks in flight ahead of the one in use (FP64: one, for registers)
-    constexpr bool PF2 = sizeof(T) == 4;
-    T lv[32], ln[32], ln2[32];
-    int nq0, nbw, nq2 = 0, nbw2 = 0;
-    rows_of(0, nq0, nbw);
-#pragma unroll
-    for (int v = 0; v < 32; v++) ln[v] = v < nbw ? lcol[(int64_t)(nq0 + v) * ncp] : T(0);
-    if (PF2 && nchunk > 1) {
-      rows_of(1, nq2, nbw2);
-#pragma unroll
-      for (int v = 0; v < 32; v++) ln2[v] = v < nbw2 ? lcol[(int64_t)(nq2 + v) * ncp] : T(0);
-    }
-    // the values of the four chunks of a block-row, loaded together once it
-    // is published and rotated chunk by chunk (FP64: the first right-hand
-    // side only, for registers)
-    constexpr int XQ = sizeof(T) == 4 ? MAX_RHS_SWEEP : 1;
-    T xq[4][XQ];
-    for (int q = 0; q < nchunk; q++) {
-      const int q0 = nq0, bwi = nbw;
-      if (PF2) {
-#pragma unroll
-        for (int v = 0; v < 32; v++) {
-          lv[v] = ln[v];
-          ln[v] = ln2[v];
-        }
-        nq0 = nq2;
-        nbw = nbw2;
-        if (q + 2 < nchunk) {
-          rows_of(q + 2, nq2, nbw2);
-#pragma unroll
-          for (int v = 0; v < 32; v++) ln2[v] = v < nbw2 ? lcol[(int64_t)(nq2 + v) * ncp] : T(0);
-        }
-      } else {
-#pragma unroll
-        for (int v = 0; v < 32; v++) lv[v] = ln[v];
-        if (q + 1 < nchunk) {
-          rows_of(q + 1, nq0, nbw);
-#pragma unroll
-          for (int v = 0; v < 32; v++) ln[v] = v < nbw ? lcol[(int64_t)(nq0 + v) * ncp] : T(0);
-        }
-      }
-      if ((q & 3) == 0) {
-        chain_wait(flags + broff + nbr - 1 - (q >> 2), err, wait);
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-          const int bw = max(0, min(32, ncol - (q0 + 32 * c)));
-#pragma unroll
-          for (int r = 0; r < XQ; r++)
-            xq[c][r] = (r < nrhs && lane < bw) ? __ldcg(xp + (int64_t)r * P.dim + col0 + q0 + 32 * c + lane) : T(0);
-        }
-      }
-      if (bwi > 0) {
-#pragma unroll
-        for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-          if (r >= nrhs) break;
-          const T xv = r < XQ ? xq[0][r]
-                              : (lane < bwi ? __ldcg(xp + (int64_t)r * P.dim + col0 + q0 + lane) : T(0));
-#pragma unroll
-          for (int v = 0; v < 32; v++) acc[r] += lv[v] * __shfl_sync(0xffffffffu, xv, v);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 3; c++)
-#pragma unroll
-        for (int r = 0; r < XQ; r++) xq[c][r] = xq[c + 1][r];
-    }
-  }
-  __syncthreads();
-  // the diagonal block-row, sub-block by sub-block from the last
-  for (int w2 = nsub - 1; w2 >= 0; w2--) {
-    if (warp == w2) {
-      const T* iw = Iv + warp * 32 * 33 + lane;        // column lane of the inverted block
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-        if (r >= nrhs) break;
-        const T w = valid ? zb[r * (CHAIN_ROWS + 1) + rw] - acc[r] : T(0);
-        T v = T(0);
-#pragma unroll
-        for (int q = 0; q < 32; q++) v += iw[q * 33] * __shfl_sync(0xffffffffu, w, q);
-        xs[r * (CHAIN_ROWS + 1) + rw] = valid ? v : T(0);
-        if (valid) xp[(int64_t)r * P.dim + col0 + R0 + rw] = v;
-      }
-    }
-    __syncthreads();
-    if (warp < w2) {
-      // acc[col rw] += sum_v L[32 w2 + v][rw] x[32 w2 + v]
-      const int nv = min(32, nr - 32 * w2);
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-        if (r >= nrhs) break;
-        const T* x = xs + r * (CHAIN_ROWS + 1) + 32 * w2;
-        T a = T(0);
-        for (int v = 0; v < nv; v++) a += Ls[(32 * w2 + v) * ldt + rw] * x[v];
-        acc[r] += a;
-      }
-    }
-  }
-  chain_publish(flags + broff + B);
-}
-
-// 16-byte vectors of factor entries (rows of L start 16-byte aligned: the
-// blocks start at multiples of 32 elements and the row stride is a multiple
-// of 4 elements)
-template <typename T> struct Vec16;
-template <> struct Vec16<float> {
-  using type = float4;
-  static constexpr int n = 4;
-};
-template <> struct Vec16<double> {
-  using type = double2;
-  static constexpr int n = 2;
-};
-
-// forward: rows below supernode s, SOLVE_ROWS per CTA:
-//   W_s[a] = (children's updates landing on row a) - L21[a,:] y_s
-// The products use tpr = 4..32 threads per row (by the supernode's width),
-// each reading 16-byte vectors of its row, and RPT rows per thread at a time,
-// so that a narrow supernode still has many loads in flight; the partial
-// sums are reduced by shuffles inside each group of tpr lanes.
-template <typename T>
-__global__ void __launch_bounds__(256) k_fwd_below(DevPlan P, DevNum<T> N, const int2* __restrict__ items,
-                                                   const int32_t* __restrict__ cptr, const int4* __restrict__ cran,
-                                                   const T* __restrict__ xp, T* __restrict__ W, int nrhs) {
-  using V = typename Vec16<T>::type;
-  constexpr int VW = Vec16<T>::n;
-  constexpr int RPT = 4;
-  __shared__ T t[SOLVE_ROWS * 8];
-  const int2 it = items[blockIdx.x];
-  const int s = it.x, a0 = it.y;
-  const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
-  const int nb = nrow - ncol;
-  const int a1 = min(a0 + SOLVE_ROWS, nb);
-  const T* Lb = N.L + P.sn_Loff[s];
-  for (int idx = threadIdx.x; idx < SOLVE_ROWS * nrhs; idx += blockDim.x) t[idx] = T(0);
-  __syncthreads();
-  // children's updates landing on these rows (ranges found on the host),
-  // child by child
-  for (int e = cptr[blockIdx.x]; e < cptr[blockIdx.x + 1]; e++) {
-    const int4 cr = cran[e];
-    const int c = cr.x;
-    const int32_t* rel = P.relmap + P.relmap_off[c];
-    for (int a = cr.y + threadIdx.x; a < cr.z; a += blockDim.x)
-      for (int r = 0; r < nrhs; r++) t[r * SOLVE_ROWS + rel[a] - ncol - a0] += W[r * P.Wtot + P.sn_Woff[c] + a];
-    __syncthreads();
-  }
-  const int nv = (ncol + VW - 1) / VW;                 // vectors per row
-  int tpr = 4;
-  while (tpr < 32 && 2 * tpr < nv) tpr *= 2;
-  const int q = threadIdx.x & (tpr - 1);
-  const int slots = blockDim.x / tpr, slot = threadIdx.x / tpr;
-  const int64_t ysz = (int64_t)P.dim;
-  // every thread runs the same number of passes (the shuffles below are
-  // warp-wide)
-  for (int base = a0; base < a1; base += RPT * slots) {
-    int ar[RPT];
-    bool ok[RPT];
-#pragma unroll
-    for (int j = 0; j < RPT; j++) {
-      ar[j] = base + j * slots + slot;
-      ok[j] = ar[j] < a1;
-    }
-    T acc[RPT][MAX_RHS_SWEEP];
-#pragma unroll
-    for (int j = 0; j < RPT; j++)
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) acc[j][r] = T(0);
-    for (int v = q; v < nv; v += tpr) {
-      V lv[RPT];
-#pragma unroll
-      for (int j = 0; j < RPT; j++) {
-        if (ok[j]) lv[j] = __ldg(reinterpret_cast<const V*>(Lb + (int64_t)(ncol + ar[j]) * ncp) + v);
-        else lv[j] = V{};
-      }
-#pragma unroll
-      for (int e = 0; e < VW; e++) {
-        const int k = v * VW + e;
-        if (k >= ncol) break;
-#pragma unroll
-        for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-          if (r >= nrhs) break;
-          const T y = __ldg(xp + r * ysz + col0 + k);
-#pragma unroll
-          for (int j = 0; j < RPT; j++) acc[j][r] += reinterpret_cast<const T*>(&lv[j])[e] * y;
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < RPT; j++) {
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) {
-        if (r >= nrhs) break;
-        T a = acc[j][r];
-        for (int o = tpr >> 1; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (q == 0 && ok[j]) W[r * P.Wtot + P.sn_Woff[s] + ar[j]] = t[r * SOLVE_ROWS + ar[j] - a0] - a;
-      }
-    }
-  }
-}
-
-// backward: partial sums of L21^T x_below over a run of SOLVE_ROWS rows and
-// a run of up to 256 columns (item (s, a0, k0)).  The level's first `narrow`
-// items (supernodes of at most 32 columns) take one warp each, eight to a
-// CTA (lane = column, the rows in order); the others one CTA each, where
-// for 33..128 columns G = 256 / (columns rounded up to 32) groups of threads
-// split the rows and their sums are added in shared memory.
-template <typename T>
-__global__ void __launch_bounds__(256) k_bwd_below(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
-                                                   int narrow, const T* __restrict__ xp, T* __restrict__ Pw,
-                                                   int nrhs) {
-  __shared__ T xb[SOLVE_ROWS * MAX_RHS_SWEEP];
-  __shared__ T red[256];
-  const int nnc = (narrow + 7) / 8;   // CTAs of the narrow items
-  if ((int)blockIdx.x < nnc) {
-    __shared__ T xw[8][SOLVE_ROWS * MAX_RHS_SWEEP];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + w;
-    if (i >= narrow) return;   // the whole warp; no CTA barrier in this branch
-    const int4 it = items[i];
-    const int s = it.x, a0 = it.y;
-    const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s];
-    const int nb = nrow - ncol;
-    const int a1 = min(a0 + SOLVE_ROWS, nb), na = a1 - a0;
-    const int chunk = a0 / SOLVE_ROWS;
-    const int32_t* rows = P.sn_rows + P.sn_rows_off[s] + ncol;
-    T* x = xw[w];
-    for (int idx = lane; idx < na * nrhs; idx += 32) {
-      const int r = idx / na, a = idx - r * na;
-      x[r * SOLVE_ROWS + a] = xp[r * P.dim + rows[a0 + a]];
-    }
-    __syncwarp();
-    const T* col = N.L + P.sn_Loff[s] + (int64_t)ncol * ncp + min(lane, ncol - 1);
-    for (int r = 0; r < nrhs; r++) {
-      const T* xr = x + r * SOLVE_ROWS - a0;
-      T acc = T(0);
-      if (lane < ncol) {
-#pragma unroll 16
-        for (int a = a0; a < a1; a++) acc += col[(int64_t)a * ncp] * xr[a];
-        Pw[r * P.Ptot + P.sn_Poff[s] + (int64_t)chunk * ncol + lane] = acc;
-      }
-    }
-    return;
-  }
-  const int4 it = items[narrow + (blockIdx.x - nnc)];
-  const int s = it.x, a0 = it.y, k0 = it.z;
-  const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s];
-  const int nb = nrow - ncol;
-  const int a1 = min(a0 + SOLVE_ROWS, nb);
-  const int chunk = a0 / SOLVE_ROWS;
-  const int kc = min(256, ncol - k0);
-  const T* Lb = N.L + P.sn_Loff[s];
-  const int32_t* rows = P.sn_rows + P.sn_rows_off[s] + ncol;
-  for (int idx = threadIdx.x; idx < (a1 - a0) * nrhs; idx += blockDim.x) {
-    const int r = idx / (a1 - a0), a = idx % (a1 - a0);
-    xb[r * SOLVE_ROWS + a] = xp[r * P.dim + rows[a0 + a]];
-  }
-  __syncthreads();
-  // G thread groups of blockDim / G >= kc threads each
-  const int cols = (kc + 31) & ~31;
-  const int G = (cols > 128 || cols <= 32) ? 1 : blockDim.x / cols;
-  const int tpg = blockDim.x / G, g = threadIdx.x / tpg, kl = threadIdx.x - g * tpg;
-  const int per = (a1 - a0 + G - 1) / G;
-  const int ga0 = a0 + g * per, ga1 = min(a1, ga0 + per);
-  const T* col = Lb + (int64_t)ncol * ncp + k0 + min(kl, kc - 1);
-  for (int r = 0; r < nrhs; r++) {
-    const T* x = xb + r * SOLVE_ROWS - a0;
-    T acc = T(0);
-    if (kl < kc) {
-#pragma unroll 16
-      for (int a = ga0; a < ga1; a++) acc += col[(int64_t)a * ncp] * x[a];
-    }
-    T* out = Pw + r * P.Ptot + P.sn_Poff[s] + (int64_t)chunk * ncol + k0;
-    if (G == 1) {
-      if (kl < kc) out[kl] = acc;
-    } else {
-      red[g * tpg + kl] = acc;
-      __syncthreads();
-      if (threadIdx.x < kc) {
-        T t = T(0);
-        for (int q = 0; q < G; q++) t += red[q * tpg + threadIdx.x];
-        out[threadIdx.x] = t;
-      }
-      __syncthreads();
-    }
-  }
-}
-
-template <typename T>
-void launch_fwd_chain(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int smem, bool multi,
-                      const int32_t* pptr, const int4* pran, T* xp, const T* W, int nrhs, int* tickets, int* flags,
-                      int* err, long long wait, cudaStream_t st) {
-  if (count <= 0) return;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_fwd_chain<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         chain_smem(CHAIN_ROWS, sizeof(T)));
-    cudaFuncSetAttribute(k_fwd_chain<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         chain_smem(CHAIN_ROWS, sizeof(T)));
-    attr = true;
-  }
-  if (multi)
-    k_fwd_chain<T, true><<<count, 128, smem, st>>>(P, N, items, pptr, pran, xp, W, nrhs, tickets, flags, err, wait);
-  else
-    k_fwd_chain<T, false><<<count, 128, smem, st>>>(P, N, items, pptr, pran, xp, W, nrhs, tickets, flags, err, wait);
-}
-template <typename T>
-void launch_fwd_below(const DevPlan& P, const DevNum<T>& N, const int2* items, const int32_t* cptr, const int4* cran,
-                      int count, T* xp, T* W, int nrhs, cudaStream_t st) {
-  if (count > 0) k_fwd_below<T><<<count, 256, 0, st>>>(P, N, items, cptr, cran, xp, W, nrhs);
-}
-template <typename T>
-void launch_bwd_below(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int narrow, const T* xp,
-                      T* Pw, int nrhs, cudaStream_t st) {
-  if (count <= 0) return;
-  const int grid = (narrow + 7) / 8 + (count - narrow);
-  k_bwd_below<T><<<grid, 256, 0, st>>>(P, N, items, narrow, xp, Pw, nrhs);
-}
-template <typename T>
-void launch_bwd_chain(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int smem, bool multi, T* xp,
-                      const T* Pw, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st) {
-  if (count <= 0) return;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_bwd_chain<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         chain_smem(CHAIN_ROWS, sizeof(T)));
-    cudaFuncSetAttribute(k_bwd_chain<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         chain_smem(CHAIN_ROWS, sizeof(T)));
-    attr = true;
-  }
-  if (multi)
-    k_bwd_chain<T, true><<<count, 128, smem, st>>>(P, N, items, xp, Pw, nrhs, tickets, flags, err, wait);
-  else
-    k_bwd_chain<T, false><<<count, 128, smem, st>>>(P, N, items, xp, Pw, nrhs, tickets, flags, err, wait);
-}
-
-// ---------------------------------------------------------------------------
-// Sweeps over the subtrees of small supernodes.
-//
-// Near the leaves the assembly tree holds very many supernodes of a few
-// columns (at the 700 x 700 grid 170k of 184k supernodes have at most 32
-// pivots); per-level launches with one CTA per supernode or per 64 rows keep
-// most lanes idle there.  A supernode with at most 32 pivots all of whose
-// descendants have at most 32 as well belongs to a region of small
-// subtrees; each maximal subtree of it is swept by ONE warp, supernode by
-// supernode in postorder (forward) or in reverse (backward), so no flags or
-// launches separate a supernode from its children.  The region's forward
-// sweep runs before the level launches of the rest of the tree, its
-// backward sweep after them.  Lane c holds column c of the supernode; the
-// 32 x 32 inverse of its unit lower pivot block is staged in the warp's
-// shared memory (row stride 33).
-//   forward:  t = own entries + children's updates (in child order),
-//             y = L11^-1 t, W_s = children's updates below - L21 y;
-//   backward: z = D^-1 y - L21^T x_below, x = L11^-T z.
-// ---------------------------------------------------------------------------
-constexpr int REG_WARPS = 8;
-
-template <typename T>
-__device__ __forceinline__ void region_stage_inverse(const DevPlan& P, const DevNum<T>& N, int s, T* iv, int lane) {
-  const T* ip = N.Linv + P.sn_Ioff[s];
-#pragma unroll 8
-  for (int i = 0; i < 32; i++) iv[i * 33 + lane] = ip[i * 32 + lane];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_region_fwd(DevPlan P, DevNum<T> N, const int2* __restrict__ items, int count,
-                                                    const int32_t* __restrict__ nodes, T* __restrict__ xp,
-                                                    T* __restrict__ W, int nrhs, int* counter) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* iv = reinterpret_cast<T*>(smem_raw) + warp * (32 * 33 + MAX_RHS_SWEEP * 33);
-  T* tb = iv + 32 * 33;                              // [MAX_RHS_SWEEP][33]
-  const int64_t dim = P.dim, Wtot = P.Wtot;
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(counter, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= count) break;
-    const int2 item = items[it];
-    for (int q = 0; q < item.y; q++) {
-      const int s = nodes[item.x + q];
-      const int ncol = P.sn_ncol[s], nb = P.sn_nrow[s] - ncol, ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
-      T* Ws = W + P.sn_Woff[s];
-      region_stage_inverse(P, N, s, iv, lane);
-      for (int r = 0; r < nrhs; r++) tb[r * 33 + lane] = lane < ncol ? xp[r * dim + col0 + lane] : T(0);
-      for (int a = lane; a < nb; a += 32)
-        for (int r = 0; r < nrhs; r++) Ws[r * Wtot + a] = T(0);
-      __syncwarp();
-      // the children's updates, child by child (distinct rows within a child)
-      for (int k = P.child_ptr[s]; k < P.child_ptr[s + 1]; k++) {
-        const int c = P.child_list[k];
-        const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
-        const int32_t* rel = P.relmap + P.relmap_off[c];
-        const T* Wc = W + P.sn_Woff[c];
-        for (int a = lane; a < nbc; a += 32) {
-          const int row = rel[a];
-          for (int r = 0; r < nrhs; r++) {
-            const T v = Wc[r * Wtot + a];
-            if (row < ncol) tb[r * 33 + row] += v;
-            else Ws[r * Wtot + row - ncol] += v;
-          }
-        }
-        __syncwarp();
-      }
-      // y = L11^-1 t (unit lower inverse, lane = row)
-      for (int r = 0; r < nrhs; r++) {
-        T y = T(0);
-#pragma unroll 8
-        for (int u = 0; u < 32; u++) y += iv[lane * 33 + u] * tb[r * 33 + u];
-        __syncwarp();
-        tb[r * 33 + lane] = lane < ncol ? y : T(0);
-        if (lane < ncol) xp[r * dim + col0 + lane] = y;
-      }
-      __syncwarp();
-      // W_s -= L21 y (lane = row below, 16-byte vectors of its row)
-      using V = typename Vec16<T>::type;
-      constexpr int VW = Vec16<T>::n;
-      const int nv = (ncol + VW - 1) / VW;
-      for (int a = lane; a < nb; a += 32) {
-        const V* row = reinterpret_cast<const V*>(N.L + P.sn_Loff[s] + (int64_t)(ncol + a) * ncp);
-        T acc[MAX_RHS_SWEEP];
-#pragma unroll
-        for (int r = 0; r < MAX_RHS_SWEEP; r++) acc[r] = T(0);
-        for (int v = 0; v < nv; v++) {
-          const V lv = __ldg(row + v);
-#pragma unroll
-          for (int e = 0; e < VW; e++) {
-            const int k = v * VW + e;
-            if (k >= ncol) break;
-            const T l = reinterpret_cast<const T*>(&lv)[e];
-#pragma unroll
-            for (int r = 0; r < MAX_RHS_SWEEP; r++)
-              if (r < nrhs) acc[r] += l * tb[r * 33 + k];
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < MAX_RHS_SWEEP; r++)
-          if (r < nrhs) Ws[r * Wtot + a] -= acc[r];
-      }
-      __syncwarp();
-    }
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_region_bwd(DevPlan P, DevNum<T> N, const int2* __restrict__ items, int count,
-                                                    const int32_t* __restrict__ nodes, T* __restrict__ xp, int nrhs,
-                                                    int* counter) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* iv = reinterpret_cast<T*>(smem_raw) + warp * (32 * 33 + MAX_RHS_SWEEP * 33);
-  T* zb = iv + 32 * 33;                              // [MAX_RHS_SWEEP][33]
-  const int64_t dim = P.dim;
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(counter, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= count) break;
-    const int2 item = items[it];
-    for (int q = item.y - 1; q >= 0; q--) {
-      const int s = nodes[item.x + q];
-      const int ncol = P.sn_ncol[s], nb = P.sn_nrow[s] - ncol, ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
-      const T* Lb = N.L + P.sn_Loff[s] + (int64_t)ncol * ncp;
-      const int32_t* rows = P.sn_rows + P.sn_rows_off[s] + ncol;
-      region_stage_inverse(P, N, s, iv, lane);
-      // z = D^-1 y - L21^T x_below (lane = column): x_below is gathered 32
-      // rows at a time (lane = row, the gathers of a chunk independent), then
-      // each row of L21 is read whole by the warp and its x value taken from
-      // the row's lane by a shuffle
-      const T dk = lane < ncol ? N.D[col0 + lane] : T(1);
-      T acc[MAX_RHS_SWEEP];
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++) acc[r] = T(0);
-      const int cl = min(lane, max(ncol - 1, 0));
-      for (int a0 = 0; a0 < nb; a0 += 32) {
-        const int a = a0 + lane;
-        const int row = a < nb ? rows[a] : 0;
-        T xb[MAX_RHS_SWEEP];
-#pragma unroll
-        for (int r = 0; r < MAX_RHS_SWEEP; r++) xb[r] = (r < nrhs && a < nb) ? xp[r * dim + row] : T(0);
-        const int cnt = min(32, nb - a0);
-        const T* lr = Lb + (int64_t)a0 * ncp + cl;
-#pragma unroll 8
-        for (int u = 0; u < cnt; u++) {
-          const T l = lr[(int64_t)u * ncp];
-#pragma unroll
-          for (int r = 0; r < MAX_RHS_SWEEP; r++)
-            if (r < nrhs) acc[r] += l * __shfl_sync(0xffffffffu, xb[r], u);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < MAX_RHS_SWEEP; r++)
-        if (r < nrhs) zb[r * 33 + lane] = lane < ncol ? xp[r * dim + col0 + lane] / dk - acc[r] : T(0);
-      __syncwarp();
-      // x = L11^-T z (lane = column of the inverse)
-      for (int r = 0; r < nrhs; r++) {
-        T x = T(0);
-#pragma unroll 8
-        for (int u = 0; u < 32; u++) x += iv[u * 33 + lane] * zb[r * 33 + u];
-        if (lane < ncol) xp[r * dim + col0 + lane] = x;
-      }
-      __syncwarp();
-    }
-  }
-}
-
-int region_smem(int esz) { return REG_WARPS * (32 * 33 + MAX_RHS_SWEEP * 33) * esz; }
-
-template <typename T>
-void launch_region_fwd(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const int32_t* nodes, T* xp,
-                       T* W, int nrhs, int* counter, int nsm, cudaStream_t st) {
-  if (count <= 0) return;
-  static bool attr = false;
-  const int smem = region_smem((int)sizeof(T));
-  if (!attr) {
-    cudaFuncSetAttribute(k_region_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
-  // as many CTAs as fit on the device at once (the warps take subtrees from a counter)
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_region_fwd<T>, 32 * REG_WARPS, smem) != cudaSuccess)
-    per_sm = 4;
-  const int grid = std::min((count + REG_WARPS - 1) / REG_WARPS, nsm * std::max(per_sm, 1));
-  k_region_fwd<T><<<grid, 32 * REG_WARPS, smem, st>>>(P, N, items, count, nodes, xp, W, nrhs, counter);
-}
-
-template <typename T>
-void launch_region_bwd(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const int32_t* nodes, T* xp,
-                       int nrhs, int* counter, int nsm, cudaStream_t st) {
-  if (count <= 0) return;
-  static bool attr = false;
-  const int smem = region_smem((int)sizeof(T));
-  if (!attr) {
-    cudaFuncSetAttribute(k_region_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_region_bwd<T>, 32 * REG_WARPS, smem) != cudaSuccess)
-    per_sm = 4;
-  const int grid = std::min((count + REG_WARPS - 1) / REG_WARPS, nsm * std::max(per_sm, 1));
-  k_region_bwd<T><<<grid, 32 * REG_WARPS, smem, st>>>(P, N, items, count, nodes, xp, nrhs, counter);
 }
 
 // ---------------------------------------------------------------------------
@@ -1388,25 +503,5 @@ void launch_slack_step(const DevPlan& P, const double* Jv, const double* rho, co
   if (total == 0) return;
   k_slack_step<<<grid_for(total), 256, 0, st>>>(P, Jv, rho, ss, nrhs, DT, ldt, RS, ldr, DS, lds);
 }
-
-#define NCL_INST(T)                                                                                               \
-  template void launch_perm_in<T>(const DevPlan&, T*, const double*, int64_t, int, cudaStream_t);                 \
-  template void launch_perm_out<T>(const DevPlan&, const T*, double*, int64_t, int, int, cudaStream_t);           \
-  template void launch_fwd_chain<T>(const DevPlan&, const DevNum<T>&, const int4*, int, int, bool,               \
-                                    const int32_t*, const int4*, T*, const T*, int, int*, int*, int*,            \
-                                    long long, cudaStream_t);                                                     \
-  template void launch_fwd_below<T>(const DevPlan&, const DevNum<T>&, const int2*, const int32_t*, const int4*,  \
-                                    int, T*, T*, int, cudaStream_t);                                              \
-  template void launch_bwd_below<T>(const DevPlan&, const DevNum<T>&, const int4*, int, int, const T*, T*, int,   \
-                                    cudaStream_t);                                                                \
-  template void launch_bwd_chain<T>(const DevPlan&, const DevNum<T>&, const int4*, int, int, bool, T*, const T*, \
-                                    int, int*, int*, int*, long long, cudaStream_t);                            \
-  template void launch_region_fwd<T>(const DevPlan&, const DevNum<T>&, const int2*, int, const int32_t*, T*, T*, \
-                                     int, int*, int, cudaStream_t);                                              \
-  template void launch_region_bwd<T>(const DevPlan&, const DevNum<T>&, const int2*, int, const int32_t*, T*, int, \
-                                     int*, int, cudaStream_t);
-NCL_INST(float)
-NCL_INST(double)
-#undef NCL_INST
 
 }  // namespace ncl
