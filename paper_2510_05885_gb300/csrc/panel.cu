@@ -1,6 +1,7 @@
 // Dense front kernels (sm_103a): the per-step macro-panel kernel of large
 // fronts (the roles are in panel_roles.cuh), and whole small fronts.
 #include "panel_roles.cuh"
+#include "panel8.cuh"
 
 #include <algorithm>
 
@@ -16,7 +17,7 @@ namespace ncl {
 // items: (front, q0, sync slot); sync[slot] = ticket counter, sync[slot + 1
 // + j] = flag of sub-block j.
 template <typename T, int NB>
-__global__ void __launch_bounds__(256, 1) k_macro_panel(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_macro_panel(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
                                                         int* sync, int* err, double eps, int policy,
                                                         long long wait) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -42,7 +43,11 @@ __global__ void __launch_bounds__(256, 1) k_macro_panel(DevPlan P, DevNum<T> N, 
 // sub-block follows, the warps update its columns.  The update
 // block F22 -= L21 D1 L21^T is left to the SIMT update kernel, which spreads
 // it over many CTAs.
-int small_front_smem(int nrow, int ncp, int esz) { return (nrow * (ncp + 1) + 2 * 32 * LDS + 64) * esz; }
+int small_front_smem(int nrow, int ncp, int esz) {
+  if (esz == 4)   // front, panel rows, pivot block and its inverse, pivots, signs and statuses
+    return (nrow * panel8_ld(ncp) + (64 + nrow) * P8_LD + 2 * 32 * LDS + 64) * 4 + 128;
+  return (nrow * (ncp + 1) + 2 * 32 * LDS + 64) * esz;
+}
 
 // Write a shared-memory front back.  A pivot block of one sub-block (at most 32
 // columns) is written as its inverse Iv, which the sweeps apply; wider ones
@@ -52,6 +57,41 @@ __device__ __forceinline__ void store_front(T* Lg, const T* F, const T* Iv, int 
   for (int idx = threadIdx.x; idx < nrow * ncp; idx += blockDim.x) {
     const int r = idx / ncp, c = idx - r * ncp;
     Lg[idx] = (r < ncol && c < r && ncol <= 32) ? Iv[r * LDS + c] : F[r * ldf + c];
+  }
+}
+
+// FP32: the pivot columns of a shared-memory front (rows x ncol, stride
+// panel8_ld(ncp)), eight at a time, the pivots and statuses to global memory
+// and, for a front of one 32-column sub-block, the inverse of its pivot block
+// to Iv (by warp 0; the other warps go on).  256 threads.
+__device__ __forceinline__ void factor_front32(const DevPlan& P, const DevNum<float>& N, float* F, int ldf, int nrow,
+                                               int ncol, int col0, float* Ls, float* Xs, float* Lu, float* Iv,
+                                               float* dsh, int8_t* sg, double eps, int policy) {
+  int8_t* pst = sg + 64;
+  const int tid = threadIdx.x;
+  if (tid < 64) sg[tid] = tid < ncol ? P.col_sign[col0 + tid] : 1;
+  __syncthreads();
+  int c = 0;
+  auto put = [&](int row, float (&l)[8]) { panel8_put(F + row * ldf + c, l, min(8, ncol - c)); };
+  if (nrow <= 256) {
+#pragma unroll 1
+    for (; c + 8 <= ncol; c += 8)
+      panel8_step<256, 1, true>(F, ldf, c, ncol, nrow, sg, (float)eps, policy, Ls, Xs, dsh, pst, put);
+  } else {
+#pragma unroll 1
+    for (; c + 8 <= ncol; c += 8)
+      panel8_step<256, 2, true>(F, ldf, c, ncol, nrow, sg, (float)eps, policy, Ls, Xs, dsh, pst, put);
+  }
+  if (c < ncol) panel8_step<256, 2, false>(F, ldf, c, ncol, nrow, sg, (float)eps, policy, Ls, Xs, dsh, pst, put);
+  if (tid < ncol) {
+    N.D[col0 + tid] = dsh[tid];
+    N.piv[col0 + tid] = pst[tid];
+  }
+  if (ncol <= 32 && tid < 32) {
+#pragma unroll 4
+    for (int u = 0; u < 32; u++) Lu[tid * LDS + u] = (u < tid && tid < ncol) ? F[tid * ldf + u] : 0.f;
+    __syncwarp();
+    invert_sub32<float>(Lu, Iv, ncol, tid);
   }
 }
 
@@ -66,6 +106,27 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_factor_small(DevPlan P, DevNu
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int s = list[blockIdx.x];
   const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
+  if constexpr (sizeof(T) == 4) {
+    const int ldf = panel8_ld(ncp);
+    float* F = reinterpret_cast<float*>(smem_raw);
+    float* Ls = F + nrow * ldf;
+    float* Xs = Ls + 64 * P8_LD;
+    float* Lu = Xs + nrow * P8_LD;
+    float* Iv = Lu + 32 * LDS;
+    float* dsh = Iv + 32 * LDS;
+    float* Lg = N.L + P.sn_Loff[s];
+    load_tile(F, ldf, Lg, ncp, nrow, ncp, [](int, int) { return true; });
+    factor_front32(P, N, F, ldf, nrow, ncol, col0, Ls, Xs, Lu, Iv, dsh, reinterpret_cast<int8_t*>(dsh + 64), eps, policy);
+    // rows below first: warp 0 may still be inverting the pivot block
+    const int nw = ncol <= 32 ? 7 : 8, w0 = 8 - nw;
+    const int warp = threadIdx.x >> 5;
+    if (warp >= w0)
+      for (int idx = (warp - w0) * 32 + (threadIdx.x & 31) + ncol * ncp; idx < nrow * ncp; idx += 32 * nw)
+        Lg[idx] = F[(idx / ncp) * ldf + idx % ncp];
+    __syncthreads();
+    store_front<T>(Lg, F, Iv, ncol, ncol, ncp, ldf);
+    return;
+  }
   const int ldf = ncp + 1;   // odd: column accesses by lanes are conflict-free
   T* F = reinterpret_cast<T*>(smem_raw);
   T* Ls = F + nrow * ldf;     // the sub-block's unit lower factor, zero padded

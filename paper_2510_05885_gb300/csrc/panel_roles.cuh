@@ -19,8 +19,10 @@
 #pragma once
 #include "runtime.h"
 #include "pivot.cuh"
+#include "panel8.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace ncl {
 
@@ -61,8 +63,12 @@ __device__ __forceinline__ void load_tile(T* dst, int ldd, const T* src, int64_t
 }
 
 // shared memory of the two roles of a panel nb columns wide (row stride nb + 1)
-inline int macro_diag_smem(int esz, int nb) { return (nb * (nb + 1) + (nb - 32) * LDS + nb) * esz + 2 * nb; }
+inline int macro_diag_smem(int esz, int nb) {
+  if (esz == 4) return 3 * nb * P8_LD * 4 + 2 * nb;
+  return (nb * (nb + 1) + (nb - 32) * LDS + nb) * esz + 2 * nb;
+}
 inline int macro_rows_smem(int esz, int nb) {
+  if (esz == 4) return ((RB + nb) * panel8_ld(nb) + nb) * 4;   // the rows, L11, D1
   const int k = nb / 32;   // the diagonal sub-blocks of L11 and those below them
   return (RB * (nb + 1) + (k + k * (k - 1) / 2) * 32 * LDS + nb) * esz;
 }
@@ -304,7 +310,148 @@ __device__ __forceinline__ void block_update(T* A, int LDM, const T* Xs, int c0,
   }
 }
 
-// Diagonal role of a macro panel (one CTA of 256 threads): factors the w x w
+// Diagonal role of a macro panel, FP32 (one CTA of 256 threads): factors the
+// w x w diagonal block (w <= 128), eight columns at a time.  The block's lower
+// part stays in registers, as 72 tiles of 16 x 8 dealt out to the warps
+// column by column (a lane holds rows g, g + 8 and columns 2 t, 2 t + 1 of a
+// tile, g = lane / 4, t = lane % 4); only the panel in work is in shared
+// memory.  Per panel: its tiles are written there; the warps with rows below
+// factor the 8 x 8 diagonal block, all lanes the same, and substitute a row
+// per thread (panel8.cuh); then every warp subtracts X L^T from its later
+// tiles.  What bounds it is that chain, about a thousand cycles a panel: eight
+// reciprocals and a substitution between two barriers.  (Measured on one CTA,
+// 128 columns: a 32-column block by one warp with shuffle broadcasts 80k
+// cycles, the trailing part in shared memory instead of registers 59k.)
+// L goes to global memory as it is found; after every 32 columns the
+// sub-block is published (fence, release flag) for the row CTAs.
+template <int MNB>
+__device__ __forceinline__ void panel_diag_role32(const DevPlan& P, const DevNum<float>& N, int s, int q0, int* flags,
+                                                  double eps, int policy, unsigned char* smem_raw) {
+  static_assert(MNB == 128, "the tiles are dealt out for 128 columns");
+  constexpr int NS = 9;                             // tiles per warp
+  float* Pb = reinterpret_cast<float*>(smem_raw);   // the panel's rows, two buffers
+  float* Ls = Pb + 2 * MNB * P8_LD;                 // L of the rows below it
+  int8_t* sg = reinterpret_cast<int8_t*>(Ls + MNB * P8_LD);
+  const int ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
+  const int w = min(MNB, ncol - q0);
+  float* Lb = N.L + P.sn_Loff[s] + (int64_t)q0 * ncp + q0;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t2 = 2 * (lane & 3);
+  // tile k of the list (column by column, rows from the diagonal down) is
+  // slot k / 8 of warp k % 8
+  int tr[NS], tj[NS];
+  {
+    int j = 0, i = warp;   // i counts from the column's first tile
+#pragma unroll
+    for (int k = 0; k < NS; k++) {
+      while (i >= 8 - j / 2) {
+        i -= 8 - j / 2;
+        j++;
+      }
+      tj[k] = j;
+      tr[k] = 16 * (i + j / 2) + g;
+      i += 8;
+    }
+  }
+  float acc[NS][4];
+#pragma unroll
+  for (int k = 0; k < NS; k++) {
+    const int c = 8 * tj[k] + t2;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int r = tr[k] + 8 * h;
+      float2 v = make_float2(0.f, 0.f);
+      if (r < w && c <= r) v = *reinterpret_cast<const float2*>(Lb + (int64_t)r * ncp + c);
+      acc[k][2 * h] = v.x;
+      acc[k][2 * h + 1] = c < r ? v.y : 0.f;
+    }
+  }
+  for (int c = tid; c < MNB; c += 256) sg[c] = c < w ? P.col_sign[col0 + q0 + c] : 1;
+  auto panel = [&](int c, auto full) {
+    constexpr bool FULL = decltype(full)::value;
+    float* Pp = Pb + ((c >> 3) & 1) * MNB * P8_LD;
+#pragma unroll
+    for (int k = 0; k < NS; k++)
+      if (8 * tj[k] == c) {
+        *reinterpret_cast<float2*>(Pp + tr[k] * P8_LD + t2) = make_float2(acc[k][0], acc[k][1]);
+        *reinterpret_cast<float2*>(Pp + (tr[k] + 8) * P8_LD + t2) = make_float2(acc[k][2], acc[k][3]);
+      }
+    __syncthreads();
+    const int pc = FULL ? 8 : w - c, rb = c + pc, R = w - rb;
+    const bool own = warp == 7;
+    float x[8], rk[8], dk[8], pr[8];
+    if (own || 32 * warp < R) {
+      float a[8][8];
+      const int8_t st = panel8_factor<FULL>(Pp + c * P8_LD, P8_LD, pc, sg + c, (float)eps, policy, own ? lane : -1, a, rk);
+#pragma unroll
+      for (int u = 0; u < 8; u++) dk[u] = a[u][u];
+      if (tid < R) {
+        float* xr = Pp + (rb + tid) * P8_LD;
+        panel8_solve<FULL>(xr, pc, a, x);
+        if (FULL) {
+          put8(xr, x);
+          float l[8];
+#pragma unroll
+          for (int u = 0; u < 8; u++) l[u] = div8(x[u], rk[u], dk[u]);
+          put8(Ls + (rb + tid) * P8_LD, l);
+        }
+      }
+      if (own) {
+        float d;
+        panel8_row(a, lane, pr, d);
+        if (lane < pc) {
+          N.D[col0 + q0 + c + lane] = d;
+          N.piv[col0 + q0 + c + lane] = st;
+          float* gr = Lb + (int64_t)(c + lane) * ncp + c;
+#pragma unroll
+          for (int u = 0; u < 8; u++)
+            if (u <= lane) gr[u] = pr[u];
+        }
+      }
+    }
+    if (tid < R) {
+      float* gr = Lb + (int64_t)(rb + tid) * ncp + c;
+      float l[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++) l[u] = div8(x[u], rk[u], dk[u]);
+      panel8_put(gr, l, pc);
+    }
+    __syncthreads();
+    if (((c & 31) == 24 || rb == w) && tid == 0) {
+      __threadfence();
+      st_release_i32(flags + c / 32, 1);
+    }
+    if (!FULL) return;
+    // later tiles: C -= X L^T
+#pragma unroll
+    for (int k = 0; k < NS; k++)
+      if (8 * tj[k] > c) {
+        float xa[2][8], la[2][8];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const float4* xp = reinterpret_cast<const float4*>(Pp + (tr[k] + 8 * h) * P8_LD);
+          const float4* lp = reinterpret_cast<const float4*>(Ls + (8 * tj[k] + t2 + h) * P8_LD);
+          const float4 x0 = xp[0], x1 = xp[1], l0 = lp[0], l1 = lp[1];
+          xa[h][0] = x0.x; xa[h][1] = x0.y; xa[h][2] = x0.z; xa[h][3] = x0.w;
+          xa[h][4] = x1.x; xa[h][5] = x1.y; xa[h][6] = x1.z; xa[h][7] = x1.w;
+          la[h][0] = l0.x; la[h][1] = l0.y; la[h][2] = l0.z; la[h][3] = l0.w;
+          la[h][4] = l1.x; la[h][5] = l1.y; la[h][6] = l1.z; la[h][7] = l1.w;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; u++)
+#pragma unroll
+          for (int h = 0; h < 2; h++) {
+            acc[k][2 * h] -= xa[h][u] * la[0][u];
+            acc[k][2 * h + 1] -= xa[h][u] * la[1][u];
+          }
+      }
+  };
+  int c = 0;
+#pragma unroll 1
+  for (; c + 8 <= w; c += 8) panel(c, std::true_type{});
+  if (c < w) panel(c, std::false_type{});
+}
+
+// Diagonal role of a macro panel, FP64 (FP32: see above; one CTA of 256 threads): factors the w x w
 // diagonal block (w <= 128) in shared memory by 32-column sub-blocks.  For
 // sub-block j: the rows below it inside the block are solved by the blocked
 // forward substitution, X = F21 L_jj^-T, and scaled, L21 = X D^-1; the next
@@ -316,6 +463,10 @@ __device__ __forceinline__ void block_update(T* A, int LDM, const T* Xs, int c0,
 template <typename T, int MNB>
 __device__ __forceinline__ void panel_diag_role(const DevPlan& P, const DevNum<T>& N, int s, int q0, int* flags,
                                                 double eps, int policy, unsigned char* smem_raw) {
+  if constexpr (sizeof(T) == 4) {
+    panel_diag_role32<MNB>(P, N, s, q0, flags, eps, policy, smem_raw);
+    return;
+  }
   constexpr int LDM = MNB + 1;   // shared row stride of the diagonal block
   T* A = reinterpret_cast<T*>(smem_raw);   // w x w block, row stride LDM
   T* Xs = A + MNB * LDM;                   // X of the rows below the sub-block
@@ -419,7 +570,132 @@ __device__ __forceinline__ void panel_diag_role(const DevPlan& P, const DevNum<T
   for (int c = tid; c < w; c += blockDim.x) N.piv[col0 + q0 + c] = pst[c];
 }
 
-// Row role of a macro panel (one CTA of 256 threads per RB rows below it): stages its rows
+// wait (bounded) for a sub-block's flag; thread 0 only
+__device__ __forceinline__ void panel_wait(const int* flag, int* err, long long wait) {
+  if (ld_acquire_i32(flag) || ld_acquire_i32(err)) return;
+  const long long t0 = clock64();
+  while (!ld_acquire_i32(flag)) {
+    if (clock64() - t0 > wait || ld_acquire_i32(err)) {
+      atomicExch(err, 1);
+      break;
+    }
+    __nanosleep(64);
+  }
+}
+
+// Row role of a macro panel, FP32 (one CTA of 256 threads per RB = 64 rows
+// below it): stages its rows while the diagonal role works; as each 32-column
+// sub-block of L11 is published, the rows go through its columns eight at a
+// time: four lanes to a row substitute with the 8 x 8 diagonal block, X = R
+// L^-T (each lane all eight values), then subtract X L^T from every fourth of
+// the row's later columns.  The four lanes belong to one warp, so no barrier
+// is needed between panels, and the lanes' columns interleave, so that the
+// shared accesses are free of bank conflicts.  Leaves X in R.
+template <int MNB>
+__device__ __forceinline__ void panel_rows_solve32(const DevPlan& P, const DevNum<float>& N, int s, int q0, int r0,
+                                                   const int* flags, int* err, long long wait, float* R, float* L,
+                                                   float* dsh) {
+  constexpr int LDM = MNB + 4;
+  const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
+  const int w = min(MNB, ncol - q0), nr = min(RB, nrow - r0);
+  const int tid = threadIdx.x;
+  float* Lb = N.L + P.sn_Loff[s];
+  {
+    // the rows (16-byte vectors; columns past w are zero)
+    constexpr int V = RB * MNB / 4 / 256;
+    float4 v[V];
+#pragma unroll
+    for (int k = 0; k < V; k++) {
+      const int idx = tid + 256 * k, r = idx / (MNB / 4), c = 4 * (idx % (MNB / 4));
+      v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < nr && c < w) {
+        v[k] = __ldcg(reinterpret_cast<const float4*>(Lb + (int64_t)(r0 + r) * ncp + q0 + c));
+        if (c + 1 >= w) v[k].y = 0.f;
+        if (c + 2 >= w) v[k].z = 0.f;
+        if (c + 3 >= w) v[k].w = 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < V; k++) {
+      const int idx = tid + 256 * k;
+      *reinterpret_cast<float4*>(R + (idx / (MNB / 4)) * LDM + 4 * (idx % (MNB / 4))) = v[k];
+    }
+  }
+  const int row = tid >> 2, q = tid & 3;
+  float* Rr = R + row * LDM;
+#pragma unroll 1
+  for (int j = 0; 32 * j < w; j++) {
+    if (tid == 0) panel_wait(flags + j, err, wait);
+    __syncthreads();
+    {
+      // columns [32 j, 32 j + 32) of L11 below the diagonal, zero elsewhere
+      float4 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int idx = tid + 256 * k, r = 32 * j + (idx >> 3), c = 32 * j + 4 * (idx & 7);
+        v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < w && c < r) v[k] = __ldcg(reinterpret_cast<const float4*>(Lb + (int64_t)(q0 + r) * ncp + q0 + c));
+      }
+      if (tid < 32) dsh[32 * j + tid] = 32 * j + tid < w ? __ldcg(N.D + col0 + q0 + 32 * j + tid) : 1.f;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int idx = tid + 256 * k, r = 32 * j + (idx >> 3), c = 32 * j + 4 * (idx & 7);
+        if (r < MNB) {
+          if (c + 1 >= r) v[k].y = 0.f;
+          if (c + 2 >= r) v[k].z = 0.f;
+          if (c + 3 >= r) v[k].w = 0.f;
+          *reinterpret_cast<float4*>(L + r * LDM + c) = v[k];
+        }
+      }
+    }
+    __syncthreads();
+    const int ce = min(32 * j + 32, w);
+#pragma unroll 1
+    for (int c = 32 * j; c < ce; c += 8) {
+      float x[8];
+      {
+        const float4 v0 = *reinterpret_cast<const float4*>(Rr + c);
+        const float4 v1 = *reinterpret_cast<const float4*>(Rr + c + 4);
+        x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w;
+        x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
+      }
+#pragma unroll
+      for (int i = 1; i < 8; i++) {
+        const float* lr = L + (c + i) * LDM + c;
+        const float4 l0 = *reinterpret_cast<const float4*>(lr);
+        const float4 l1 = i > 4 ? *reinterpret_cast<const float4*>(lr + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float l[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
+#pragma unroll
+        for (int k = 0; k < i; k++) x[i] -= x[k] * l[k];
+      }
+      __syncwarp();
+      if (q == 0) {
+        *reinterpret_cast<float4*>(Rr + c) = make_float4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<float4*>(Rr + c + 4) = make_float4(x[4], x[5], x[6], x[7]);
+      }
+#pragma unroll 1
+      for (int cb = c + 8 + q; cb < w; cb += 16) {
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const int cc = cb + 4 * i;
+          if (cc < w) {
+            const float* lr = L + cc * LDM + c;
+            const float4 l0 = *reinterpret_cast<const float4*>(lr);
+            const float4 l1 = *reinterpret_cast<const float4*>(lr + 4);
+            float v = x[0] * l0.x + x[1] * l0.y + x[2] * l0.z + x[3] * l0.w;
+            v += x[4] * l1.x + x[5] * l1.y + x[6] * l1.z + x[7] * l1.w;
+            Rr[cc] -= v;
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+}
+
+// Row role of a macro panel (one CTA of 256 threads per RB rows below it; FP32 solves
+// them as above): stages its rows
 // while the diagonal role works, then for each 32-column sub-block j, as
 // soon as it is published, X_j = R_j L_jj^-T by the blocked forward
 // substitution and R_i -= X_j L_ij^T for the later sub-blocks (lane =
@@ -429,83 +705,77 @@ template <typename T, int MNB>
 __device__ __forceinline__ void panel_rows_role(const DevPlan& P, const DevNum<T>& N, int s, int q0, int r0,
                                                 const int* flags, int* err, long long wait,
                                                 unsigned char* smem_raw) {
-  constexpr int LDM = MNB + 1;
+  constexpr bool F32 = sizeof(T) == 4;
+  constexpr int LDM = F32 ? MNB + 4 : MNB + 1;
   constexpr int KB = MNB / 32;             // sub-blocks of the panel
   T* R = reinterpret_cast<T*>(smem_raw);   // RB rows x w columns, stride LDM
-  T* Ld = R + RB * LDM;                    // the KB unit lower diagonal sub-blocks of L11
-  T* Lo = Ld + KB * 32 * LDS;              // the KB (KB - 1) / 2 off-diagonal sub-blocks (i > j) of L11
-  T* dsh = Lo + (KB * (KB - 1) / 2) * 32 * LDS;   // D1
+  T* Ld = R + RB * LDM;                    // FP32: L11, stride LDM; FP64: its KB unit lower diagonal sub-blocks
+  T* Lo = Ld + KB * 32 * LDS;              // FP64: the KB (KB - 1) / 2 off-diagonal sub-blocks (i > j) of L11
+  T* dsh = F32 ? Ld + MNB * LDM : Lo + (KB * (KB - 1) / 2) * 32 * LDS;   // D1
   const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
   const int w = min(MNB, ncol - q0);
   const int nbk = (w + 31) / 32;
   const int nr = min(RB, nrow - r0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   T* Lb = N.L + P.sn_Loff[s];
-  load_tile(R, LDM, Lb + (int64_t)r0 * ncp + q0, ncp, RB, MNB, [&](int r, int c) { return r < nr && c < w; });
   constexpr int KR = RB / 8;   // rows per warp in the updates (lane = column)
-  T* Rw = R + warp * LDM;      // row warp + 8 k is Rw[8 k LDM + ...]
-  for (int j = 0; j < nbk; j++) {
-    // wait (bounded) for sub-block j, then fetch its published columns
-    if (tid == 0) {
-      if (!ld_acquire_i32(flags + j) && !ld_acquire_i32(err)) {
-        const long long t0 = clock64();
-        while (!ld_acquire_i32(flags + j)) {
-          if (clock64() - t0 > wait || ld_acquire_i32(err)) {
-            atomicExch(err, 1);
-            break;
+  if constexpr (F32) {
+    panel_rows_solve32<MNB>(P, N, s, q0, r0, flags, err, wait, R, Ld, dsh);
+  } else {
+    load_tile(R, LDM, Lb + (int64_t)r0 * ncp + q0, ncp, RB, MNB, [&](int r, int c) { return r < nr && c < w; });
+    T* Rw = R + warp * LDM;      // row warp + 8 k is Rw[8 k LDM + ...]
+    for (int j = 0; j < nbk; j++) {
+      // wait (bounded) for sub-block j, then fetch its published columns
+      if (tid == 0) panel_wait(flags + j, err, wait);
+      __syncthreads();
+      {
+        // the published blocks (i, j), i >= j, and D_j: every load in flight
+        // before the shared stores (256 threads, four entries of each block)
+        T v[KB][4];
+#pragma unroll
+        for (int q = 0; q < KB; q++) {
+          const int i = j + q;
+          const int rows = min(32, w - 32 * i);
+          const T* src = Lb + (int64_t)(q0 + 32 * i) * ncp + q0 + 32 * j;
+#pragma unroll
+          for (int t = 0; t < 4; t++) {
+            const int e = tid + 256 * t, rr = e >> 5, cc = e & 31;
+            v[q][t] = (i < nbk && rr < rows && (i > j || cc < rr)) ? __ldcg(src + (int64_t)rr * ncp + cc) : T(0);
           }
-          __nanosleep(64);
         }
-      }
-    }
-    __syncthreads();
-    {
-      // the published blocks (i, j), i >= j, and D_j: every load in flight
-      // before the shared stores (256 threads, four entries of each block)
-      T v[KB][4];
+        const T dv = (tid < 32 && 32 * j + tid < w) ? __ldcg(N.D + col0 + q0 + 32 * j + tid) : T(1);
 #pragma unroll
-      for (int q = 0; q < KB; q++) {
-        const int i = j + q;
-        const int rows = min(32, w - 32 * i);
-        const T* src = Lb + (int64_t)(q0 + 32 * i) * ncp + q0 + 32 * j;
+        for (int q = 0; q < KB; q++) {
+          const int i = j + q;
+          if (i >= nbk) break;
+          T* dst = (i == j) ? Ld + i * 32 * LDS : Lo + (i * (i - 1) / 2 + j) * 32 * LDS;
 #pragma unroll
-        for (int t = 0; t < 4; t++) {
-          const int e = tid + 256 * t, rr = e >> 5, cc = e & 31;
-          v[q][t] = (i < nbk && rr < rows && (i > j || cc < rr)) ? __ldcg(src + (int64_t)rr * ncp + cc) : T(0);
+          for (int t = 0; t < 4; t++) {
+            const int e = tid + 256 * t;
+            dst[(e >> 5) * LDS + (e & 31)] = v[q][t];
+          }
         }
+        if (tid < 32) dsh[32 * j + tid] = dv;
       }
-      const T dv = (tid < 32 && 32 * j + tid < w) ? __ldcg(N.D + col0 + q0 + 32 * j + tid) : T(1);
+      __syncthreads();
+      block_trsm32<T>(R + 32 * j, LDM, nr, min(32, w - 32 * j), Ld + j * 32 * LDS, LDS);
+      __syncthreads();
+      for (int i = j + 1; i < nbk; i++) {
+        const T* lij = Lo + (i * (i - 1) / 2 + j) * 32 * LDS;
+        T x[KR];
 #pragma unroll
-      for (int q = 0; q < KB; q++) {
-        const int i = j + q;
-        if (i >= nbk) break;
-        T* dst = (i == j) ? Ld + i * 32 * LDS : Lo + (i * (i - 1) / 2 + j) * 32 * LDS;
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-          const int e = tid + 256 * t;
-          dst[(e >> 5) * LDS + (e & 31)] = v[q][t];
-        }
-      }
-      if (tid < 32) dsh[32 * j + tid] = dv;
-    }
-    __syncthreads();
-    block_trsm32<T>(R + 32 * j, LDM, nr, min(32, w - 32 * j), Ld + j * 32 * LDS, LDS);
-    __syncthreads();
-    for (int i = j + 1; i < nbk; i++) {
-      const T* lij = Lo + (i * (i - 1) / 2 + j) * 32 * LDS;
-      T x[KR];
-#pragma unroll
-      for (int k = 0; k < KR; k++) x[k] = T(0);
+        for (int k = 0; k < KR; k++) x[k] = T(0);
 #pragma unroll 4
-      for (int u = 0; u < 32; u++) {
-        const T b = lij[lane * LDS + u];
+        for (int u = 0; u < 32; u++) {
+          const T b = lij[lane * LDS + u];
 #pragma unroll
-        for (int k = 0; k < KR; k++) x[k] += Rw[8 * k * LDM + 32 * j + u] * b;
+          for (int k = 0; k < KR; k++) x[k] += Rw[8 * k * LDM + 32 * j + u] * b;
+        }
+#pragma unroll
+        for (int k = 0; k < KR; k++) Rw[8 * k * LDM + 32 * i + lane] -= x[k];
       }
-#pragma unroll
-      for (int k = 0; k < KR; k++) Rw[8 * k * LDM + 32 * i + lane] -= x[k];
+      __syncthreads();
     }
-    __syncthreads();
   }
   // L21 = X D1^-1 (+ split operands of L21 and W = X for a tensor-core front)
   int64_t so = -1;
@@ -521,7 +791,9 @@ __device__ __forceinline__ void panel_rows_role(const DevPlan& P, const DevNum<T
       const int r = warp + 8 * k;
       if (r >= nr) continue;
       const T xv = c < w ? R[r * LDM + c] : T(0);
-      const T l = xv * invd;
+      T l;
+      if constexpr (F32) l = c < w ? div8(xv, invd, dsh[c]) : 0.f;
+      else l = xv * invd;
       if (c < w) Lb[(int64_t)(r0 + r) * ncp + q0 + c] = l;
       if constexpr (sizeof(T) == 4) {
         if (so >= 0) {

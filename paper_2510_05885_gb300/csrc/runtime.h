@@ -20,7 +20,7 @@ constexpr int SWEEP_CHUNK_BYTES = 64 * 1024;   // staged vector of a sweep's str
 constexpr int SWEEP_BLOCK_BELOW = 1024;        // rows below its pivots, at most
 constexpr int SWEEP_BLOCK_BYTES = 96 * 1024;   // front of a supernode swept by one CTA, at most
 constexpr int SMALL_SMEM = 64 * 1024;      // front bytes (nrow x ncolp) of a small front, at most
-constexpr int SMALL_SMEM_MAX = 96 * 1024;  // dynamic smem limit of the small-front kernel
+constexpr int SMALL_SMEM_MAX = 112 * 1024;  // dynamic smem limit of the small-front kernel
 
 // What the sweeps need of a supernode, in one 48-byte record: factor block and
 // row offsets, first entry of W, first pivot, sizes.
