@@ -16,21 +16,20 @@ static unsigned grid_for(int64_t n, int per = 256) {
 }
 
 // ---------------------------------------------------------------------------
-// FP64 residual R = B - K X on the FP64 KKT values (4 lanes per row, 8 rows
-// per warp trip), with per-instance ||R||_inf and ||X||_inf (bit patterns,
-// atomicMax).  Kf holds the values of the full pattern in its row order
-// (written before ||K||), so the entries and column indices are read
-// contiguously and only X is gathered; an entry is read once for all NR
-// right-hand sides, and every load of a trip that does not depend on
-// another (row bounds, B, the row's own X) is issued before the products.
-// Each warp takes a contiguous run of rows, so that its running maxima
-// change instance (and go to the atomics) only at an instance boundary.
+// FP64 residual R = B - K X on the FP64 KKT values, with per-instance
+// ||R||_inf and ||X||_inf (bit patterns, atomicMax).  Kf holds the values of
+// the full pattern in its row order (written before ||K||), so the entries
+// and column indices are read contiguously and only X is gathered.  Each warp
+// takes a contiguous run of rows, so that its running maxima change instance
+// (and go to the atomics) only at an instance boundary.
+//
+// One right-hand side: 4 lanes per row, 8 rows per warp trip; every load of a
+// trip that does not depend on another (row bounds, B, the row's own X) is
+// issued before the products.
 // ---------------------------------------------------------------------------
-template <int NR>
 __global__ void __launch_bounds__(256) k_residual(DevPlan P, const double* __restrict__ Kf,
-                                                  const double* __restrict__ B, int64_t ldb,
-                                                  const double* __restrict__ X, int64_t ldx, double* __restrict__ R,
-                                                  int64_t ldr, int nrhs, unsigned long long* rnorm,
+                                                  const double* __restrict__ B, const double* __restrict__ X,
+                                                  double* __restrict__ R, unsigned long long* rnorm,
                                                   unsigned long long* xnorm, int64_t rows_per_warp) {
   constexpr int LPR = 4;   // lanes per row
   const int lane = threadIdx.x & 31, sub = lane & (LPR - 1);
@@ -39,9 +38,7 @@ __global__ void __launch_bounds__(256) k_residual(DevPlan P, const double* __res
   const int64_t r_end = min(P.dim, r_begin + rows_per_warp);
   // running maxima of |r| and |x| for the instance of this lane's rows
   int cur = -1;
-  unsigned long long rmx[NR], xmx[NR];
-#pragma unroll
-  for (int r = 0; r < NR; r++) rmx[r] = xmx[r] = 0ull;
+  unsigned long long rmx = 0ull, xmx = 0ull;
   // the trip count is uniform across the warp so that the full-mask
   // shuffles are safe
   for (int64_t rb = r_begin; rb < r_end; rb += 32 / LPR) {
@@ -49,63 +46,109 @@ __global__ void __launch_bounds__(256) k_residual(DevPlan P, const double* __res
     const bool valid = row < r_end;
     const int64_t q0 = valid ? P.F_rowptr[row] : 0, q1 = valid ? P.F_rowptr[row + 1] : 0;
     const int inst = valid ? P.row_inst[row] : -1;
-    double bv[NR], xv[NR];
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-      const bool use = valid && sub == 0 && r < nrhs;
-      bv[r] = use ? B[r * ldb + row] : 0.0;
-      xv[r] = use ? X[r * ldx + row] : 0.0;
-    }
-    double acc[NR];
-#pragma unroll
-    for (int r = 0; r < NR; r++) acc[r] = 0.0;
+    const bool use = valid && sub == 0;
+    const double bv = use ? B[row] : 0.0, xv = use ? X[row] : 0.0;
+    double acc = 0.0;
     int64_t q = q0 + sub;
     for (; q + LPR < q1; q += 2 * LPR) {
       const double k0 = Kf[q], k1 = Kf[q + LPR];
       const int64_t c0 = P.F_col[q], c1 = P.F_col[q + LPR];
-#pragma unroll
-      for (int r = 0; r < NR; r++)
-        if (r < nrhs) acc[r] = fma(k1, X[r * ldx + c1], fma(k0, X[r * ldx + c0], acc[r]));
+      acc = fma(k1, X[c1], fma(k0, X[c0], acc));
     }
-    if (q < q1) {
-      const double k0 = Kf[q];
-      const int64_t c0 = P.F_col[q];
-#pragma unroll
-      for (int r = 0; r < NR; r++)
-        if (r < nrhs) acc[r] = fma(k0, X[r * ldx + c0], acc[r]);
-    }
-    if (valid && sub == 0 && inst != cur) {
-      if (cur >= 0)
-#pragma unroll
-        for (int r = 0; r < NR; r++)
-          if (r < nrhs) {
-            atomicMax(&rnorm[cur * nrhs + r], rmx[r]);
-            atomicMax(&xnorm[cur * nrhs + r], xmx[r]);
-          }
-#pragma unroll
-      for (int r = 0; r < NR; r++) rmx[r] = xmx[r] = 0ull;
+    if (q < q1) acc = fma(Kf[q], X[P.F_col[q]], acc);
+    if (use && inst != cur) {
+      if (cur >= 0) {
+        atomicMax(&rnorm[cur], rmx);
+        atomicMax(&xnorm[cur], xmx);
+      }
+      rmx = xmx = 0ull;
       cur = inst;
     }
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-      if (r >= nrhs) break;
-      double a = acc[r];
-      a += __shfl_xor_sync(FULL_MASK, a, 2);
-      a += __shfl_xor_sync(FULL_MASK, a, 1);
-      if (valid && sub == 0) {
-        const double res = bv[r] - a;
-        R[r * ldr + row] = res;
-        const unsigned long long u = dbits(fabs(res)), v = dbits(fabs(xv[r]));
-        rmx[r] = u > rmx[r] ? u : rmx[r];
-        xmx[r] = v > xmx[r] ? v : xmx[r];
-      }
+    acc += __shfl_xor_sync(FULL_MASK, acc, 2);
+    acc += __shfl_xor_sync(FULL_MASK, acc, 1);
+    if (use) {
+      const double res = bv - acc;
+      R[row] = res;
+      const unsigned long long u = dbits(fabs(res)), v = dbits(fabs(xv));
+      rmx = u > rmx ? u : rmx;
+      xmx = v > xmx ? v : xmx;
     }
   }
+  warp_flush_max(rnorm, cur, rmx);
+  warp_flush_max(xnorm, cur, xmx);
+}
+
+// Several right-hand sides: one lane per (row, right-hand side), 32 / NR rows
+// per warp trip.  FP64 runs at two products per clock and SM here, so what
+// counts is the number of FP64 warp instructions: a lane that owns its sum
+// needs no additions across lanes and no idle lanes at the end of a row.
+// With 4 lanes per row that each carried all right-hand sides: 64 scenarios
+// of 100 buses, 4 of them: 1.42 -> 0.91 ms; 300x300, 8 of them: 0.45 ->
+// 0.29 ms (0.7 TFLOP/s).  Gathering X from an interleaved copy instead gave
+// nothing (0.96 and 0.28 ms with the copy): the gathers are not the bound.
+template <int NR>
+__global__ void __launch_bounds__(256) k_residual_rhs(DevPlan P, const double* __restrict__ Kf,
+                                                      const double* __restrict__ B, int64_t ldb,
+                                                      const double* __restrict__ X, int64_t ldx,
+                                                      double* __restrict__ R, int64_t ldr, int nrhs,
+                                                      unsigned long long* rnorm, unsigned long long* xnorm,
+                                                      int64_t rows_per_warp) {
+  constexpr int U = 4;   // entries in flight
+  const int lane = threadIdx.x & 31, r = lane & (NR - 1);
+  const int64_t gwarp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t r_begin = gwarp * rows_per_warp;
+  const int64_t r_end = min(P.dim, r_begin + rows_per_warp);
+  const double* Xr = X + min(r, nrhs - 1) * ldx;
+  int key = -1;   // instance * nrhs + right-hand side of the running maxima
+  unsigned long long rmx = 0ull, xmx = 0ull;
+  if (r < nrhs)
+    for (int64_t row = r_begin + lane / NR; row < r_end; row += 32 / NR) {
+      const int64_t q0 = P.F_rowptr[row], q1 = P.F_rowptr[row + 1];
+      const int k = P.row_inst[row] * nrhs + r;
+      const double bv = B[r * ldb + row], xv = Xr[row];
+      double a0 = 0.0, a1 = 0.0;
+      for (int64_t q = q0; q < q1; q += U) {
+        double kv[U], x[U];
 #pragma unroll
-  for (int r = 0; r < NR; r++) {
-    if (r >= nrhs) break;
-    warp_flush_max(rnorm + r, cur < 0 ? -1 : cur * nrhs, rmx[r]);
-    warp_flush_max(xnorm + r, cur < 0 ? -1 : cur * nrhs, xmx[r]);
+        for (int u = 0; u < U; u++) {
+          kv[u] = q + u < q1 ? Kf[q + u] : 0.0;
+          x[u] = q + u < q1 ? Xr[P.F_col[q + u]] : 0.0;
+        }
+        a0 = fma(kv[0], x[0], a0);
+#pragma unroll
+        for (int u = 1; u < U; u++)
+          if (q + u < q1) {
+            if (u & 1) a1 = fma(kv[u], x[u], a1);
+            else a0 = fma(kv[u], x[u], a0);
+          }
+      }
+      if (k != key) {
+        if (key >= 0) {
+          atomicMax(&rnorm[key], rmx);
+          atomicMax(&xnorm[key], xmx);
+        }
+        rmx = xmx = 0ull;
+        key = k;
+      }
+      const double res = bv - (a0 + a1);
+      R[r * ldr + row] = res;
+      const unsigned long long u = dbits(fabs(res)), v = dbits(fabs(xv));
+      rmx = u > rmx ? u : rmx;
+      xmx = v > xmx ? v : xmx;
+    }
+  // lanes of one right-hand side and one instance go to memory together
+  const int k0 = __shfl_sync(FULL_MASK, key, r);
+  const bool same = key == k0;
+  unsigned long long rw = same ? rmx : 0ull, xw = same ? xmx : 0ull;
+#pragma unroll
+  for (int o = 16; o >= NR; o >>= 1) {
+    const unsigned long long u = __shfl_xor_sync(FULL_MASK, rw, o), v = __shfl_xor_sync(FULL_MASK, xw, o);
+    rw = u > rw ? u : rw;
+    xw = v > xw ? v : xw;
+  }
+  if (key >= 0 && (lane < NR || !same)) {
+    atomicMax(&rnorm[key], same ? rw : rmx);
+    atomicMax(&xnorm[key], same ? xw : xmx);
   }
 }
 
@@ -116,14 +159,12 @@ void launch_residual(const DevPlan& P, const double* Kf, const double* B, int64_
   const unsigned grid = grid_for(P.dim * 8);
   const int64_t nwarp = (int64_t)grid * 8;
   const int64_t rpw = ((P.dim + nwarp - 1) / nwarp + 7) / 8 * 8;
-  if (nrhs <= 1)
-    k_residual<1><<<grid, 256, 0, st>>>(P, Kf, B, ldb, X, ldx, R, ldr, nrhs, rnorm, xnorm, rpw);
-  else if (nrhs <= 2)
-    k_residual<2><<<grid, 256, 0, st>>>(P, Kf, B, ldb, X, ldx, R, ldr, nrhs, rnorm, xnorm, rpw);
-  else if (nrhs <= 4)
-    k_residual<4><<<grid, 256, 0, st>>>(P, Kf, B, ldb, X, ldx, R, ldr, nrhs, rnorm, xnorm, rpw);
-  else
-    k_residual<MAX_RHS_SWEEP><<<grid, 256, 0, st>>>(P, Kf, B, ldb, X, ldx, R, ldr, nrhs, rnorm, xnorm, rpw);
+  if (nrhs <= 1) {
+    k_residual<<<grid, 256, 0, st>>>(P, Kf, B, X, R, rnorm, xnorm, rpw);
+    return;
+  }
+  const auto k = nrhs <= 2 ? k_residual_rhs<2> : nrhs <= 4 ? k_residual_rhs<4> : k_residual_rhs<8>;
+  k<<<grid, 256, 0, st>>>(P, Kf, B, ldb, X, ldx, R, ldr, nrhs, rnorm, xnorm, rpw);
 }
 
 // per-instance ||B||_inf; each CTA takes a contiguous run of rows (see k_knorm)
