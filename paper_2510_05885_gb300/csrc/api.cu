@@ -342,7 +342,7 @@ void build_schedule(ncl_kkt_s* h) {
   std::vector<GemmProb>& probv = hs.probv;
   hs.tc = is_fp32(h) && h->opt.use_tensor_cores;
   hs.dag = h->opt.persistent_fronts != 0;
-  const int PNB = MACRO_NB;   // pivot columns per panel step
+  const int PNB = panel_cols((int)esz), PRB = panel_rows((int)esz);   // pivot columns and rows per panel step
   hs.dagv.clear();
   hs.dag_counters = (int64_t)P.nlevels;   // one queue head per level first
   hs.inv64.clear();
@@ -435,7 +435,8 @@ void build_schedule(ncl_kkt_s* h) {
   // problems of one launch are pushed consecutively; each launch's tiles map
   // to its problems through a contiguous run of the per-tile index arrays
   auto push_gemm = [&](GemmProb g, int64_t prob_base, int64_t& tiles, Cost& c) {
-    const int Mt = (g.M + GEMM_TILE - 1) / GEMM_TILE, Nt = (g.N + GEMM_TILE - 1) / GEMM_TILE;
+    const int TB = gemm_tile((int)esz);
+    const int Mt = (g.M + TB - 1) / TB, Nt = (g.N + TB - 1) / TB;
     g.Nt = Nt;
     g.tile0 = tiles;
     const int64_t nt = (int64_t)Nt * (Nt + 1) / 2 + (int64_t)(Mt - Nt) * Nt;
@@ -608,14 +609,32 @@ void build_schedule(ncl_kkt_s* h) {
         const int q0 = m * PNB;
         if (q0 >= ncol) continue;
         const int qe = std::min(q0 + PNB, ncol), w = qe - q0;
-        // one diagonal CTA and one CTA per MACRO_ROWS rows below, sharing a
+        // one diagonal CTA and one CTA per PRB rows below, sharing a
         // sync slot (ticket counter, four sub-block flags)
-        const int nrc = (nrow - qe + MACRO_ROWS - 1) / MACRO_ROWS;
+        const int nrc = (nrow - qe + PRB - 1) / PRB;
         for (int k = 0; k <= nrc; k++) panelv.push_back(make_int4(s, q0, (int32_t)hs.panel_sync, 0));
         hs.panel_sync += 8;
         S.panel_cost.flops += 2.0 * w * (double)w * w / 3.0 + 32.0 * 32 * w + (double)(nrow - qe) * w * (w + 1.0);
         S.panel_cost.bytes += esz * ((double)w * (w + 1) + 1024.0 * ((w + 31) / 32) + 2.0 * w) +
                               esz * 2.0 * (nrow - qe) * w + (fid[s] >= 0 ? 16.0 * (nrow - qe) * w : 0.0);
+        if (esz == 8) {
+          // the previous panel's update of the columns to the right of this one
+          // (this panel's own share is taken by its CTAs)
+          if (m == 0 || qe >= ncol) continue;
+          GemmProb g{};
+          g.c_off = P.sn_Loff[s] + (int64_t)qe * ncp + qe;
+          g.a_off = P.sn_Loff[s] + (int64_t)qe * ncp + q0 - PNB;
+          g.b_off = g.a_off;
+          g.d_off = P.sn_col0[s] + q0 - PNB;
+          g.ldc = ncp;
+          g.lda = ncp;
+          g.M = nrow - qe;
+          g.N = ncol - qe;
+          g.K = PNB;
+          g.c_in_u = 0;
+          push_gemm(g, S.prob_off, S.tiles, S.gemm_cost);
+          continue;
+        }
         if (qe >= ncol) continue;
         if (fid[s] >= 0 && h->opt.use_tensor_cores > 1 && w % 32 == 0) {
           TcProb q{};
@@ -923,7 +942,7 @@ void build_schedule(ncl_kkt_s* h) {
         bad("small front smem");
     for (const Level& L : h->levels)
       if (L.small_smem > SMALL_SMEM_MAX) bad("small front smem");
-    // every sync slot is shared by exactly 1 + (rows below / MACRO_ROWS) items
+    // every sync slot is shared by exactly 1 + (rows below / PRB) items
     // of one front and panel (the roles come from the slot's ticket counter)
     for (size_t i = 0; i < panelv.size();) {
       const int4 it = panelv[i];
@@ -932,7 +951,7 @@ void build_schedule(ncl_kkt_s* h) {
           it.z + 8 > hs.panel_sync || it.z % 8)
         bad("macro panel item");
       const int qe = std::min(it.y + PNB, P.sn_ncol[s]);
-      const size_t n = 1 + (size_t)((P.sn_nrow[s] - qe + MACRO_ROWS - 1) / MACRO_ROWS);
+      const size_t n = 1 + (size_t)((P.sn_nrow[s] - qe + PRB - 1) / PRB);
       if (i + n > panelv.size()) bad("macro panel item");
       for (size_t k = 0; k < n; k++)
         if (panelv[i + k].x != s || panelv[i + k].y != it.y || panelv[i + k].z != it.z) bad("macro panel item");
@@ -1389,18 +1408,27 @@ void run_factor(ncl_kkt_s* h, DevNum<T>& N, cudaStream_t st) {
     }
     for (const Step& S : L.steps) {
       if (L.dag_cnt > 0) break;
-      klaunch(h, st, f32 ? "macro_panel_f32" : "macro_panel_f64", S.panel_cnt, S.panel_cost, [&] {
-        launch_macro_panel<T>(P, N, h->d_panel + S.panel_off, S.panel_cnt, h->d_panel_sync, h->d_err,
-                              eps, pol, h->opt.wait_cycles, st);
-      });
-      klaunch(h, st, f32 ? "update_simt_f32" : "update_simt_f64", S.tiles, S.gemm_cost, [&] {
-        launch_gemm_simt<T>(P, N, h->d_probs + S.prob_off, h->d_tilep + S.tp_off, S.tiles, st);
-      });
-      if constexpr (sizeof(T) == 4)
-        klaunch(h, st, "update_tc_f32", S.tc_tiles, S.tc_cost, [&] {
-          launch_update_tc(P, N, h->d_tc + S.tc_off, h->d_tilep_tc + S.ttp_off, S.tc_tiles, 3, h->d_maps,
-                           h->d_err, h->opt.wait_cycles, st);
+      if constexpr (sizeof(T) == 8) {
+        Cost cost = S.panel_cost;
+        cost.flops += S.gemm_cost.flops;
+        cost.bytes += S.gemm_cost.bytes;
+        klaunch(h, st, "macro_panel_f64", S.panel_cnt, cost, [&] {
+          launch_panel64(P, N, h->d_panel + S.panel_off, S.panel_cnt, h->d_panel_sync, h->d_err, eps, pol,
+                         h->opt.wait_cycles, h->d_probs + S.prob_off, h->d_tilep + S.tp_off, S.tiles, st);
         });
+      } else {
+        klaunch(h, st, "macro_panel_f32", S.panel_cnt, S.panel_cost, [&] {
+          launch_macro_panel(P, N, h->d_panel + S.panel_off, S.panel_cnt, h->d_panel_sync, h->d_err, eps, pol,
+                             h->opt.wait_cycles, st);
+        });
+        klaunch(h, st, "update_simt_f32", S.tiles, S.gemm_cost, [&] {
+          launch_gemm_simt<T>(P, N, h->d_probs + S.prob_off, h->d_tilep + S.tp_off, S.tiles, st);
+        });
+        klaunch(h, st, "update_tc_f32", S.tc_tiles, S.tc_cost, [&] {
+          launch_update_tc(P, N, h->d_tc + S.tc_off, h->d_tilep_tc + S.ttp_off, S.tc_tiles, 3, h->d_maps, h->d_err,
+                           h->opt.wait_cycles, st);
+        });
+      }
     }
     klaunch(h, st, f32 ? "update_simt_f32" : "update_simt_f64", L.syrk_tiles, L.syrk_cost, [&] {
       launch_gemm_simt<T>(P, N, h->d_probs + L.syrk_off, h->d_tilep + L.syrk_tp_off, L.syrk_tiles, st);
@@ -2814,8 +2842,8 @@ ncl_status selftest_timeout(ncl_kkt_s* h, DevNum<T>& N, int which, long long wai
     int nrc = 0;
     for (size_t i = 0; i < hs.panelv.size();) {
       const int4 it = hs.panelv[i];
-      const int qe = std::min(it.y + MACRO_NB, (int)P.sn_ncol[it.x]);
-      const int n = (P.sn_nrow[it.x] - qe + MACRO_ROWS - 1) / MACRO_ROWS;
+      const int qe = std::min(it.y + panel_cols(sizeof(T)), (int)P.sn_ncol[it.x]);
+      const int n = (P.sn_nrow[it.x] - qe + panel_rows(sizeof(T)) - 1) / panel_rows(sizeof(T));
       if (n >= 1) {
         g0 = (int64_t)i;
         nrc = n;
@@ -2828,8 +2856,12 @@ ncl_status selftest_timeout(ncl_kkt_s* h, DevNum<T>& N, int which, long long wai
     CK(cudaMemcpyAsync(h->d_panel_sync + hs.panelv[g0].z, &one, sizeof(int), cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
     g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
-    launch_macro_panel<T>(h->dp, N, h->d_panel + g0, nrc, h->d_panel_sync, h->d_err,
-                          h->opt.pivot_eps, h->opt.pivot_policy, wait, st);
+    if constexpr (sizeof(T) == 8)
+      launch_panel64(h->dp, N, h->d_panel + g0, nrc, h->d_panel_sync, h->d_err, h->opt.pivot_eps,
+                     h->opt.pivot_policy, wait, nullptr, nullptr, 0, st);
+    else
+      launch_macro_panel(h->dp, N, h->d_panel + g0, nrc, h->d_panel_sync, h->d_err, h->opt.pivot_eps,
+                         h->opt.pivot_policy, wait, st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&herr, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));

@@ -14,6 +14,7 @@
 #include "runtime.h"
 #include "pivot.cuh"
 #include "reduce.cuh"
+#include "simt_tile.cuh"
 
 #include <math_constants.h>
 
@@ -230,115 +231,12 @@ void launch_assemble(const DevPlan& P, const DevNum<T>& N, const int2* items, co
   k_assemble<T><<<count, 256, 0, st>>>(P, N, items, cptr, cran);
 }
 
-// ---------------------------------------------------------------------------
-// SIMT update C -= A diag(d) B^T (lower part), 64 x 64 tiles, 256 threads,
-// 4 x 4 outputs per thread: rows 4 ty .. 4 ty + 3 (one 16-byte shared load
-// of A per k) and columns tx + 16 b (four conflict-free loads of B, and
-// coalesced row segments of C).  FP64 uses DFMA, FP32 FFMA.
-// ---------------------------------------------------------------------------
-// four consecutive entries of a 16-byte aligned shared array
-__device__ __forceinline__ void ld4_shared(const float* p, float (&v)[4]) {
-  const float4 x = *reinterpret_cast<const float4*>(p);
-  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-}
-__device__ __forceinline__ void ld4_shared(const double* p, double (&v)[4]) {
-  const double2 x = reinterpret_cast<const double2*>(p)[0], y = reinterpret_cast<const double2*>(p)[1];
-  v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-}
-
-__device__ __forceinline__ void decode_tile(int64_t t, int Nt, int& ti, int& tj) {
-  const int64_t tri = (int64_t)Nt * (Nt + 1) / 2;
-  if (t < tri) {
-    int a = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-    while ((int64_t)a * (a + 1) / 2 > t) a--;
-    while ((int64_t)(a + 1) * (a + 2) / 2 <= t) a++;
-    ti = a;
-    tj = (int)(t - (int64_t)a * (a + 1) / 2);
-  } else {
-    const int64_t u = t - tri;
-    ti = Nt + (int)(u / Nt);
-    tj = (int)(u % Nt);
-  }
-}
-
+// trailing updates outside the tensor cores, a CTA per tile (simt_tile.cuh)
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm_simt(DevPlan P, DevNum<T> N, const GemmProb* __restrict__ probs,
                                                    const int32_t* __restrict__ tile_prob) {
-  constexpr int TB = GEMM_TILE, KC = 16;
-  __shared__ __align__(16) T As[KC][TB + 4];   // rows 16-byte aligned
-  __shared__ T Bs[KC][TB + 1];
-  const int64_t gt = blockIdx.x;
-  const GemmProb pb = probs[tile_prob[gt]];
-  int ti, tj;
-  decode_tile(gt - pb.tile0, pb.Nt, ti, tj);
-  const int i0 = ti * TB, j0 = tj * TB;
-  const T* A = N.L + pb.a_off;
-  const T* B = N.L + pb.b_off;
-  const T* d = N.D + pb.d_off;
-  T* C = (pb.c_in_u ? N.U : N.L) + pb.c_off;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  T acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; a++)
-#pragma unroll
-    for (int b = 0; b < 4; b++) acc[a][b] = T(0);
-  // the next K chunk is fetched into registers while the current one is
-  // multiplied (thread: k = kk, rows rr + 16 q of A and of B)
-  const int kk = threadIdx.x & 15, rr = threadIdx.x >> 4;
-  T fa[4], fb[4];
-  auto fetch = [&](int k0) {
-    const int k = k0 + kk;
-    const bool kin = k < pb.K;
-    const T dk = kin ? d[k] : T(0);
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const int ia = i0 + rr + 16 * q, jb = j0 + rr + 16 * q;
-      fa[q] = (ia < pb.M && kin) ? A[(int64_t)ia * pb.lda + k] : T(0);
-      fb[q] = (jb < pb.N && kin) ? B[(int64_t)jb * pb.lda + k] * dk : T(0);
-    }
-  };
-  fetch(0);
-  for (int k0 = 0; k0 < pb.K; k0 += KC) {
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      As[kk][rr + 16 * q] = fa[q];
-      Bs[kk][rr + 16 * q] = fb[q];
-    }
-    __syncthreads();
-    if (k0 + KC < pb.K) fetch(k0 + KC);
-#pragma unroll
-    for (int k2 = 0; k2 < KC; k2++) {
-      T av[4], bv[4];
-      ld4_shared(&As[k2][4 * ty], av);
-#pragma unroll
-      for (int b = 0; b < 4; b++) bv[b] = Bs[k2][tx + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; a++)
-#pragma unroll
-        for (int b = 0; b < 4; b++) acc[a][b] += av[a] * bv[b];
-    }
-    __syncthreads();
-  }
-  // all 16 loads of C first, then the stores
-  T cv[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; a++) {
-    const int i = i0 + 4 * ty + a;
-#pragma unroll
-    for (int b = 0; b < 4; b++) {
-      const int j = j0 + tx + 16 * b;
-      cv[a][b] = (i < pb.M && j < pb.N && j <= i) ? C[(int64_t)i * pb.ldc + j] : T(0);
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < 4; a++) {
-    const int i = i0 + 4 * ty + a;
-#pragma unroll
-    for (int b = 0; b < 4; b++) {
-      const int j = j0 + tx + 16 * b;
-      if (i < pb.M && j < pb.N && j <= i) C[(int64_t)i * pb.ldc + j] = cv[a][b] - acc[a][b];
-    }
-  }
+  __shared__ __align__(16) SimtTile<T> sh;
+  simt_tile<T>(N, probs, tile_prob, blockIdx.x, sh);
 }
 
 template <typename T>

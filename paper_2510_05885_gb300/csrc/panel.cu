@@ -2,6 +2,7 @@
 // fronts (the roles are in panel_roles.cuh), and whole small fronts.
 #include "panel_roles.cuh"
 #include "panel8.cuh"
+#include "panel64.cuh"
 
 #include <algorithm>
 
@@ -35,18 +36,53 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_macro_panel(Dev
   }
 }
 
+// FP64: one launch per 32-column panel (panel64.cuh).  The first npanel CTAs
+// take the panels' roles as above, each with its own tile's share of the
+// previous panel's update; the other CTAs are the tiles of that update to the
+// right of the panel.  (One to four CTAs per SM, by the shared memory asked
+// for: 11.48, 11.29, 11.29 and 11.30 ms for the whole call, so no more is
+// asked for than is used.)
+__global__ void __launch_bounds__(256) k_panel64(DevPlan P, DevNum<double> N, const int4* __restrict__ items,
+                                                 int npanel, int* sync, int* err, double eps, int policy,
+                                                 long long wait, const GemmProb* __restrict__ probs,
+                                                 const int32_t* __restrict__ tile_prob) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int ticket;
+  if ((int)blockIdx.x >= npanel) {
+    simt_tile<double>(N, probs, tile_prob, blockIdx.x - npanel, *reinterpret_cast<SimtTile<double>*>(smem_raw));
+    return;
+  }
+  Panel64Smem& sh = *reinterpret_cast<Panel64Smem*>(smem_raw);
+  const int4 it = items[blockIdx.x];
+  const int s = it.x, q0 = it.y;
+  int* slot = sync + it.z;
+  if (threadIdx.x == 0) ticket = atomicAdd(slot, 1);
+  __syncthreads();
+  if (ticket == 0)
+    panel_diag_role64(P, N, s, q0, slot + 1, eps, policy, sh);
+  else
+    panel_rows_role64(P, N, s, q0, min(q0 + 32, P.sn_ncol[s]) + 32 * (ticket - 1), slot + 1, err, wait, sh);
+}
+
+void launch_panel64(const DevPlan& P, const DevNum<double>& N, const int4* items, int count, int* sync, int* err,
+                    double eps, int policy, long long wait, const GemmProb* probs, const int32_t* tile_prob,
+                    int64_t tiles, cudaStream_t st) {
+  if (count <= 0) return;
+  static_assert(sizeof(SimtTile<double>) <= sizeof(Panel64Smem), "one size for both");
+  static_assert(sizeof(Panel64Smem) <= 48 * 1024, "no opt-in needed");
+  k_panel64<<<(unsigned)(count + tiles), 256, sizeof(Panel64Smem), st>>>(P, N, items, count, sync, err, eps, policy,
+                                                                         wait, probs, tile_prob);
+}
+
 // Small fronts (ncol <= 64): one CTA factors the pivot columns of the whole
-// front in shared memory by 32-column sub-blocks, as the diagonal-block
-// kernel does: one warp factors the sub-block (factor_sub32; a front's only
-// sub-block is inverted too, for the triangular sweeps), the rows below it are solved by the blocked
-// forward substitution, L21 = F21 L_jj^-T D^-1, and, when a second
-// sub-block follows, the warps update its columns.  The update
-// block F22 -= L21 D1 L21^T is left to the SIMT update kernel, which spreads
-// it over many CTAs.
+// front in shared memory, FP32 eight columns at a time (panel8.cuh), FP64 by
+// 32-column sub-blocks (panel64.cuh); a front's only sub-block is inverted too,
+// for the triangular sweeps.  The update block F22 -= L21 D1 L21^T is left to
+// the SIMT update kernel, which spreads it over many CTAs.
 int small_front_smem(int nrow, int ncp, int esz) {
   if (esz == 4)   // front, panel rows, pivot block and its inverse, pivots, signs and statuses
     return (nrow * panel8_ld(ncp) + (64 + nrow) * P8_LD + 2 * 32 * LDS + 64) * 4 + 128;
-  return (nrow * (ncp + 1) + 2 * 32 * LDS + 64) * esz;
+  return (nrow * (ncp + 1) + 2 * 32 * LDS + 32 + 64 + 64) * esz + 128;
 }
 
 // Write a shared-memory front back.  A pivot block of one sub-block (at most 32
@@ -127,66 +163,20 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_factor_small(DevPlan P, DevNu
     store_front<T>(Lg, F, Iv, ncol, ncol, ncp, ldf);
     return;
   }
-  const int ldf = ncp + 1;   // odd: column accesses by lanes are conflict-free
-  T* F = reinterpret_cast<T*>(smem_raw);
-  T* Ls = F + nrow * ldf;     // the sub-block's unit lower factor, zero padded
-  T* Iv = Ls + 32 * LDS;      // its inverse (fronts of one sub-block)
-  T* dsh = Iv + 32 * LDS;     // pivots
-  T* Lg = N.L + P.sn_Loff[s];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  load_tile(F, ldf, Lg, ncp, nrow, ncp, [](int, int) { return true; });
-  __syncthreads();
-  constexpr int RW = 8;   // rows per register batch of a warp
-  for (int c0 = 0; c0 < ncol; c0 += 32) {
-    const int cw = min(32, ncol - c0);
-    if (warp == 0) {
-      int8_t st;
-      const T d = factor_sub32<T, true>(F + c0 * ldf + c0, ldf, cw, lane < cw ? P.col_sign[col0 + c0 + lane] : 1, eps,
-                                  policy, lane, st);
-      dsh[c0 + lane] = d;
-      if (lane < cw) {
-        N.D[col0 + c0 + lane] = d;
-        N.piv[col0 + c0 + lane] = st;
-      }
-      // the unit lower sub-block, zero above the diagonal and on the padding
-#pragma unroll 4
-      for (int u = 0; u < 32; u++) Ls[lane * LDS + u] = (u < lane && lane < cw) ? F[(c0 + lane) * ldf + c0 + u] : T(0);
-      __syncwarp();
-      if (ncol <= 32) invert_sub32<T>(Ls, Iv, cw, lane);
-    }
-    __syncthreads();
-    // rows below the sub-block: L21 = F21 L_jj^-T D^-1 (blocked forward
-    // substitution, then the scaling)
-    const int rb = c0 + cw;
-    block_trsm32<T>(F + rb * ldf + c0, ldf, nrow - rb, cw, Ls, LDS);
-    __syncthreads();
-    for (int idx = tid; idx < (nrow - rb) * 32; idx += blockDim.x) {
-      const int r = idx >> 5, c = idx & 31;
-      if (c < cw) F[(rb + r) * ldf + c0 + c] /= dsh[c0 + c];
-    }
-    __syncthreads();
-    // update the next sub-block's columns: F[r][c] -= sum_u L[r][u] d_u L[c][u]
-    if (c0 + 32 < ncol) {
-      const int c = c0 + 32 + lane;
-      const bool cok = c < ncol;
-      for (int r0 = c0 + 32 + warp * RW; r0 < nrow; r0 += (SMALL_THREADS / 32) * RW) {
-        T acc[RW];
-#pragma unroll
-        for (int m = 0; m < RW; m++) acc[m] = T(0);
-#pragma unroll 4
-        for (int u = 0; u < 32; u++) {
-          const T b = F[min(c, ncol - 1) * ldf + c0 + u] * dsh[c0 + u];
-#pragma unroll
-          for (int m = 0; m < RW; m++) acc[m] += F[min(r0 + m, nrow - 1) * ldf + c0 + u] * b;
-        }
-#pragma unroll
-        for (int m = 0; m < RW; m++)
-          if (cok && r0 + m < nrow && c <= r0 + m) F[(r0 + m) * ldf + c] -= acc[m];
-      }
-      __syncthreads();
-    }
+  if constexpr (sizeof(T) == 8) {
+    const int ldf = ncp + 1;   // odd: column accesses by lanes are conflict-free
+    double* F = reinterpret_cast<double*>(smem_raw);
+    double* L = F + nrow * ldf;
+    double* Iv = L + 32 * LDS;
+    double* rd = Iv + 32 * LDS;
+    double* ws = rd + 32;
+    double* d = ws + 64;
+    int8_t* sg = reinterpret_cast<int8_t*>(d + 64);
+    double* Lg = N.L + P.sn_Loff[s];
+    load_tile(F, ldf, Lg, ncp, nrow, ncp, [](int, int) { return true; });
+    factor_front64(P, N, F, ldf, nrow, ncol, col0, L, Iv, rd, ws, d, sg, sg + 64, eps, policy);
+    store_front<T>(Lg, F, Iv, nrow, ncol, ncp, ldf);
   }
-  store_front<T>(Lg, F, Iv, nrow, ncol, ncp, ldf);
 }
 
 template <typename T>
@@ -379,31 +369,19 @@ template void launch_factor_small<float>(const DevPlan&, const DevNum<float>&, c
 template void launch_factor_small<double>(const DevPlan&, const DevNum<double>&, const int32_t*, int, int, double,
                                           int, cudaStream_t);
 
-template <typename T, int NB>
-static void launch_macro_panel_nb(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int* sync,
-                                  int* err, double eps, int policy, long long wait, cudaStream_t st) {
-  static bool attr = false;
-  const int smem = macro_panel_smem((int)sizeof(T), NB);
-  if (!attr) {
-    cudaFuncSetAttribute(k_macro_panel<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
-  k_macro_panel<T, NB><<<count, 256, smem, st>>>(P, N, items, sync, err, eps, policy, wait);
-}
-
 // (a 192-column FP32 panel was measured slower than 128 columns on the
 // condensed 300 x 300 and stabilized 700 x 700 grids: the diagonal role's
 // serial chain of 32-column factorisations grows with the width)
-template <typename T>
-void launch_macro_panel(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int* sync, int* err,
+void launch_macro_panel(const DevPlan& P, const DevNum<float>& N, const int4* items, int count, int* sync, int* err,
                         double eps, int policy, long long wait, cudaStream_t st) {
   if (count <= 0) return;
-  launch_macro_panel_nb<T, MACRO_NB>(P, N, items, count, sync, err, eps, policy, wait, st);
+  static bool attr = false;
+  const int smem = macro_panel_smem(4, MACRO_NB);
+  if (!attr) {
+    cudaFuncSetAttribute(k_macro_panel<float, MACRO_NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    attr = true;
+  }
+  k_macro_panel<float, MACRO_NB><<<count, 256, smem, st>>>(P, N, items, sync, err, eps, policy, wait);
 }
-
-template void launch_macro_panel<float>(const DevPlan&, const DevNum<float>&, const int4*, int, int*, int*,
-                                        double, int, long long, cudaStream_t);
-template void launch_macro_panel<double>(const DevPlan&, const DevNum<double>&, const int4*, int, int*, int*,
-                                         double, int, long long, cudaStream_t);
 
 }  // namespace ncl

@@ -83,7 +83,6 @@ inline int macro_panel_smem(int esz, int nb) { return std::max(macro_diag_smem(e
 // division's slow path (pivots are normal numbers: |d| > eps or replaced)
 __device__ __forceinline__ float pivot_rcp(float d) { return __frcp_rn(d); }
 __device__ __forceinline__ double pivot_rcp(double d) { return 1.0 / d; }
-
 // One column step of the 32 x 32 factorisation in registers: rows above the
 // pivot get a zero multiplier, so the update needs no per-column select or
 // branch; entries above a lane's diagonal are never read.

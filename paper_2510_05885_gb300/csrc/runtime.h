@@ -12,7 +12,10 @@ constexpr int ASM_ROWS = 32;      // front rows per assembly CTA
 constexpr int PANEL_NB = 32;      // pivot columns of a diagonal sub-block
 constexpr int MACRO_NB = 128;     // pivot columns per panel of a large front
 constexpr int MACRO_ROWS = 64;    // rows below the macro panel per CTA
-constexpr int GEMM_TILE = 64;     // SIMT update tile (rows x cols)
+// FP64 panels: 32 columns, 32 rows per row CTA (panel64.cuh says why)
+constexpr int panel_cols(int esz) { return esz == 8 ? 32 : MACRO_NB; }
+constexpr int panel_rows(int esz) { return esz == 8 ? 32 : MACRO_ROWS; }
+constexpr int gemm_tile(int esz) { return esz == 8 ? 32 : 64; }   // SIMT update tile (rows x cols)
 constexpr int SOLVE_ROWS = 64;     // rows per partial sum in the no-alloc workspace's size
 constexpr int MAX_RHS_SWEEP = 8;   // right-hand sides per triangular sweep
 constexpr int CHAIN_ROWS = 128;    // pivot rows per CTA of the chained sweeps (FP64), and of an inverted diagonal block
@@ -195,9 +198,12 @@ int small_front_smem(int nrow, int ncp, int esz);
 template <typename T>
 void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
                            int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st);
-template <typename T>
-void launch_macro_panel(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, int* sync, int* err,
+void launch_macro_panel(const DevPlan& P, const DevNum<float>& N, const int4* items, int count, int* sync, int* err,
                         double eps, int policy, long long wait, cudaStream_t st);
+// FP64: the panels and the previous panels' updates to their right
+void launch_panel64(const DevPlan& P, const DevNum<double>& N, const int4* items, int count, int* sync, int* err,
+                    double eps, int policy, long long wait, const GemmProb* probs, const int32_t* tile_prob,
+                    int64_t tiles, cudaStream_t st);
 template <typename T>
 void launch_inertia(const DevPlan& P, const DevNum<T>& N, long long* counts, cudaStream_t st);
 
