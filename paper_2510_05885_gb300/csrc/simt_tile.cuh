@@ -90,8 +90,10 @@ __device__ __forceinline__ void simt_tile(const DevNum<T>& N, const GemmProb* __
     }
     __syncthreads();
     if (k0 + KC < pb.K) fetch(k0 + KC);
-#pragma unroll
-    for (int k2 = 0; k2 < KC; k2++) {
+    // (FP64: the last chunk only as far as it goes, in fours)
+    const int kc = sizeof(T) == 8 ? min(KC, (pb.K - k0 + 3) & ~3) : KC;
+#pragma unroll (sizeof(T) == 8 ? 4 : KC)
+    for (int k2 = 0; k2 < kc; k2++) {
       T av[TM], bv[TM];
       ld_shared(&As[k2][TM * ty], av);
 #pragma unroll

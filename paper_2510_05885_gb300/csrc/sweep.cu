@@ -55,6 +55,8 @@ template <> struct Vec16<double> {
   using type = double2;
   static constexpr int n = 2;
 };
+template <typename T> struct Vec2 { using type = float2; };
+template <> struct Vec2<double> { using type = double2; };
 
 __device__ __forceinline__ SnMeta load_meta(const SnMeta* p) {
   union {
@@ -1020,41 +1022,49 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_fwd_chain(DevPlan P, DevNum<T
 #pragma unroll
     for (int r = 0; r < NR; r++) ts[i * NR + r] = t[0][r];
   }
-  // 16 warps, eight rows each; a lane sums the columns lane, lane + 32, ...
-  // of its rows, and the lanes' sums are added up at the end
-  constexpr int RW = CHAIN_ROWS / (CHAIN_THREADS / 32);
-  T acc[RW][NR];
+  // four lanes to a row: a lane sums the columns 8 j + 2 t, 8 j + 2 t + 1 of
+  // its row (t = lane % 4), so that two additions across lanes end a sum.  (A
+  // warp over a row needs five, at 64 cycles each in FP64, for every row; that
+  // was more than the products: 88 -> 37 us for the levels with more than 128 pivots of the condensed
+  // 100 x 100 grid's root.)  A block's entries are loaded before the wait for
+  // the vector they meet.
+  static_assert(CHAIN_THREADS == 4 * CHAIN_ROWS, "four lanes to a row");
+  const int row = threadIdx.x >> 2, t2 = 2 * (threadIdx.x & 3);
+  const T* Lr = Lb + (int64_t)(row < nr ? row : 0) * m.ncp + t2;
+  using V2 = typename Vec2<T>::type;
+  constexpr int NV = CHAIN_ROWS / 8;
+  V2 l[NV];
+  auto fetch = [&](int c0, bool tri) {
 #pragma unroll
-  for (int k = 0; k < RW; k++)
+    for (int j = 0; j < NV; j++) {
+      l[j] = V2{T(0), T(0)};
+      if (row < nr && (!tri || 8 * j + t2 < row)) l[j] = __ldg(reinterpret_cast<const V2*>(Lr + c0 + 8 * j));
+    }
+  };
+  T acc[NR];
 #pragma unroll
-    for (int r = 0; r < NR; r++) acc[k][r] = T(0);
-  auto product = [&](const T* blk, const T* v, bool tri) {
+  for (int r = 0; r < NR; r++) acc[r] = T(0);
+  auto product = [&](const T* v, bool tri) {
 #pragma unroll
-    for (int c = 0; c < CHAIN_ROWS / 32; c++) {
-      const int col = 32 * c + lane;
-      T l[RW];
-#pragma unroll
-      for (int k = 0; k < RW; k++) {
-        const int i = RW * warp + k;
-        l[k] = (i < nr && (!tri || col < i)) ? __ldg(blk + (int64_t)i * m.ncp + col) : T(0);
-      }
+    for (int j = 0; j < NV; j++) {
+      const int c = 8 * j + t2;
+      const T l1 = !tri || c + 1 < row ? l[j].y : T(0);
 #pragma unroll
       for (int r = 0; r < NR; r++) {
-        const T x = v[col * NR + r];
-#pragma unroll
-        for (int k = 0; k < RW; k++) acc[k][r] += l[k] * x;
+        acc[r] += l[j].x * v[c * NR + r];
+        acc[r] += l1 * v[(c + 1) * NR + r];
       }
     }
   };
   auto reduce = [&] {
 #pragma unroll
-    for (int k = 0; k < RW; k++)
-#pragma unroll
-      for (int r = 0; r < NR; r++)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[k][r] += __shfl_xor_sync(0xffffffffu, acc[k][r], o);
+    for (int r = 0; r < NR; r++) {
+      acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 1);
+      acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 2);
+    }
   };
   for (int J = 0; J < B; J++) {
+    fetch(CHAIN_ROWS * J, false);
     if (threadIdx.x == 0) chain_wait(flags + it.y + J, err, wait);
     __syncthreads();
     for (int i = threadIdx.x; i < CHAIN_ROWS * NR; i += blockDim.x) {
@@ -1062,30 +1072,24 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_fwd_chain(DevPlan P, DevNum<T
       ys[i] = r < nrhs ? __ldcg(yv + (int64_t)(m.col0 + CHAIN_ROWS * J + c) * nrhs + r) : T(0);
     }
     __syncthreads();
-    product(Lb + CHAIN_ROWS * J, ys, false);
+    product(ys, false);
   }
+  fetch(R0, true);
   reduce();
   __syncthreads();
-  if (lane == 0)
+  if (t2 == 0)
 #pragma unroll
-    for (int k = 0; k < RW; k++)
-#pragma unroll
-      for (int r = 0; r < NR; r++) ts[(RW * warp + k) * NR + r] -= acc[k][r];
+    for (int r = 0; r < NR; r++) ts[row * NR + r] -= acc[r];
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < RW; k++)
-#pragma unroll
-    for (int r = 0; r < NR; r++) acc[k][r] = T(0);
-  product(Lb + R0, ts, true);
+  for (int r = 0; r < NR; r++) acc[r] = T(0);
+  product(ts, true);
   reduce();
-  if (lane == 0)
+  if (t2 == 0) {
 #pragma unroll
-    for (int k = 0; k < RW; k++) {
-      const int i = RW * warp + k;
-#pragma unroll
-      for (int r = 0; r < NR; r++) acc[k][r] += ts[i * NR + r];
-      if (i < nr) store_rhs<T, NR>(yv, m.col0 + R0 + i, nrhs, acc[k]);
-    }
+    for (int r = 0; r < NR; r++) acc[r] += ts[row * NR + r];
+    if (row < nr) store_rhs<T, NR>(yv, m.col0 + R0 + row, nrhs, acc);
+  }
   __syncthreads();
   if (threadIdx.x == 0) st_release(flags + it.y + B, 1);
 }
