@@ -145,6 +145,11 @@ struct Pulls {
 // U loads in flight per lane and 32 K rows below staged at a time: many in the
 // level launches, whose time is one warp's; few in the subtree launches, which
 // have more warps than fit and gain more from registers saved.
+// Sums over the lanes go step by step for eight values together: one after the
+// other, each a chain of shuffles, they took longer than the products (a block
+// of 34 pivots 1.7 us for either product, backward 0.65 us; the refined solve
+// of the stabilized 93 x 107 grid 1.06 -> 0.99 ms).
+constexpr int SUMS(int nr, int n) { return nr >= 8 ? 1 : n < 8 / nr ? n : 8 / nr; }
 constexpr int NARROW_K(int nr) { return nr >= 8 ? 2 : 4; }
 constexpr int NARROW_SMEM(int nr, int k) { return (64 + 32 * k) * nr; }   // values per warp
 
@@ -209,10 +214,14 @@ __device__ __forceinline__ void warp_fwd(const DevPlan& P, const DevNum<T>& N, i
 #pragma unroll
       for (int r = 0; r < NR; r++) x[e][r] = src[(v * VW + e) * NR + r];
   };
-  auto row_sum = [&](T (&a)[NR]) {
+  constexpr int B = SUMS(NR, U);
+  static_assert(U % B == 0, "whole batches");
+  auto row_sums = [&](T (&a)[B][NR]) {
     for (int o = vpr >> 1; o > 0; o >>= 1)
 #pragma unroll
-      for (int r = 0; r < NR; r++) a[r] += __shfl_xor_sync(0xffffffffu, a[r], o);
+      for (int u = 0; u < B; u++)
+#pragma unroll
+        for (int r = 0; r < NR; r++) a[u][r] += __shfl_xor_sync(0xffffffffu, a[u][r], o);
   };
   // y = L11^-1 t
   lane_vec(tb);
@@ -221,23 +230,29 @@ __device__ __forceinline__ void warp_fwd(const DevPlan& P, const DevNum<T>& N, i
 #pragma unroll
       for (int u = 0; u < U; u++) li[u] = row_vec((u0 + u) * G + g, m.ncol);
 #pragma unroll
-    for (int u = 0; u < U; u++) {
-      const int i = (u0 + u) * G + g;
-      if ((u0 + u) * G >= m.ncol) break;
-      T a[NR];
+    for (int ub = 0; ub < U; ub += B) {
+      if ((u0 + ub) * G >= m.ncol) break;
+      T a[B][NR];
 #pragma unroll
-      for (int r = 0; r < NR; r++) a[r] = T(0);
+      for (int u = 0; u < B; u++) {
+        const int i = (u0 + ub + u) * G + g;
 #pragma unroll
-      for (int e = 0; e < VW; e++) {
-        const T l = v * VW + e < i ? reinterpret_cast<const T*>(&li[u])[e] : T(0);
+        for (int r = 0; r < NR; r++) a[u][r] = T(0);
 #pragma unroll
-        for (int r = 0; r < NR; r++) a[r] += l * x[e][r];
+        for (int e = 0; e < VW; e++) {
+          const T l = v * VW + e < i ? reinterpret_cast<const T*>(&li[ub + u])[e] : T(0);
+#pragma unroll
+          for (int r = 0; r < NR; r++) a[u][r] += l * x[e][r];
+        }
       }
-      row_sum(a);
-      if (v == 0 && i < m.ncol) {
+      row_sums(a);
 #pragma unroll
-        for (int r = 0; r < NR; r++) ty[i * NR + r] = a[r] += tb[i * NR + r];
-        store_rhs<T, NR>(yv, m.col0 + i, nrhs, a);
+      for (int u = 0; u < B; u++) {
+        const int i = (u0 + ub + u) * G + g;
+        if (v != 0 || i >= m.ncol) continue;
+#pragma unroll
+        for (int r = 0; r < NR; r++) ty[i * NR + r] = a[u][r] += tb[i * NR + r];
+        store_rhs<T, NR>(yv, m.col0 + i, nrhs, a[u]);
       }
     }
   }
@@ -260,21 +275,26 @@ __device__ __forceinline__ void warp_fwd(const DevPlan& P, const DevNum<T>& N, i
 #pragma unroll
         for (int u = 0; u < U; u++) lb[u] = row_vec(m.ncol + c0 + (u0 + u) * G + g, m.nrow);
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        const int a0 = (u0 + u) * G + g;
-        if ((u0 + u) * G >= n) break;
-        T a[NR];
+      for (int ub = 0; ub < U; ub += B) {
+        if ((u0 + ub) * G >= n) break;
+        T a[B][NR];
 #pragma unroll
-        for (int r = 0; r < NR; r++) a[r] = T(0);
+        for (int u = 0; u < B; u++) {
 #pragma unroll
-        for (int e = 0; e < VW; e++)   // (the padding columns of L are zero, and so is y there)
+          for (int r = 0; r < NR; r++) a[u][r] = T(0);
 #pragma unroll
-          for (int r = 0; r < NR; r++) a[r] += reinterpret_cast<const T*>(&lb[u])[e] * x[e][r];
-        row_sum(a);
-        if (v == 0 && a0 < n) {
+          for (int e = 0; e < VW; e++)   // (the padding columns of L are zero, and so is y there)
 #pragma unroll
-          for (int r = 0; r < NR; r++) a[r] = gs[a0 * NR + r] - a[r];
-          store_rhs<T, NR>(W, (int64_t)m.W + c0 + a0, nrhs, a);
+            for (int r = 0; r < NR; r++) a[u][r] += reinterpret_cast<const T*>(&lb[ub + u])[e] * x[e][r];
+        }
+        row_sums(a);
+#pragma unroll
+        for (int u = 0; u < B; u++) {
+          const int a0 = (u0 + ub + u) * G + g;
+          if (v != 0 || a0 >= n) continue;
+#pragma unroll
+          for (int r = 0; r < NR; r++) a[u][r] = gs[a0 * NR + r] - a[u][r];
+          store_rhs<T, NR>(W, (int64_t)m.W + c0 + a0, nrhs, a[u]);
         }
       }
     }
@@ -499,11 +519,15 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
       }
     }
 #pragma unroll
-    for (int k = 0; k < RPT; k++) {
-      const int row = row0 + k * slots + slot;
+    for (int k0 = 0; k0 < RPT; k0 += SUMS(NR, RPT))
       for (int o = tpr >> 1; o > 0; o >>= 1)
 #pragma unroll
-        for (int r = 0; r < NR; r++) acc[k][r] += __shfl_xor_sync(0xffffffffu, acc[k][r], o);
+        for (int k = k0; k < k0 + SUMS(NR, RPT); k++)
+#pragma unroll
+          for (int r = 0; r < NR; r++) acc[k][r] += __shfl_xor_sync(0xffffffffu, acc[k][r], o);
+#pragma unroll
+    for (int k = 0; k < RPT; k++) {
+      const int row = row0 + k * slots + slot;
       if (v0 == 0 && row < end) {
         if (tri) {
 #pragma unroll
