@@ -26,6 +26,8 @@ void launch_adjoint_scalars(const DevPlan& P, const int64_t* inst_n, const int64
 using namespace ncl;
 
 namespace {
+constexpr int N_SM = 152;   // multiprocessors that the schedules are laid out for
+
 
 thread_local std::string g_last_error;
 
@@ -470,7 +472,23 @@ void build_schedule(ncl_kkt_s* h) {
     L.block_off = (int64_t)hs.blockv.size();
     L.chain_off = (int64_t)hs.chainv.size();
     std::vector<int4> prow, brow, bcol, pcol;
-    std::vector<int32_t> large, small;
+    std::vector<int32_t> large, small, wide;
+    // Roles in the sweeps: a warp, a CTA, or strips of CTAs (two launches).  A
+    // warp goes through the entries below the pivots a load's latency for
+    // every 1024 of them, a CTA for every 8192.  That is hidden where other
+    // supernodes fill the chip and is the level's time where they do not:
+    //  - a warp takes up to 4096 entries, 512 where every supernode can have a
+    //    CTA resident (20 x 25: 777 -> 700 us per step, 93 x 107 solve 984 ->
+    //    770 us, with the shorter strips below);
+    //  - a CTA takes up to 48 KB of front where a level has an SM for each
+    //    supernode (96 KB: condensed 100 x 100 2.94 -> 2.85 ms, stabilized 150 x
+    //    150 3.75 -> 3.65 ms), any front otherwise (against 96 KB: 700 x 700
+    //    65.2 -> 62.7 ms, scenarios 42.1 -> 41.0 ms, eight right-hand sides
+    //    11.5 -> 10.8 ms).
+    int nout = 0;   // supernodes outside the subtree region
+    for (int32_t k = P.level_ptr[l]; k < P.level_ptr[l + 1]; k++) nout += !hs.inreg[P.level_list[k]];
+    const int narrow_max = nout <= 4 * N_SM ? 512 : 4096;
+    const int64_t block_max = nout <= N_SM ? SWEEP_BLOCK_BYTES : INT64_MAX;
     for (int32_t k = P.level_ptr[l]; k < P.level_ptr[l + 1]; k++) {
       const int32_t s = P.level_list[k];
       const int nrow = P.sn_nrow[s], ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s];
@@ -491,32 +509,15 @@ void build_schedule(ncl_kkt_s* h) {
         hs.asm_cptr.push_back((int32_t)hs.asm_cran.size());
       }
       if (!reg) {
-        // role in the sweeps: a warp, a CTA, or strips.  A warp streams up to
-        // 4096 entries below its pivots and a CTA 96 KB of front (2 to 3 us
-        // each, hidden by the level's other supernodes); larger fronts are
-        // spread over CTAs, 16 KB to 64 KB of factor to a strip.
         const int nb = nrow - ncol;
-        if (ncol <= 32 && (int64_t)nb * ncp <= 4096) {
+        if (ncol <= 32 && (int64_t)nb * ncp <= narrow_max) {
           hs.narrowv.push_back(s);
-        } else if (ncol <= CHAIN_ROWS && (int64_t)nrow * ncp * (int64_t)esz <= SWEEP_BLOCK_BYTES &&
+        } else if (ncol <= CHAIN_ROWS && (int64_t)nrow * ncp * (int64_t)esz <= block_max &&
                    nb <= SWEEP_BLOCK_BELOW) {
           hs.blockv.push_back(s);
           L.block_below = std::max(L.block_below, nb);
         } else {
-          const int rows = std::max(16, std::min(128, 16384 / ncp / 16 * 16));
-          const bool chain = esz == 8 && ncol > CHAIN_ROWS;
-          for (int r0 = (ncol - 1) / rows * rows; r0 >= 0 && !chain; r0 -= rows) {   // longest rows first
-            prow.push_back(make_int4(s, r0, std::min(r0 + rows, ncol), 0));
-            L.prow.vec = std::max(L.prow.vec, std::min(r0 + rows, ncol));
-          }
-          for (int r0 = ncol; r0 < nrow; r0 += rows) brow.push_back(make_int4(s, r0, std::min(r0 + rows, nrow), 0));
-          for (int j0 = 0; j0 < ncol; j0 += 16) {
-            if (nb > 0) bcol.push_back(make_int4(s, j0, 0, 0));
-            if (!chain) pcol.push_back(make_int4(s, j0, 0, 0));
-          }
-          if (nb > 0) L.brow.vec = std::max(L.brow.vec, ncol);
-          L.bcol.vec = std::max(L.bcol.vec, nb);
-          if (!chain) L.pcol.vec = std::max(L.pcol.vec, ncol);
+          wide.push_back(s);
           if (ncol > CHAIN_ROWS) {
             const int nbr = (ncol + CHAIN_ROWS - 1) / CHAIN_ROWS;
             for (int B = 0; B < nbr; B++) hs.chainv.push_back(make_int2(s, (int32_t)hs.nbrows));
@@ -565,6 +566,32 @@ void build_schedule(ncl_kkt_s* h) {
           hs.inv_cost.bytes += q * esz * w * w;
         }
       }
+    }
+    // strips of rows (forward): each takes sixteen rows at a time, one load's
+    // latency for each, so that a strip is as short as leaves the chip full
+    // (against 16384 entries to every strip: condensed 100 x 100 3.01 -> 2.93 ms
+    // per step, Newton 61 x 83 2.32 -> 2.08 ms; with 2048 to every strip the
+    // staged vector costs: scenarios 42.2 -> 42.9 ms, eight right-hand sides
+    // 11.7 -> 12.2 ms)
+    int64_t wide_entries = 0;
+    for (int32_t s : wide) wide_entries += (int64_t)P.sn_nrow[s] * P.sn_ncolp[s];
+    const int64_t strip = std::min<int64_t>(16384, wide_entries / (4 * N_SM));
+    for (int32_t s : wide) {
+      const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], nb = nrow - ncol;
+      const int rows = std::max(16, std::min(128, (int)(strip / ncp) / 16 * 16));
+      const bool chain = esz == 8 && ncol > CHAIN_ROWS;
+      for (int r0 = (ncol - 1) / rows * rows; r0 >= 0 && !chain; r0 -= rows) {   // longest rows first
+        prow.push_back(make_int4(s, r0, std::min(r0 + rows, ncol), 0));
+        L.prow.vec = std::max(L.prow.vec, std::min(r0 + rows, ncol));
+      }
+      for (int r0 = ncol; r0 < nrow; r0 += rows) brow.push_back(make_int4(s, r0, std::min(r0 + rows, nrow), 0));
+      for (int j0 = 0; j0 < ncol; j0 += 16) {
+        if (nb > 0) bcol.push_back(make_int4(s, j0, 0, 0));
+        if (!chain) pcol.push_back(make_int4(s, j0, 0, 0));
+      }
+      if (nb > 0) L.brow.vec = std::max(L.brow.vec, ncol);
+      L.bcol.vec = std::max(L.bcol.vec, nb);
+      if (!chain) L.pcol.vec = std::max(L.pcol.vec, ncol);
     }
     L.asm_cnt = (int)(asmv.size() - L.asm_off);
     L.small_cnt = (int)(smallv.size() - L.small_off);

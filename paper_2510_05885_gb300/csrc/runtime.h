@@ -21,7 +21,7 @@ constexpr int MAX_RHS_SWEEP = 8;   // right-hand sides per triangular sweep
 constexpr int CHAIN_ROWS = 128;    // pivot rows per CTA of the chained sweeps (FP64), and of an inverted diagonal block
 constexpr int SWEEP_CHUNK_BYTES = 64 * 1024;   // staged vector of a sweep's strip
 constexpr int SWEEP_BLOCK_BELOW = 1024;        // rows below its pivots, at most
-constexpr int SWEEP_BLOCK_BYTES = 96 * 1024;   // front of a supernode swept by one CTA, at most
+constexpr int SWEEP_BLOCK_BYTES = 48 * 1024;   // front of a supernode swept by one CTA, at most, on a level of few
 constexpr int SMALL_SMEM = 64 * 1024;      // front bytes (nrow x ncolp) of a small front, at most
 constexpr int SMALL_SMEM_MAX = 112 * 1024;  // dynamic smem limit of the small-front kernel
 

@@ -13,8 +13,9 @@
 //
 // Roles (a block's role follows from its index):
 //   narrow   at most 32 pivots and a small front: one warp per supernode;
-//   block    at most 128 pivots and a front of at most SWEEP_BLOCK_BYTES: one
-//            CTA of 256 threads per supernode, both steps in one launch;
+//   block    at most 128 pivots and, on a level of few supernodes, a front of
+//            at most SWEEP_BLOCK_BYTES: one CTA of 256 threads per supernode,
+//            both steps in one launch;
 //   strips   larger ones: runs of rows of [L11^-1; L21] (forward) or 16
 //            columns of them (backward) per CTA, one launch for each of the
 //            two steps.
