@@ -95,6 +95,8 @@ struct Level {
   // triangular sweeps: the level's supernodes by role (sweep.cu)
   int64_t narrow_off = 0, block_off = 0;
   int narrow_cnt = 0, block_cnt = 0, block_below = 0;
+  int64_t fblock_off = 0;
+  int fblock_cnt = 0, fblock_below = 0;
   // strips of the large ones: pivot rows and rows below (forward), columns
   // of L21 and of the pivot block (backward); vec: most entries of a strip's
   // vector
@@ -128,7 +130,7 @@ struct HostSched {
   std::vector<int32_t> smallv;
   // triangular sweeps (sweep.cu): supernodes by role, strips of the large ones
   std::vector<int32_t> narrowv, blockv;
-  std::vector<int4> stripv;
+  std::vector<int4> fblockv, stripv;
   std::vector<int2> chainv;               // (supernode, first block-row flag) per block-row of the wide ones
   int64_t nbrows = 0;                     // block-row flags in all
   std::vector<int32_t> asm_cptr;          // per assembly item: its run of child row ranges
@@ -210,6 +212,7 @@ struct ncl_kkt_s {
   int32_t* d_tilep_tc = nullptr;
   int32_t* d_narrow = nullptr;
   int32_t* d_block = nullptr;
+  int4* d_fblock = nullptr;
   int4* d_strips = nullptr;
   int2* d_chain = nullptr;
   int* d_chain_sync = nullptr;              // tickets (fwd, bwd) then flags (fwd, bwd) of the block-rows
@@ -470,25 +473,38 @@ void build_schedule(ncl_kkt_s* h) {
     L.small_off = (int64_t)smallv.size();
     L.narrow_off = (int64_t)hs.narrowv.size();
     L.block_off = (int64_t)hs.blockv.size();
+    L.fblock_off = (int64_t)hs.fblockv.size();
     L.chain_off = (int64_t)hs.chainv.size();
     std::vector<int4> prow, brow, bcol, pcol;
-    std::vector<int32_t> large, small, wide;
-    // Roles in the sweeps: a warp, a CTA, or strips of CTAs (two launches).  A
+    std::vector<int32_t> large, small, mid, wide;
+    // Roles in the sweeps: a warp, a CTA (forward: several, each with a part of
+    // the rows below and the pivot block anew), or strips (two launches).  A
     // warp goes through the entries below the pivots a load's latency for
     // every 1024 of them, a CTA for every 8192.  That is hidden where other
     // supernodes fill the chip and is the level's time where they do not:
     //  - a warp takes up to 4096 entries, 512 where every supernode can have a
     //    CTA resident (20 x 25: 777 -> 700 us per step, 93 x 107 solve 984 ->
     //    770 us, with the shorter strips below);
-    //  - a CTA takes up to 48 KB of front where a level has an SM for each
-    //    supernode (96 KB: condensed 100 x 100 2.94 -> 2.85 ms, stabilized 150 x
-    //    150 3.75 -> 3.65 ms), any front otherwise (against 96 KB: 700 x 700
-    //    65.2 -> 62.7 ms, scenarios 42.1 -> 41.0 ms, eight right-hand sides
-    //    11.5 -> 10.8 ms).
+    //  - a CTA takes up to 48 KB of front on a level with less than 8192
+    //    entries for each SM (96 KB: condensed 100 x 100 2.94 -> 2.85 ms,
+    //    stabilized 150 x 150 3.75 -> 3.65 ms), any front of up to 128 pivots on
+    //    larger ones (against 96 KB: 700 x 700 65.2 -> 62.7 ms, scenarios 42.1
+    //    -> 41.0 ms, eight right-hand sides 11.5 -> 10.8 ms).  (2048, 4096 and
+    //    16384 entries: condensed 100 x 100 2.93, 2.83, 2.85 against 2.83 ms,
+    //    stabilized 150 x 150 3.67, 3.64, 3.65 against 3.62.)
     int nout = 0;   // supernodes outside the subtree region
     for (int32_t k = P.level_ptr[l]; k < P.level_ptr[l + 1]; k++) nout += !hs.inreg[P.level_list[k]];
     const int narrow_max = nout <= 4 * N_SM ? 512 : 4096;
-    const int64_t block_max = nout <= N_SM ? SWEEP_BLOCK_BYTES : INT64_MAX;
+    auto is_narrow = [&](int32_t s) {
+      return P.sn_ncol[s] <= 32 && (int64_t)(P.sn_nrow[s] - P.sn_ncol[s]) * P.sn_ncolp[s] <= narrow_max;
+    };
+    int64_t block_entries = 0;   // of the supernodes that a CTA could take
+    for (int32_t k = P.level_ptr[l]; k < P.level_ptr[l + 1]; k++) {
+      const int32_t s = P.level_list[k];
+      if (!hs.inreg[s] && P.sn_ncol[s] <= CHAIN_ROWS && !is_narrow(s))
+        block_entries += (int64_t)P.sn_nrow[s] * P.sn_ncolp[s];
+    }
+    const int64_t block_max = block_entries <= 8192 * N_SM ? SWEEP_BLOCK_BYTES : INT64_MAX;
     for (int32_t k = P.level_ptr[l]; k < P.level_ptr[l + 1]; k++) {
       const int32_t s = P.level_list[k];
       const int nrow = P.sn_nrow[s], ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s];
@@ -510,11 +526,12 @@ void build_schedule(ncl_kkt_s* h) {
       }
       if (!reg) {
         const int nb = nrow - ncol;
-        if (ncol <= 32 && (int64_t)nb * ncp <= narrow_max) {
+        if (is_narrow(s)) {
           hs.narrowv.push_back(s);
         } else if (ncol <= CHAIN_ROWS && (int64_t)nrow * ncp * (int64_t)esz <= block_max &&
                    nb <= SWEEP_BLOCK_BELOW) {
           hs.blockv.push_back(s);
+          mid.push_back(s);
           L.block_below = std::max(L.block_below, nb);
         } else {
           wide.push_back(s);
@@ -551,7 +568,7 @@ void build_schedule(ncl_kkt_s* h) {
         L.small_cost.bytes += esz * 2.0 * nrow * ncp;
       }
       if (!reg) {
-        const bool strips = !(hs.narrowv.size() && hs.narrowv.back() == s) && !(hs.blockv.size() && hs.blockv.back() == s);
+        const bool strips = !wide.empty() && wide.back() == s;
         Cost& cd = strips ? L.diag_cost : L.one_cost;
         Cost& cb = strips ? L.below_cost : L.one_cost;
         cd.bytes += esz * 0.5 * ncol * (ncol + 1.0);
@@ -573,9 +590,26 @@ void build_schedule(ncl_kkt_s* h) {
     // per step, Newton 61 x 83 2.32 -> 2.08 ms; with 2048 to every strip the
     // staged vector costs: scenarios 42.2 -> 42.9 ms, eight right-hand sides
     // 11.7 -> 12.2 ms)
-    int64_t wide_entries = 0;
+    int64_t wide_entries = 0, mid_entries = 0;
     for (int32_t s : wide) wide_entries += (int64_t)P.sn_nrow[s] * P.sn_ncolp[s];
+    for (int32_t s : mid) mid_entries += (int64_t)P.sn_nrow[s] * P.sn_ncolp[s];
     const int64_t strip = std::min<int64_t>(16384, wide_entries / (4 * N_SM));
+    // rows below per CTA of the block role, forward: an SM's share of the
+    // level, at least 64 (one CTA per supernode: adjoint 8.92 -> 8.78 ms, slack
+    // 6.48 -> 6.40 ms; half or a quarter of the share: eight right-hand sides
+    // 10.7 -> 10.8, 11.1 ms, the pivot blocks are read too often)
+    for (int32_t s : mid) {
+      const int ncol = P.sn_ncol[s], nb = P.sn_nrow[s] - ncol;
+      const int rows = (int)std::min<int64_t>(
+          SWEEP_BLOCK_BELOW, std::max<int64_t>(64, mid_entries / N_SM / P.sn_ncolp[s] / 16 * 16));
+      const int n = std::max(1, (nb + rows - 1) / rows);
+      for (int k = 0; k < n; k++) {
+        const int lo = (int)((int64_t)nb * k / n), hi = (int)((int64_t)nb * (k + 1) / n);
+        hs.fblockv.push_back(make_int4(s, ncol + lo, ncol + hi, 0));
+        L.fblock_below = std::max(L.fblock_below, hi - lo);
+      }
+    }
+    L.fblock_cnt = (int)(hs.fblockv.size() - L.fblock_off);
     for (int32_t s : wide) {
       const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], nb = nrow - ncol;
       const int rows = std::max(16, std::min(128, (int)(strip / ncp) / 16 * 16));
@@ -905,7 +939,19 @@ void build_schedule(ncl_kkt_s* h) {
             bad("block supernode");
         }
       // strips: rows and columns of each large supernode covered exactly once
-      std::vector<int64_t> pr(P.ns, 0), br(P.ns, 0), bc(P.ns, 0), pc(P.ns, 0);
+      std::vector<int64_t> pr(P.ns, 0), br(P.ns, 0), bc(P.ns, 0), pc(P.ns, 0), fb(P.ns, -1);
+      for (const Level& L : h->levels)
+        for (int i = 0; i < L.fblock_cnt; i++) {
+          // a supernode's items follow one another, its first rows first
+          const int4 it = hs.fblockv[L.fblock_off + i];
+          if (it.x < 0 || it.x >= P.ns || hs.inreg[it.x] || P.sn_ncol[it.x] > CHAIN_ROWS ||
+              it.y != (fb[it.x] < 0 ? P.sn_ncol[it.x] : fb[it.x]) || it.z < it.y || it.z > P.sn_nrow[it.x] ||
+              it.z - it.y > std::min(L.fblock_below, SWEEP_BLOCK_BELOW))
+            bad("forward block");
+          fb[it.x] = it.z;
+        }
+      for (int32_t s : hs.blockv)
+        if (fb[s] != P.sn_nrow[s]) bad("forward blocks");
       for (const Level& L : h->levels) {
         auto each = [&](const Level::Strips& S, auto f) {
           if (S.off < 0 || S.off + S.cnt > (int64_t)hs.stripv.size()) bad("strips");
@@ -1313,6 +1359,7 @@ void build_device(ncl_kkt_s* h) {
   h->d_tilep = h->upload(hs.tilep);
   h->d_narrow = h->upload(hs.narrowv);
   h->d_block = h->upload(hs.blockv);
+  h->d_fblock = h->upload(hs.fblockv);
   h->d_strips = h->upload(hs.stripv);
   h->d_chain = h->upload(hs.chainv);
   h->d_chain_sync = h->alloc<int>(2 * (int64_t)P.ns + 2 * hs.nbrows);
@@ -1511,14 +1558,15 @@ void run_sweeps(ncl_kkt_s* h, DevNum<T>& N, int nrhs, cudaStream_t st) {
     return a;
   };
   // one: the level's narrow and block supernodes take part in the launch
-  auto items = [&](const Level& L, const Level::Strips& S, bool one) {
+  auto items = [&](const Level& L, const Level::Strips& S, bool one, bool fwd) {
     SweepItems I{};
     if (one) {
       I.narrow = h->d_narrow + L.narrow_off;
       I.nnarrow = L.narrow_cnt;
       I.block = h->d_block + L.block_off;
-      I.nblock = L.block_cnt;
-      I.block_below = L.block_below;
+      I.fblock = h->d_fblock + L.fblock_off;
+      I.nblock = fwd ? L.fblock_cnt : L.block_cnt;
+      I.block_below = fwd ? L.fblock_below : L.block_below;
     }
     I.strips = h->d_strips + S.off;
     I.nstrips = S.cnt;
@@ -1529,24 +1577,24 @@ void run_sweeps(ncl_kkt_s* h, DevNum<T>& N, int nrhs, cudaStream_t st) {
   // wider than one block-row apart)
   for (const Level& L : h->levels) {
     klaunch(h, st, f32 ? (L.multi ? "fwd_chain_multi_f32" : "fwd_chain_f32") : "fwd_chain_f64",
-            L.narrow_cnt + L.block_cnt + L.prow.cnt, scaled(sum(L.one_cost, L.diag_cost), nrhs),
-            [&] { launch_fwd_level<T>(P, N, items(L, L.prow, true), xp, yv, W, nrhs, f32 || nb == 0, st); });
+            L.narrow_cnt + L.fblock_cnt + L.prow.cnt, scaled(sum(L.one_cost, L.diag_cost), nrhs),
+            [&] { launch_fwd_level<T>(P, N, items(L, L.prow, true, true), xp, yv, W, nrhs, f32 || nb == 0, st); });
     if (!f32)
       klaunch(h, st, "fwd_chain_multi_f64", L.chain_cnt, scaled(L.diag_cost, nrhs), [&] {
         launch_fwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, W, nrhs, tk_f, fl_f, serr,
                             h->opt.wait_cycles, st);
       });
     klaunch(h, st, f32 ? "fwd_below_f32" : "fwd_below_f64", L.brow.cnt, scaled(L.below_cost, nrhs),
-            [&] { launch_fwd_level<T>(P, N, items(L, L.brow, false), xp, yv, W, nrhs, f32 || nb == 0, st); });
+            [&] { launch_fwd_level<T>(P, N, items(L, L.brow, false, true), xp, yv, W, nrhs, f32 || nb == 0, st); });
   }
   for (int l = (int)h->levels.size() - 1; l >= 0; l--) {
     const Level& L = h->levels[l];
     klaunch(h, st, f32 ? "bwd_below_f32" : "bwd_below_f64", L.narrow_cnt + L.block_cnt + L.bcol.cnt,
             scaled(sum(L.one_cost, L.below_cost), nrhs),
-            [&] { launch_bwd_level<T>(P, N, items(L, L.bcol, true), false, xp, yv, nrhs, st); });
+            [&] { launch_bwd_level<T>(P, N, items(L, L.bcol, true, false), false, xp, yv, nrhs, st); });
     klaunch(h, st, f32 ? (L.multi ? "bwd_chain_multi_f32" : "bwd_chain_f32") : "bwd_chain_f64", L.pcol.cnt,
             scaled(L.diag_cost, nrhs),
-            [&] { launch_bwd_level<T>(P, N, items(L, L.pcol, false), true, xp, yv, nrhs, st); });
+            [&] { launch_bwd_level<T>(P, N, items(L, L.pcol, false, false), true, xp, yv, nrhs, st); });
     if (!f32)
       klaunch(h, st, "bwd_chain_multi_f64", L.chain_cnt, scaled(L.diag_cost, nrhs), [&] {
         launch_bwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, nrhs, tk_b, fl_b, serr,

@@ -218,10 +218,11 @@ void launch_invert_merge(const DevPlan& P, const DevNum<float>& N, const int4* i
 // The supernodes of one level launch of a sweep, by role (sweep.cu).
 struct SweepItems {
   const int32_t* narrow;
-  const int32_t* block;
+  const int32_t* block;   // backward
+  const int4* fblock;     // forward: (supernode, first row below its pivots, end row)
   const int4* strips;     // (supernode, first row, end row) forward; (supernode, first column) backward
   int nnarrow, nblock, nstrips;
-  int block_below;        // most rows below a block supernode
+  int block_below;        // most rows below of a block item
   int vec;                // most entries of a strip's staged vector
 };
 

@@ -13,9 +13,10 @@
 //
 // Roles (a block's role follows from its index):
 //   narrow   at most 32 pivots and a small front: one warp per supernode;
-//   block    at most 128 pivots and, on a level of few supernodes, a front of
-//            at most SWEEP_BLOCK_BYTES: one CTA of 256 threads per supernode,
-//            both steps in one launch;
+//   block    at most 128 pivots and, on a level with little work, a front of at
+//            most SWEEP_BLOCK_BYTES: one CTA of 256 threads per supernode, both
+//            steps in one launch; forward, a large front's rows below are dealt
+//            out to several CTAs, each forming y for itself;
 //   strips   larger ones: runs of rows of [L11^-1; L21] (forward) or 16
 //            columns of them (backward) per CTA, one launch for each of the
 //            two steps.
@@ -430,7 +431,7 @@ __device__ __forceinline__ void warp_bwd(const DevPlan& P, const DevNum<T>& N, i
 constexpr int BLOCK_RPT(int nr) { return nr >= 4 ? 4 : 8; }
 
 template <typename T, int NR>
-__device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, int s, const T* xp, T* yv, T* W,
+__device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, const int4 it, const T* xp, T* yv, T* W,
                                           int nrhs, T* smem) {
   using V = typename Vec16<T>::type;
   constexpr int VW = Vec16<T>::n, RPT = BLOCK_RPT(NR), PK = NR >= 4 ? 1 : 2;   // pulled rows per thread at a time
@@ -439,9 +440,9 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
   T* ts = smem;              // [NR][128]
   T* ys = ts + 128 * NR;     // [NR][128]
   T* gs = ys + 128 * NR;     // rows below * NR
-  const SnMeta m = load_meta(P.sn_meta + s);
+  const SnMeta m = load_meta(P.sn_meta + it.x);
   const T* Lb = N.L + m.L;
-  const int nb = m.nrow - m.ncol, tid = threadIdx.x;
+  const int rlo = it.y, nb = it.z - it.y, tid = threadIdx.x;
   const int nv = (m.ncol + VW - 1) / VW;
   int tpr = 4;
   while (tpr < 32 && tpr < nv) tpr *= 2;
@@ -449,7 +450,7 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
   Pulls<T, NR, 1> pt;
   Pulls<T, NR, PK> pb;
   pt.index(P, [&](int) { return tid < m.ncol ? m.rows + tid : (int64_t)-1; });
-  auto below = [&](int k) { return tid + 256 * k < nb ? m.rows + m.ncol + tid + 256 * k : (int64_t)-1; };
+  auto below = [&](int k) { return tid + 256 * k < nb ? m.rows + rlo + tid + 256 * k : (int64_t)-1; };
   pb.index(P, below);
   // the pivot rows' first vectors (FP32: the row's only one for each lane)
   V l[RPT];
@@ -533,19 +534,19 @@ __device__ __forceinline__ void block_fwd(const DevPlan& P, const DevNum<T>& N, 
         if (tri) {
 #pragma unroll
           for (int r = 0; r < NR; r++) ys[r * 128 + row] = acc[k][r] += ts[r * 128 + row];
-          store_rhs<T, NR>(yv, m.col0 + row, nrhs, acc[k]);
+          if (rlo == m.ncol) store_rhs<T, NR>(yv, m.col0 + row, nrhs, acc[k]);
         } else {
 #pragma unroll
-          for (int r = 0; r < NR; r++) acc[k][r] = gs[(row - m.ncol) * NR + r] - acc[k][r];
+          for (int r = 0; r < NR; r++) acc[k][r] = gs[(row - rlo) * NR + r] - acc[k][r];
           store_rhs<T, NR>(W, (int64_t)m.W + row - m.ncol, nrhs, acc[k]);
         }
       }
     }
   };
   for (int r0 = 0; r0 < m.ncol; r0 += RPT * slots) pass(r0, m.ncol, ts, true, r0 == 0);
-  fetch(m.ncol, m.nrow, v0, false);   // (in flight across the barrier)
+  fetch(rlo, it.z, v0, false);   // (in flight across the barrier)
   __syncthreads();
-  for (int r0 = m.ncol; r0 < m.nrow; r0 += RPT * slots) pass(r0, m.nrow, ys, false, r0 == m.ncol);
+  for (int r0 = rlo; r0 < it.z; r0 += RPT * slots) pass(r0, it.z, ys, false, r0 == rlo);
 }
 
 template <typename T, int NR>
@@ -909,7 +910,7 @@ __global__ void __launch_bounds__(256) k_fwd_level(DevPlan P, DevNum<T> N, Sweep
   }
   b -= nw;
   if (b < I.nblock) {
-    block_fwd<T, NR>(P, N, I.block[b], xp, yv, W, nrhs, smem);
+    block_fwd<T, NR>(P, N, I.fblock[b], xp, yv, W, nrhs, smem);
     return;
   }
   strip_fwd<T, NR>(P, N, I.strips[b - I.nblock], xp, yv, W, nrhs, smem,

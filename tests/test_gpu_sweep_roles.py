@@ -1,7 +1,7 @@
-"""Sweep roles that depend on how many supernodes a level has: the same front
-alone (one CTA up to 48 KB, strips beyond; a warp up to 512 entries below the
-pivots), among 153 (one CTA whatever its size) and among 609 (a warp up to 4096
-entries).  Every instance of a batch is solved without refinement; the bound is
+"""Sweep roles that depend on what else a level has: the same front alone (one
+CTA up to 48 KB, strips beyond; a warp up to 512 entries below the pivots),
+among 30 (several CTAs, each with a part of the rows below), among 153 (one CTA
+whatever its size) and among 609 (a warp up to 4096 entries).  Every instance of a batch is solved without refinement; the bound is
 the backward error of LDL^T factors in working precision, 8 n u for these
 diagonally dominant matrices (3 n u times a growth below 2, rounded up).
 """
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec", ["fp32_ir", "fp64"])
-@pytest.mark.parametrize("count,size,border", [(1, 120, 300), (153, 120, 300), (153, 100, 33), (1, 30, 100),
+@pytest.mark.parametrize("count,size,border", [(1, 120, 300), (30, 120, 300), (30, 128, 401), (153, 120, 300), (153, 100, 33), (1, 30, 100),
                                                (609, 30, 100), (609, 9, 40)])
 def test_roles_by_level_size(count, size, border, prec):
     from paper_2510_05885_gb300 import ncl_kkt as nk
