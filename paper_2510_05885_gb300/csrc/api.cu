@@ -362,7 +362,7 @@ void build_schedule(ncl_kkt_s* h) {
     // for the shared-memory front (the subtree factorisation)
     for (int32_t s = 0; s < P.ns; s++)
       hs.inreg[s] = P.sn_ncol[s] <= 32 && P.sn_nrow[s] <= 512 &&
-                    (int64_t)P.sn_nrow[s] * P.sn_ncolp[s] * (int64_t)esz <= SMALL_SMEM;
+                    (int64_t)P.sn_nrow[s] * P.sn_ncolp[s] * (int64_t)esz <= SUBTREE_FRONT;
     // children come before their parent: a supernode outside the region
     // takes its parent out
     for (int32_t s = 0; s < P.ns; s++)
@@ -410,7 +410,7 @@ void build_schedule(ncl_kkt_s* h) {
       hs.regitems.swap(sorted);
     }
     for (int32_t s : hs.regnodes) {
-      hs.reg_smem = std::max<int64_t>(hs.reg_smem, (small_front_smem(P.sn_nrow[s], P.sn_ncolp[s], (int)esz) + 15) / 16 * 16);
+      hs.reg_smem = std::max<int64_t>(hs.reg_smem, (subtree_front_smem(P.sn_nrow[s], P.sn_ncolp[s], (int)esz) + 15) / 16 * 16);
       {
         // subtree factorisation: zero + assemble (L block, update block,
         // children's update blocks), write back, the update block's update
@@ -920,7 +920,7 @@ void build_schedule(ncl_kkt_s* h) {
       if (hs.reg_smem > SMALL_SMEM_MAX) bad("subtree shared memory");
       for (int32_t v = 0; v < P.ns; v++)
         if (hs.inreg[v] && (P.sn_ncol[v] > 32 || P.sn_nrow[v] > 512 ||
-                            small_front_smem(P.sn_nrow[v], P.sn_ncolp[v], (int)esz) > hs.reg_smem))
+                            subtree_front_smem(P.sn_nrow[v], P.sn_ncolp[v], (int)esz) > hs.reg_smem))
           bad("subtree front");
     }
     for (const int2& it : hs.chainv)

@@ -85,6 +85,9 @@ int small_front_smem(int nrow, int ncp, int esz) {
   return (nrow * (ncp + 1) + 2 * 32 * LDS + 32 + 64 + 64) * esz + 128;
 }
 
+// the subtree factorisation's front, pivot block, its inverse, pivots
+int subtree_front_smem(int nrow, int ncp, int esz) { return (nrow * (ncp + 1) + 2 * 32 * LDS + 32) * esz; }
+
 // Write a shared-memory front back.  A pivot block of one sub-block (at most 32
 // columns) is written as its inverse Iv, which the sweeps apply; wider ones
 // are inverted after the factorisation (invert.cu).
@@ -204,11 +207,21 @@ void launch_factor_small(const DevPlan& P, const DevNum<T>& N, const int32_t* li
 //   that land below the pivot columns go to this front's update block in
 //   global memory, zeroed first), the 32-column pivot block is factored by
 //   one warp, the rows below by the blocked substitution, L21 = F21 L11^-T
-//   D1^-1, the factor block written back, and the update block
-//   F22 -= L21 D1 L21^T formed from the shared-memory front.
+//   D1^-1 (one warp inverts the pivot block meanwhile), the factor block
+//   written back, and the update block F22 -= L21 D1 L21^T formed from the
+//   shared-memory front.
 // The children's update blocks were written by the same CTA earlier, so a
 // barrier orders them; nothing waits across CTAs.
+// What bounds it is each front's chain of small steps: half of a warp's time
+// goes to barriers behind the pivot block's warp and to instruction fetches
+// (37 % of the issue slots used, 530 GB/s).  So many fronts run side by side:
+// CTAs of four warps, six to an SM, which the region's limit on a front's size
+// allows (api.cu), and no chain of dependent trips to memory within a front.
+// 700 x 700 7.9 -> 6.2 ms, 64 scenarios 9.1 -> 8.3 ms, 64 uneven instances
+// 1.96 -> 1.49 ms.  (256 threads: 700 x 700 1.4 ms slower, scenarios 2.0 ms.)
 // ---------------------------------------------------------------------------
+constexpr int SUBTREE_THREADS = 128;
+
 template <typename T>
 __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>& N, int s, double eps, int policy,
                                               unsigned char* smem_raw) {
@@ -222,42 +235,72 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
   T* Lg = N.L + P.sn_Loff[s];
   T* Ub = N.U + P.sn_Uoff[s];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  // zero the front and the update block
+  // zero the front and, where children add to it, the update block
+  const int ch0 = P.child_ptr[s], ch1 = P.child_ptr[s + 1];
   for (int idx = tid; idx < nrow * ldf; idx += blockDim.x) F[idx] = T(0);
-  for (int idx = tid; idx < nb * nb; idx += blockDim.x) Ub[idx] = T(0);
+  if (ch1 > ch0)
+    for (int idx = tid; idx < nb * nb; idx += blockDim.x) Ub[idx] = T(0);
   __syncthreads();
   // original entries (each lands in its own position): the front's entries
-  // spread over all threads, so that their loads are independent
+  // spread over all threads, four at a time
   const int64_t rbase = P.sn_rows_off[s];
   {
     const int64_t q0 = P.amap_ptr[rbase], q1 = P.amap_ptr[rbase + nrow];
-    for (int64_t q = q0 + tid; q < q1; q += blockDim.x)
-      F[P.amap_row[q] * ldf + P.amap_col[q]] = (T)N.Klow[P.amap_src[q]];
+    for (int64_t q = q0 + tid; q < q1; q += 4 * blockDim.x) {
+      T v[4];
+      int at[4];
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const int64_t e = q + i * blockDim.x;
+        at[i] = -1;
+        if (e < q1) {
+          at[i] = P.amap_row[e] * ldf + P.amap_col[e];
+          v[i] = (T)N.Klow[P.amap_src[e]];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (at[i] >= 0) F[at[i]] = v[i];
+    }
   }
   // the children's update blocks, child by child (the targets of one child
-  // are distinct: its relative map is increasing); each child's lower
-  // triangle spread over all threads
-  for (int k = P.child_ptr[s]; k < P.child_ptr[s + 1]; k++) {
+  // are distinct: its relative map is increasing): four rows of a child to a
+  // warp, its loads before its stores (the compiler has to take a store for a
+  // possible change of the next load, and one by one each is a trip to L2)
+  for (int k = ch0; k < ch1; k++) {
     __syncthreads();
     const int c = P.child_list[k];
     const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
     const int32_t* rel = P.relmap + P.relmap_off[c];
     const T* Uc = N.U + P.sn_Uoff[c];
-    const int tot = nbc * (nbc + 1) / 2;
-    for (int e = tid; e < tot; e += blockDim.x) {
-      int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-      while (a * (a + 1) / 2 > e) a--;
-      while ((a + 1) * (a + 2) / 2 <= e) a++;
-      const int b = e - a * (a + 1) / 2;
-      const int ra = rel[a], rb = rel[b];
-      const T v = Uc[(int64_t)a * nbc + b];
-      if (rb < ncol) F[ra * ldf + rb] += v;
-      else Ub[(int64_t)(ra - ncol) * nb + (rb - ncol)] += v;
+    for (int a0 = warp; a0 < nbc; a0 += 4 * nw) {
+      int ra[4];
+#pragma unroll
+      for (int i = 0; i < 4; i++) ra[i] = rel[min(a0 + i * nw, nbc - 1)];
+      for (int b = lane; b <= min(a0 + 3 * nw, nbc - 1); b += 32) {
+        const int rb = rel[b];
+        T v[4], t[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const int a = a0 + i * nw;
+          const bool ok = a < nbc && b <= a;
+          v[i] = ok ? Uc[(int64_t)a * nbc + b] : T(0);
+          t[i] = !ok ? T(0) : rb < ncol ? F[ra[i] * ldf + rb] : Ub[(int64_t)(ra[i] - ncol) * nb + (rb - ncol)];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const int a = a0 + i * nw;
+          if (a < nbc && b <= a) {
+            if (rb < ncol) F[ra[i] * ldf + rb] = t[i] + v[i];
+            else Ub[(int64_t)(ra[i] - ncol) * nb + (rb - ncol)] = t[i] + v[i];
+          }
+        }
+      }
     }
   }
   __syncthreads();
   // the pivot block (one 32-column sub-block) by warp 0: LDL^T, pivots,
-  // statuses, the zero-padded unit lower block and its inverse
+  // statuses and the zero-padded unit lower block
   if (warp == 0) {
     int8_t st;
     const T d = factor_sub32<T, true>(F, ldf, ncol, lane < ncol ? P.col_sign[col0 + lane] : 1, eps, policy, lane, st);
@@ -268,22 +311,25 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
     }
 #pragma unroll 4
     for (int u = 0; u < 32; u++) Ls[lane * LDS + u] = (u < lane && lane < ncol) ? F[lane * ldf + u] : T(0);
-    __syncwarp();
-    invert_sub32<T>(Ls, Iv, ncol, lane);
   }
   __syncthreads();
-  // rows below: L21 = F21 L11^-T D1^-1
-  block_trsm32<T>(F + ncol * ldf, ldf, nb, ncol, Ls, LDS);
-  __syncthreads();
-  for (int idx = tid; idx < nb * 32; idx += blockDim.x) {
-    const int r = idx >> 5, c = idx & 31;
-    if (c < ncol) F[(ncol + r) * ldf + c] *= pivot_rcp(dsh[c]);
+  // warp 0: the pivot block's inverse; the others, the rows below: L21 = F21
+  // L11^-T D1^-1
+  if (warp == 0) {
+    invert_sub32<T>(Ls, Iv, ncol, lane);
+  } else {
+    block_trsm32<T>(F + ncol * ldf, ldf, nb, ncol, Ls, LDS, 32, blockDim.x - 32);
+    asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x - 32) : "memory");
+    const T rd = pivot_rcp(dsh[lane]);
+    if (lane < ncol)
+      for (int r = warp - 1; r < nb; r += nw - 1) F[(ncol + r) * ldf + lane] *= rd;
   }
   __syncthreads();
   // write the factor block back, and form the update block from it:
   // 4 x 4 register tiles of its lower triangle spread over all threads
   // (9 shared loads per 16 products), F22[a][b] -= sum_k (L[a][k] d_k) L[b][k]
-  store_front<T>(Lg, F, Iv, nrow, ncol, ncp, ldf);
+  for (int r = warp; r < nrow; r += nw)
+    if (lane < ncp) Lg[(int64_t)r * ncp + lane] = (r < ncol && lane < r) ? Iv[r * LDS + lane] : F[r * ldf + lane];
   const int T4 = (nb + 3) / 4;
   const int ntl = T4 * (T4 + 1) / 2;
   for (int e = tid; e < ntl; e += blockDim.x) {
@@ -312,18 +358,26 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[i][j] += av[i] * bv[j];
     }
+    // (all loads, then all stores)
 #pragma unroll
     for (int i = 0; i < 4; i++)
 #pragma unroll
       for (int j = 0; j < 4; j++) {
         const int a = a0 + i, b = b0 + j;
-        if (a < nb && b <= a) Ub[(int64_t)a * nb + b] -= acc[i][j];
+        acc[i][j] = (ch1 > ch0 && a < nb && b <= a ? Ub[(int64_t)a * nb + b] : T(0)) - acc[i][j];
+      }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int a = a0 + i, b = b0 + j;
+        if (a < nb && b <= a) Ub[(int64_t)a * nb + b] = acc[i][j];
       }
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_subtree_factor(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
+__global__ void __launch_bounds__(SUBTREE_THREADS) k_subtree_factor(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
                                                         int count, const int32_t* __restrict__ nodes, int* counter,
                                                         double eps, int policy) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -353,10 +407,10 @@ void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* ite
   }
   // as many CTAs as fit on the device at once (they take subtrees from a counter)
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_subtree_factor<T>, 256, smem) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_subtree_factor<T>, SUBTREE_THREADS, smem) != cudaSuccess)
     per_sm = 4;
   const int grid = std::min(count, nsm * std::max(per_sm, 1));
-  k_subtree_factor<T><<<grid, 256, smem, st>>>(P, N, items, count, nodes, counter, eps, policy);
+  k_subtree_factor<T><<<grid, SUBTREE_THREADS, smem, st>>>(P, N, items, count, nodes, counter, eps, policy);
 }
 
 template void launch_subtree_factor<float>(const DevPlan&, const DevNum<float>&, const int4*, int, const int32_t*,

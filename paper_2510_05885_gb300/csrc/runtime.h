@@ -23,6 +23,7 @@ constexpr int SWEEP_CHUNK_BYTES = 64 * 1024;   // staged vector of a sweep's str
 constexpr int SWEEP_BLOCK_BELOW = 1024;        // rows below its pivots, at most
 constexpr int SWEEP_BLOCK_BYTES = 48 * 1024;   // front of a supernode swept by one CTA, at most, on a level of few
 constexpr int SMALL_SMEM = 64 * 1024;      // front bytes (nrow x ncolp) of a small front, at most
+constexpr int SUBTREE_FRONT = 16 * 1024;   // front bytes of a front in a small subtree, at most (six CTAs to an SM)
 constexpr int SMALL_SMEM_MAX = 112 * 1024;  // dynamic smem limit of the small-front kernel
 
 // What the sweeps need of a supernode, in one 48-byte record: factor block and
@@ -195,6 +196,7 @@ void launch_gemm_simt(const DevPlan& P, const DevNum<T>& N, const GemmProb* prob
 
 // launchers (panel.cu)
 int small_front_smem(int nrow, int ncp, int esz);
+int subtree_front_smem(int nrow, int ncp, int esz);
 template <typename T>
 void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
                            int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st);
