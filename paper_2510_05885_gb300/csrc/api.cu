@@ -78,6 +78,7 @@ struct Step {                 // one macro panel of every large front of a level
 
 struct Level {
   int64_t asm_off = 0;
+  int64_t asm_smem = 0;
   int asm_cnt = 0;
   int64_t small_off = 0;
   int small_cnt = 0;
@@ -126,7 +127,7 @@ struct Pending {
 std::atomic<int64_t> g_kernel_launches{0};
 
 struct HostSched {
-  std::vector<int2> asmv;
+  std::vector<int4> asmv;                // (supernode, first row, end row, pitch in shared memory or 0)
   std::vector<int32_t> smallv;
   // triangular sweeps (sweep.cu): supernodes by role, strips of the large ones
   std::vector<int32_t> narrowv, blockv;
@@ -134,7 +135,7 @@ struct HostSched {
   std::vector<int2> chainv;               // (supernode, first block-row flag) per block-row of the wide ones
   int64_t nbrows = 0;                     // block-row flags in all
   std::vector<int32_t> asm_cptr;          // per assembly item: its run of child row ranges
-  std::vector<int4> asm_cran;             // (child, alo, ahi, 0)
+  std::vector<AsmChild> asm_cran;
   std::vector<int4> panelv;
   int64_t panel_sync = 0;                 // ints of the panel tickets and sub-block flags
   std::vector<GemmProb> probv;
@@ -201,9 +202,9 @@ struct ncl_kkt_s {
   // schedule
   std::vector<Level> levels;
   HostSched hs;
-  int2* d_asm = nullptr;
+  int4* d_asm = nullptr;
   int32_t* d_asm_cptr = nullptr;
-  int4* d_asm_cran = nullptr;
+  AsmChild* d_asm_cran = nullptr;
   int32_t* d_small = nullptr;
   int4* d_panel = nullptr;
   int* d_panel_sync = nullptr;
@@ -341,7 +342,7 @@ void build_schedule(ncl_kkt_s* h) {
   Plan& P = h->plan;
   const size_t esz = is_fp32(h) ? 4 : 8;
   HostSched& hs = h->hs;
-  std::vector<int2>& asmv = hs.asmv;
+  std::vector<int4>& asmv = hs.asmv;
   std::vector<int32_t>& smallv = hs.smallv;
   std::vector<int4>& panelv = hs.panelv;
   std::vector<GemmProb>& probv = hs.probv;
@@ -509,18 +510,27 @@ void build_schedule(ncl_kkt_s* h) {
       const int32_t s = P.level_list[k];
       const int nrow = P.sn_nrow[s], ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s];
       const bool reg = hs.inreg[s] != 0;   // factored and swept by the subtree kernels
-      for (int r0 = 0; r0 < nrow && !reg; r0 += ASM_ROWS) {
-        asmv.push_back(make_int2(s, r0));
+      for (int r0 = 0, r1; r0 < nrow && !reg; r0 = r1) {
+        // as many rows as fit in shared memory, the longest with r1 entries
+        auto pitch = [](int r) { return (r + 3) / 4 * 4; };
+        r1 = std::min(r0 + ASM_ROWS, nrow);
+        while (r1 > r0 + 1 && (int64_t)(r1 - r0) * pitch(r1) * (int64_t)esz > ASM_SMEM) r1--;
+        int64_t bytes = (int64_t)(r1 - r0) * pitch(r1) * (int64_t)esz;
+        if (bytes > ASM_SMEM) {   // a single row does not: in global memory
+          bytes = 0;
+          r1 = std::min(r0 + ASM_ROWS, nrow);
+        }
+        L.asm_smem = std::max(L.asm_smem, bytes);
+        asmv.push_back(make_int4(s, r0, r1, bytes ? pitch(r1) : 0));
         // rows [alo, ahi) of each child's update block that land on the
         // item's rows [r0, r1) (the relative map is increasing)
-        const int r1 = std::min(r0 + ASM_ROWS, nrow);
         for (int32_t k2 = P.child_ptr[s]; k2 < P.child_ptr[s + 1]; k2++) {
           const int32_t c = P.child_list[k2];
           const int32_t* rel = P.relmap.data() + P.relmap_off[c];
           const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
           const int alo = (int)(std::lower_bound(rel, rel + nbc, r0) - rel);
           const int ahi = (int)(std::lower_bound(rel, rel + nbc, r1) - rel);
-          if (ahi > alo) hs.asm_cran.push_back(make_int4(c, alo, ahi, 0));
+          if (ahi > alo) hs.asm_cran.push_back(AsmChild{P.sn_Uoff[c], P.relmap_off[c], nbc, alo, ahi, c});
         }
         hs.asm_cptr.push_back((int32_t)hs.asm_cran.size());
       }
@@ -998,14 +1008,17 @@ void build_schedule(ncl_kkt_s* h) {
       }
     if (hs.asm_cptr.size() != asmv.size() + 1) bad("assembly child ranges");
     for (size_t i = 0; i < asmv.size(); i++) {
-      const int2 it = asmv[i];
-      if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.y >= P.sn_nrow[it.x]) bad("assembly item");
+      const int4 it = asmv[i];
+      if (it.x < 0 || it.x >= P.ns || it.y < 0 || it.z <= it.y || it.z > P.sn_nrow[it.x] ||
+          (it.w && (it.w < it.z || (int64_t)(it.z - it.y) * it.w * (int64_t)esz > ASM_SMEM)))
+        bad("assembly item");
       if (hs.asm_cptr[i] > hs.asm_cptr[i + 1] || hs.asm_cptr[i + 1] > (int32_t)hs.asm_cran.size())
         bad("assembly child ranges");
       for (int32_t e = hs.asm_cptr[i]; e < hs.asm_cptr[i + 1]; e++) {
-        const int4 cr = hs.asm_cran[e];
-        if (cr.x < 0 || cr.x >= P.ns || P.sn_parent[cr.x] != it.x || cr.y < 0 || cr.y >= cr.z ||
-            cr.z > P.sn_nrow[cr.x] - P.sn_ncol[cr.x])
+        const AsmChild& c = hs.asm_cran[e];
+        if (c.child < 0 || c.child >= P.ns || P.sn_parent[c.child] != it.x || c.alo < 0 || c.alo >= c.ahi ||
+            c.ahi > c.nb || c.nb != P.sn_nrow[c.child] - P.sn_ncol[c.child] || c.U != P.sn_Uoff[c.child] ||
+            c.rel != P.relmap_off[c.child] || P.relmap[c.rel + c.alo] < it.y || P.relmap[c.rel + c.ahi - 1] >= it.z)
           bad("assembly child ranges");
       }
     }
@@ -1465,7 +1478,7 @@ void run_factor(ncl_kkt_s* h, DevNum<T>& N, cudaStream_t st) {
   for (const Level& L : h->levels) {
     klaunch(h, st, f32 ? "assemble_f32" : "assemble_f64", L.asm_cnt, L.asm_cost,
             [&] {
-              launch_assemble<T>(P, N, h->d_asm + L.asm_off, h->d_asm_cptr + L.asm_off, h->d_asm_cran, L.asm_cnt, st);
+              launch_assemble<T>(P, N, h->d_asm + L.asm_off, h->d_asm_cptr + L.asm_off, h->d_asm_cran, L.asm_cnt, (int)L.asm_smem, st);
             });
     klaunch(h, st, f32 ? "factor_small_f32" : "factor_small_f64", L.small_cnt, L.small_cost, [&] {
       launch_factor_small<T>(P, N, h->d_small + L.small_off, L.small_cnt, (int)L.small_smem, eps, pol, st);

@@ -154,81 +154,129 @@ void launch_knorm(const DevPlan& P, const double* Kf, unsigned long long* knorm,
 }
 
 // ---------------------------------------------------------------------------
-// Front assembly.  One CTA per (supernode, run of ASM_ROWS front rows):
-// zero the rows, store the original entries, then add the children's update
-// blocks child by child (a child's rows map to distinct parent rows, so the
-// threads of one child never collide; children are added in a fixed order).
+// Front assembly.  One CTA per (supernode, run of front rows): the rows are
+// put together in shared memory (original entries, then the children's update
+// blocks child by child: a child's rows map to distinct parent rows, so that
+// the threads of one child never collide; children are added in a fixed order)
+// and written once.  What bounds it is the chain of dependent loads on small
+// levels and the traffic on large ones; zeroing and adding in global memory
+// took a trip to L2 and back for each child and moved every entry twice more
+// (condensed 300 x 300 1.69 -> 1.16 ms per factorisation, 700 x 700 4.41 -> 3.17
+// ms, condensed 100 x 100 0.35 -> 0.27 ms).  A CTA's rows fill up to 32 KB (16
+// KB: 700 x 700 59.7 -> 62.5 ms per step; 48 KB: 60.3 ms).  Rows too long for shared memory (pitch 0) are still assembled there.
 // ---------------------------------------------------------------------------
-
 template <typename T>
-__global__ void __launch_bounds__(256) k_assemble(DevPlan P, DevNum<T> N, const int2* __restrict__ items,
-                                                  const int32_t* __restrict__ cptr, const int4* __restrict__ cran) {
-  const int2 it = items[blockIdx.x];
-  const int s = it.x, r0 = it.y;
+__device__ void assemble_global(const DevPlan& P, const DevNum<T>& N, const int4 it, const AsmChild* __restrict__ c0,
+                                const AsmChild* __restrict__ c1) {
+  const int s = it.x, r0 = it.y, r1 = it.z;
   const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s];
   const int nb = nrow - ncol;
-  const int r1 = min(r0 + ASM_ROWS, nrow);
   T* Lb = N.L + P.sn_Loff[s];
   T* Ub = N.U + P.sn_Uoff[s];
-  // zero
-  for (int idx = threadIdx.x; idx < (r1 - r0) * ncp; idx += blockDim.x) Lb[(int64_t)r0 * ncp + idx] = T(0);
-  for (int r = max(r0, ncol); r < r1; r++) {
-    int a = r - ncol;
-    for (int b = threadIdx.x; b <= a; b += blockDim.x) Ub[(int64_t)a * nb + b] = T(0);
-  }
-  __syncthreads();
-  // original entries (each lands in its own position)
-  const int64_t rbase = P.sn_rows_off[s];
-  for (int r = r0 + (threadIdx.x >> 5); r < r1; r += (blockDim.x >> 5)) {
-    int64_t q0 = P.amap_ptr[rbase + r], q1 = P.amap_ptr[rbase + r + 1];
-    for (int64_t q = q0 + (threadIdx.x & 31); q < q1; q += 32)
-      Lb[(int64_t)r * ncp + P.amap_col[q]] = (T)N.Klow[P.amap_src[q]];
-  }
-  // children, in a fixed order: the rows [alo, ahi) of child c's update
-  // block land on this CTA's rows (ranges found on the host).  Loads are
-  // batched four per lane before the read-modify-writes: the targets of one
-  // child row are distinct, and each warp owns whole rows.
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int e = cptr[blockIdx.x]; e < cptr[blockIdx.x + 1]; e++) {
+  for (int idx = threadIdx.x; idx < (r1 - r0) * ncp; idx += blockDim.x) Lb[(int64_t)r0 * ncp + idx] = T(0);
+  for (int r = max(r0, ncol); r < r1; r++)
+    for (int b = threadIdx.x; b <= r - ncol; b += blockDim.x) Ub[(int64_t)(r - ncol) * nb + b] = T(0);
+  __syncthreads();
+  const int64_t rbase = P.sn_rows_off[s];
+  for (int r = r0 + warp; r < r1; r += nw)
+    for (int64_t q = P.amap_ptr[rbase + r] + lane; q < P.amap_ptr[rbase + r + 1]; q += 32)
+      Lb[(int64_t)r * ncp + P.amap_col[q]] = (T)N.Klow[P.amap_src[q]];
+  for (const AsmChild* c = c0; c < c1; c++) {
     __syncthreads();
-    const int4 cr = cran[e];
-    const int c = cr.x, alo = cr.y, ahi = cr.z;
-    const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
-    const int32_t* rel = P.relmap + P.relmap_off[c];
-    const T* Uc = N.U + P.sn_Uoff[c];
-    for (int a = alo + warp; a < ahi; a += nw) {
+    const int32_t* rel = P.relmap + c->rel;
+    for (int a = c->alo + warp; a < c->ahi; a += nw) {
       const int ra = rel[a];
-      const T* urow = Uc + (int64_t)a * nbc;
+      const T* urow = N.U + c->U + (int64_t)a * c->nb;
       T* lrow = Lb + (int64_t)ra * ncp;
       T* urow_p = ra >= ncol ? Ub + (int64_t)(ra - ncol) * nb - ncol : Ub;   // indexed by rb >= ncol
-      for (int b0 = 0; b0 <= a; b0 += 128) {
-        int rb[4];
-        T v[4], old[4];
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-          const int b = b0 + lane + 32 * t;
-          rb[t] = b <= a ? rel[b] : -1;
-          v[t] = b <= a ? urow[b] : T(0);
-        }
-#pragma unroll
-        for (int t = 0; t < 4; t++)
-          if (rb[t] >= 0) old[t] = rb[t] < ncol ? lrow[rb[t]] : urow_p[rb[t]];
-#pragma unroll
-        for (int t = 0; t < 4; t++)
-          if (rb[t] >= 0) {
-            if (rb[t] < ncol) lrow[rb[t]] = old[t] + v[t];
-            else urow_p[rb[t]] = old[t] + v[t];
-          }
+      for (int b = lane; b <= a; b += 32) {
+        const int rb = rel[b];
+        if (rb < ncol) lrow[rb] += urow[b];
+        else urow_p[rb] += urow[b];
       }
     }
   }
 }
 
+// items: (supernode, first row, end row, pitch); cptr: an item's run of cran
 template <typename T>
-void launch_assemble(const DevPlan& P, const DevNum<T>& N, const int2* items, const int32_t* cptr, const int4* cran,
-                     int count, cudaStream_t st) {
+__global__ void __launch_bounds__(256) k_assemble(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
+                                                  const int32_t* __restrict__ cptr,
+                                                  const AsmChild* __restrict__ cran) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* F = reinterpret_cast<T*>(smem_raw);
+  const int4 it = items[blockIdx.x];
+  const int e0 = cptr[blockIdx.x], e1 = cptr[blockIdx.x + 1];
+  const int s = it.x, r0 = it.y, r1 = it.z, pitch = it.w;
+  if (pitch == 0) {
+    assemble_global<T>(P, N, it, cran + e0, cran + e1);
+    return;
+  }
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+  const int ncol = P.sn_ncol[s], ncp = P.sn_ncolp[s], nb = P.sn_nrow[s] - ncol;
+  const int64_t rbase = P.sn_rows_off[s];
+  const int64_t q0 = P.amap_ptr[rbase + r0], q1 = P.amap_ptr[rbase + r1];
+  for (int idx = tid; idx < (r1 - r0) * pitch; idx += 256) F[idx] = T(0);
+  __syncthreads();
+  for (int64_t q = q0 + tid; q < q1; q += 4 * 256) {
+    T v[4];
+    int at[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const int64_t e = q + 256 * i;
+      at[i] = -1;
+      if (e < q1) {
+        at[i] = (P.amap_row[e] - r0) * pitch + P.amap_col[e];
+        v[i] = (T)N.Klow[P.amap_src[e]];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+      if (at[i] >= 0) F[at[i]] = v[i];
+  }
+  for (int e = e0; e < e1; e++) {
+    const AsmChild c = cran[e];
+    const int32_t* rel = P.relmap + c.rel;
+    const T* Uc = N.U + c.U;
+    const int nch = (c.ahi + 127) / 128, nt = (c.ahi - c.alo) * nch;   // 128 entries of a row at a time
+    __syncthreads();
+    for (int t = warp; t < nt; t += nw) {
+      const int a = c.alo + t / nch, b0 = (t - t / nch * nch) * 128;
+      if (b0 > a) continue;
+      T* row = F + (rel[a] - r0) * pitch;
+      const T* urow = Uc + (int64_t)a * c.nb;
+      int rb[4];
+      T v[4];
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const int b = b0 + lane + 32 * i;
+        rb[i] = b <= a ? rel[b] : -1;
+        v[i] = b <= a ? urow[b] : T(0);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (rb[i] >= 0) row[rb[i]] += v[i];
+    }
+  }
+  __syncthreads();
+  T* Lb = N.L + P.sn_Loff[s] + (int64_t)r0 * ncp;
+  for (int i = warp; i < r1 - r0; i += nw) {
+    const int r = r0 + i, len = min(ncol, r + 1);
+    for (int c = lane; c < ncp; c += 32) Lb[(int64_t)i * ncp + c] = c < len ? F[i * pitch + c] : T(0);
+    if (r >= ncol) {
+      T* Ur = N.U + P.sn_Uoff[s] + (int64_t)(r - ncol) * nb;
+      for (int b = lane; b <= r - ncol; b += 32) Ur[b] = F[i * pitch + ncol + b];
+    }
+  }
+}
+
+template <typename T>
+void launch_assemble(const DevPlan& P, const DevNum<T>& N, const int4* items, const int32_t* cptr,
+                     const AsmChild* cran, int count, int smem, cudaStream_t st) {
   if (count <= 0) return;
-  k_assemble<T><<<count, 256, 0, st>>>(P, N, items, cptr, cran);
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k_assemble<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  k_assemble<T><<<count, 256, smem, st>>>(P, N, items, cptr, cran);
 }
 
 // trailing updates outside the tensor cores, a CTA per tile (simt_tile.cuh)
@@ -294,8 +342,8 @@ void launch_inertia(const DevPlan& P, const DevNum<T>& N, long long* counts, cud
 }
 
 #define NCL_INST(T)                                                                                     \
-  template void launch_assemble<T>(const DevPlan&, const DevNum<T>&, const int2*, const int32_t*,       \
-                                   const int4*, int, cudaStream_t);                                     \
+  template void launch_assemble<T>(const DevPlan&, const DevNum<T>&, const int4*, const int32_t*,       \
+                                   const AsmChild*, int, int, cudaStream_t);                            \
   template void launch_gemm_simt<T>(const DevPlan&, const DevNum<T>&, const GemmProb*, const int32_t*,  \
                                     int64_t, cudaStream_t);                                             \
   template void launch_inertia<T>(const DevPlan&, const DevNum<T>&, long long*, cudaStream_t);

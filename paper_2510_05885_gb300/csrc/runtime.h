@@ -8,7 +8,8 @@
 namespace ncl {
 
 // Tile/chunk constants shared by the launch planner and the kernels.
-constexpr int ASM_ROWS = 32;      // front rows per assembly CTA
+constexpr int ASM_ROWS = 32;      // front rows per assembly CTA, at most
+constexpr int ASM_SMEM = 32 * 1024;   // and their bytes
 constexpr int PANEL_NB = 32;      // pivot columns of a diagonal sub-block
 constexpr int MACRO_NB = 128;     // pivot columns per panel of a large front
 constexpr int MACRO_ROWS = 64;    // rows below the macro panel per CTA
@@ -25,6 +26,13 @@ constexpr int SWEEP_BLOCK_BYTES = 48 * 1024;   // front of a supernode swept by 
 constexpr int SMALL_SMEM = 64 * 1024;      // front bytes (nrow x ncolp) of a small front, at most
 constexpr int SUBTREE_FRONT = 16 * 1024;   // front bytes of a front in a small subtree, at most (six CTAs to an SM)
 constexpr int SMALL_SMEM_MAX = 112 * 1024;  // dynamic smem limit of the small-front kernel
+
+// Rows [alo, ahi) of a child's update block, which land on the rows of an
+// assembly item: the block's offset in U, its order, its relative map.
+struct AsmChild {
+  int64_t U, rel;
+  int32_t nb, alo, ahi, child;
+};
 
 // What the sweeps need of a supernode, in one 48-byte record: factor block and
 // row offsets, first entry of W, first pivot, sizes.
@@ -185,8 +193,8 @@ void launch_slack_step(const DevPlan& P, const double* Jv, const double* rho, co
 void launch_full_values(const DevPlan& P, const double* Klow, double* Kf, int64_t nnzF, cudaStream_t st);
 void launch_knorm(const DevPlan& P, const double* Kf, unsigned long long* knorm, cudaStream_t st);
 template <typename T>
-void launch_assemble(const DevPlan& P, const DevNum<T>& N, const int2* items, const int32_t* cptr, const int4* cran,
-                     int count, cudaStream_t st);
+void launch_assemble(const DevPlan& P, const DevNum<T>& N, const int4* items, const int32_t* cptr,
+                     const AsmChild* cran, int count, int smem, cudaStream_t st);
 template <typename T>
 void launch_factor_small(const DevPlan& P, const DevNum<T>& N, const int32_t* list, int count, int smem_bytes,
                          double eps, int policy, cudaStream_t st);
