@@ -161,17 +161,25 @@ template void launch_invert_diag<double>(const DevPlan&, const DevNum<double>&, 
 // tile of T (SECOND = false, stored transposed above the diagonal) or of X,
 // 8 x 4 outputs per thread, the operands' next 16 columns fetched while the
 // current ones are multiplied; the triangular operand's zero part is skipped.
+// FINE: 64 x 32 tiles, 4 x 2 outputs per thread, 32 columns at a time, four
+// CTAs to an item: a launch that does not fill the chip lasts as long as a
+// tile, and a 128 x 64 tile lasts as long as its multiplications, a 64 x 32 one
+// as half as many load latencies (condensed 100 x 100 2.75 -> 2.66 ms per step,
+// stabilized 150 x 150 3.47 -> 3.38 ms).  The products of an entry are summed
+// in the same order either way.
 // ---------------------------------------------------------------------------
-template <bool SECOND>
+template <bool SECOND, bool FINE>
 __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N, const int4* __restrict__ items,
                                                       int h) {
-  constexpr int TM = 128, TN = 64, KC = 16;
+  constexpr int TM = FINE ? 64 : 128, TN = FINE ? 32 : 64, KC = FINE ? 32 : 16, RA = TM / 16, RB = TN / 16;
   __shared__ __align__(16) float As[KC][TM + 4];
   __shared__ __align__(16) float Bs[KC][TN + 4];
-  const int4 it = items[blockIdx.x];
+  const int4 it = items[FINE ? blockIdx.x >> 2 : blockIdx.x];
+  const int sub = FINE ? blockIdx.x & 3 : 0;
   const int ncol = P.sn_ncol[it.x], ncp = P.sn_ncolp[it.x];
-  const int q0 = it.y, i0 = TM * it.z, n0 = TN * it.w;
+  const int q0 = it.y, i0 = 128 * it.z + TM * (sub & 1), n0 = 64 * it.w + TN * (sub >> 1);
   const int m = min(h, ncol - q0 - h);
+  if (FINE && i0 >= m) return;
   float* Lb = N.L + P.sn_Loff[it.x];
   float* low = Lb + (int64_t)(q0 + h) * ncp + q0;        // B, then X
   float* up = Lb + (int64_t)q0 * ncp + q0 + h;           // T transposed: up[n][i]
@@ -179,7 +187,7 @@ __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N
   const float* Ci = Lb + (int64_t)(q0 + h) * ncp + q0 + h;
   // T[i][n] = sum_{k >= n} B[i][k] Ai[k][n];  X[i][n] = -sum_{k <= i} Ci[i][k] T[k][n]
   const int kbeg = SECOND ? 0 : n0, kend = SECOND ? min(m, i0 + TM) : h;
-  const int t = threadIdx.x, ar = t >> 1, ak = (t & 1) * 8;
+  const int t = threadIdx.x, ar = t / (KC / 8), ak = t % (KC / 8) * 8;
   float4 fa[2], fb;
   auto fetch = [&](int k0) {
     const int i = i0 + ar;
@@ -197,7 +205,7 @@ __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N
     }
     fb = make_float4(0.f, 0.f, 0.f, 0.f);
     if (!SECOND) {
-      const int k = k0 + (t >> 4), n = n0 + (t & 15) * 4;
+      const int k = k0 + t / (TN / 4), n = n0 + t % (TN / 4) * 4;
       if (k < kend) {
         fb = __ldg(reinterpret_cast<const float4*>(Ai + (int64_t)k * ncp + n));
         float* f = reinterpret_cast<float*>(&fb);
@@ -205,7 +213,7 @@ __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N
         for (int e = 0; e < 4; e++) f[e] = n + e < k ? f[e] : (n + e == k ? 1.f : 0.f);
       }
     } else {
-      const int n = n0 + (t >> 2), k = k0 + (t & 3) * 4;
+      const int n = n0 + t / (KC / 4), k = k0 + t % (KC / 4) * 4;
       if (k < kend) {
         fb = __ldg(reinterpret_cast<const float4*>(up + (int64_t)n * ncp + k));
         float* f = reinterpret_cast<float*>(&fb);
@@ -214,12 +222,12 @@ __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N
       }
     }
   };
-  const int tx = t & 15, ty = t >> 4;   // outputs: rows 8 ty.., columns 4 tx..
-  float acc[8][4];
+  const int tx = t & 15, ty = t >> 4;   // outputs: rows RA ty.., columns RB tx..
+  float acc[RA][RB];
 #pragma unroll
-  for (int a = 0; a < 8; a++)
+  for (int a = 0; a < RA; a++)
 #pragma unroll
-    for (int b = 0; b < 4; b++) acc[a][b] = 0.f;
+    for (int b = 0; b < RB; b++) acc[a][b] = 0.f;
   fetch(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += KC) {
 #pragma unroll
@@ -227,34 +235,34 @@ __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N
 #pragma unroll
       for (int e = 0; e < 4; e++) As[ak + 4 * q + e][ar] = reinterpret_cast<const float*>(&fa[q])[e];
     if (!SECOND) {
-      *reinterpret_cast<float4*>(&Bs[t >> 4][(t & 15) * 4]) = fb;
+      *reinterpret_cast<float4*>(&Bs[t / (TN / 4)][t % (TN / 4) * 4]) = fb;
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; e++) Bs[(t & 3) * 4 + e][t >> 2] = reinterpret_cast<const float*>(&fb)[e];
+      for (int e = 0; e < 4; e++) Bs[t % (KC / 4) * 4 + e][t / (KC / 4)] = reinterpret_cast<const float*>(&fb)[e];
     }
     __syncthreads();
     if (k0 + KC < kend) fetch(k0 + KC);
 #pragma unroll
     for (int k = 0; k < KC; k++) {
-      const float4 x0 = *reinterpret_cast<const float4*>(&As[k][8 * ty]);
-      const float4 x1 = *reinterpret_cast<const float4*>(&As[k][8 * ty + 4]);
-      const float4 y = *reinterpret_cast<const float4*>(&Bs[k][4 * tx]);
-      const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-      const float ys[4] = {y.x, y.y, y.z, y.w};
+      float xs[RA], ys[RB];
 #pragma unroll
-      for (int a = 0; a < 8; a++)
+      for (int a = 0; a < RA; a += 4) *reinterpret_cast<float4*>(xs + a) = *reinterpret_cast<const float4*>(&As[k][RA * ty + a]);
+      if constexpr (RB == 4) *reinterpret_cast<float4*>(ys) = *reinterpret_cast<const float4*>(&Bs[k][RB * tx]);
+      else *reinterpret_cast<float2*>(ys) = *reinterpret_cast<const float2*>(&Bs[k][RB * tx]);
 #pragma unroll
-        for (int b = 0; b < 4; b++) acc[a][b] = fmaf(xs[a], ys[b], acc[a][b]);
+      for (int a = 0; a < RA; a++)
+#pragma unroll
+        for (int b = 0; b < RB; b++) acc[a][b] = fmaf(xs[a], ys[b], acc[a][b]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 8; a++) {
-    const int i = i0 + 8 * ty + a;
+  for (int a = 0; a < RA; a++) {
+    const int i = i0 + RA * ty + a;
     if (i >= m) break;
 #pragma unroll
-    for (int b = 0; b < 4; b++) {
-      const int n = n0 + 4 * tx + b;
+    for (int b = 0; b < RB; b++) {
+      const int n = n0 + RB * tx + b;
       if (SECOND) low[(int64_t)i * ncp + n] = -acc[a][b];
       else up[(int64_t)n * ncp + i] = acc[a][b];
     }
@@ -264,8 +272,12 @@ __global__ void __launch_bounds__(256) k_invert_merge(DevPlan P, DevNum<float> N
 void launch_invert_merge(const DevPlan& P, const DevNum<float>& N, const int4* items, int count, int h, bool second,
                          cudaStream_t st) {
   if (count <= 0) return;
-  if (second) k_invert_merge<true><<<count, 256, 0, st>>>(P, N, items, h);
-  else k_invert_merge<false><<<count, 256, 0, st>>>(P, N, items, h);
+  // four CTAs to an SM (76, 152, 304, 608 items: slack 200 6.16, 6.11, 6.09, 6.09 ms, condensed 300 12.91, 12.91, 12.87,
+  // 12.85 ms, the others alike)
+  const bool fine = count <= 608;
+  const auto k = second ? (fine ? k_invert_merge<true, true> : k_invert_merge<true, false>)
+                        : (fine ? k_invert_merge<false, true> : k_invert_merge<false, false>);
+  k<<<fine ? 4 * count : count, 256, 0, st>>>(P, N, items, h);
 }
 
 }  // namespace ncl
