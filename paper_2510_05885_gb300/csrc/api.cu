@@ -1472,7 +1472,7 @@ void run_factor(ncl_kkt_s* h, DevNum<T>& N, cudaStream_t st) {
   // one launch): every front below a level launch's fronts is then done
   klaunch(h, st, f32 ? "subtree_factor_f32" : "subtree_factor_f64", (int64_t)h->hs.regitems.size(),
           h->hs.reg_fac_cost, [&] {
-            launch_subtree_factor<T>(P, N, h->d_regitems, (int)h->hs.regitems.size(), h->d_regnodes,
+            launch_subtree_factor<T>(P, N, h->d_regitems, (int)h->hs.regitems.size(), h->d_regnodes, h->d_regbounds,
                                      h->d_dag_cnt + h->hs.dag_counters, (int)h->hs.reg_smem, h->n_sm, eps, pol, st);
           });
   for (const Level& L : h->levels) {

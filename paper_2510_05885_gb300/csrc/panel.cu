@@ -218,7 +218,7 @@ void launch_factor_small(const DevPlan& P, const DevNum<T>& N, const int32_t* li
 // CTAs of four warps, six to an SM, which the region's limit on a front's size
 // allows (api.cu), and no chain of dependent trips to memory within a front.
 // 700 x 700 7.9 -> 6.2 ms, 64 scenarios 9.1 -> 8.3 ms, 64 uneven instances
-// 1.96 -> 1.49 ms.  (256 threads: 700 x 700 1.4 ms slower, scenarios 2.0 ms.)
+// 1.96 -> 1.49 ms (before leaves were done by a warp each, see below).  (256 threads: 700 x 700 1.4 ms slower, scenarios 2.0 ms.)
 // ---------------------------------------------------------------------------
 constexpr int SUBTREE_THREADS = 128;
 
@@ -376,12 +376,105 @@ __device__ __forceinline__ void subtree_front(const DevPlan& P, const DevNum<T>&
   }
 }
 
+// A leaf of a subtree by one warp: the front in shared memory, right-looking with
+// a lane to a row, the pivot block's inverse with a lane to a column, the update
+// block row by row.  Half of the region's fronts are leaves, of 6 pivots and 30
+// rows in the middle: too small for a CTA's barriers, and four at a time wait for
+// memory together (subtree factorisation of 64 scenarios 8.3 -> 5.9 ms, of 64
+// uneven instances 1.49 -> 1.17 ms).  Short loops instead of a 32-column block in
+// registers, whose code would not stay in the instruction cache beside the rest.
+__host__ __device__ inline int leaf_words(int nrow, int ncol, int ncp) {
+  return nrow * (ncp + 1) + ncol * (ncol + 1) + ncol;   // front, inverse, pivots
+}
 template <typename T>
-__global__ void __launch_bounds__(SUBTREE_THREADS) k_subtree_factor(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
-                                                        int count, const int32_t* __restrict__ nodes, int* counter,
+__device__ __forceinline__ void subtree_leaf(const DevPlan& P, const DevNum<T>& N, int s, double eps, int policy, T* F) {
+  const int ncol = P.sn_ncol[s], nrow = P.sn_nrow[s], ncp = P.sn_ncolp[s], col0 = P.sn_col0[s];
+  const int nb = nrow - ncol, ldf = ncp + 1, ldi = ncol + 1, lane = threadIdx.x & 31;
+  T* Iv = F + nrow * ldf;
+  T* ds = Iv + ncol * ldi;
+  T* Lg = N.L + P.sn_Loff[s];
+  T* Ub = N.U + P.sn_Uoff[s];
+  const int64_t rbase = P.sn_rows_off[s];
+  const int64_t q0 = P.amap_ptr[rbase], q1 = P.amap_ptr[rbase + nrow];
+  for (int idx = lane; idx < nrow * ldf; idx += 32) F[idx] = T(0);
+  __syncwarp();
+  for (int64_t q = q0 + lane; q < q1; q += 4 * 32) {
+    T v[4];
+    int at[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const int64_t e = q + 32 * i;
+      at[i] = -1;
+      if (e < q1) {
+        at[i] = P.amap_row[e] * ldf + P.amap_col[e];
+        v[i] = (T)N.Klow[P.amap_src[e]];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+      if (at[i] >= 0) F[at[i]] = v[i];
+  }
+  const int sign = lane < ncol ? P.col_sign[col0 + lane] : 1;
+  int8_t my_st = 0;
+  T my_d = T(1);
+  __syncwarp();
+#pragma unroll 1
+  for (int k = 0; k < ncol; k++) {
+    int8_t st;
+    const T d = static_pivot(F[k * ldf + k], __shfl_sync(0xffffffffu, sign, k), eps, policy, st);
+    const T rd = pivot_rcp(d);
+    if (lane == k) {
+      my_d = d;
+      my_st = st;
+    }
+    // the rows' later columns, with the pivot rows' entries of column k before they are scaled
+    for (int r = k + 1 + lane; r < nrow; r += 32) {
+      const T l = F[r * ldf + k] * rd;
+      const int ce = min(r + 1, ncol);
+#pragma unroll 4
+      for (int c = k + 1; c < ce; c++) F[r * ldf + c] -= l * F[c * ldf + k];
+    }
+    __syncwarp();
+    for (int r = k + 1 + lane; r < nrow; r += 32) F[r * ldf + k] *= rd;
+    __syncwarp();
+  }
+  if (lane < ncol) {
+    ds[lane] = my_d;
+    N.D[col0 + lane] = my_d;
+    N.piv[col0 + lane] = my_st;
+    for (int i = lane + 1; i < ncol; i++) {
+      T a = F[i * ldf + lane];
+      for (int k = lane + 1; k < i; k++) a += F[i * ldf + k] * Iv[k * ldi + lane];
+      Iv[i * ldi + lane] = -a;
+    }
+  }
+  __syncwarp();
+  for (int r = 0; r < nrow; r++)
+    if (lane < ncp)
+      Lg[(int64_t)r * ncp + lane] =
+          r < ncol ? (lane < r ? Iv[r * ldi + lane] : lane == r ? ds[r] : T(0)) : F[r * ldf + lane];
+  for (int a = 0; a < nb; a++)
+    for (int b = lane; b <= a; b += 32) {
+      T acc = T(0);
+#pragma unroll 4
+      for (int k = 0; k < ncol; k++) acc += (F[(ncol + a) * ldf + k] * ds[k]) * F[(ncol + b) * ldf + k];
+      Ub[(int64_t)a * nb + b] = -acc;
+    }
+  __syncwarp();
+}
+
+// items: (first node, nodes, first level bound, levels); the nodes of level 0
+// (leaves) come first, and those that fit a warp's share of the shared memory
+// are done four at a time
+template <typename T>
+__global__ void __launch_bounds__(SUBTREE_THREADS, sizeof(T) == 4 ? 6 : 4) k_subtree_factor(DevPlan P, DevNum<T> N, const int4* __restrict__ items,
+                                                        int count, const int32_t* __restrict__ nodes,
+                                                        const int32_t* __restrict__ bounds, int* counter, int words,
                                                         double eps, int policy) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_item;
+  constexpr int NW = SUBTREE_THREADS / 32;
+  const int warp = threadIdx.x >> 5, share = words / NW;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
@@ -389,8 +482,17 @@ __global__ void __launch_bounds__(SUBTREE_THREADS) k_subtree_factor(DevPlan P, D
     const int it = s_item;
     if (it >= count) break;
     const int4 item = items[it];
+    const int leaves = bounds[item.z + 1];
+    auto fits = [&](int s) { return leaf_words(P.sn_nrow[s], P.sn_ncol[s], P.sn_ncolp[s]) <= share; };
+    for (int q = warp; q < leaves; q += NW) {
+      const int s = nodes[item.x + q];
+      if (fits(s)) subtree_leaf<T>(P, N, s, eps, policy, reinterpret_cast<T*>(smem_raw) + warp * share);
+    }
+    __syncthreads();
     for (int q = 0; q < item.y; q++) {
-      subtree_front<T>(P, N, nodes[item.x + q], eps, policy, smem_raw);
+      const int s = nodes[item.x + q];
+      if (q < leaves && fits(s)) continue;
+      subtree_front<T>(P, N, s, eps, policy, smem_raw);
       __syncthreads();
     }
   }
@@ -398,7 +500,7 @@ __global__ void __launch_bounds__(SUBTREE_THREADS) k_subtree_factor(DevPlan P, D
 
 template <typename T>
 void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
-                           int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st) {
+                           const int32_t* bounds, int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st) {
   if (count <= 0) return;
   static bool attr = false;
   if (!attr) {
@@ -410,13 +512,14 @@ void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* ite
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_subtree_factor<T>, SUBTREE_THREADS, smem) != cudaSuccess)
     per_sm = 4;
   const int grid = std::min(count, nsm * std::max(per_sm, 1));
-  k_subtree_factor<T><<<grid, SUBTREE_THREADS, smem, st>>>(P, N, items, count, nodes, counter, eps, policy);
+  k_subtree_factor<T><<<grid, SUBTREE_THREADS, smem, st>>>(P, N, items, count, nodes, bounds, counter, smem / (int)sizeof(T), eps,
+                                                          policy);
 }
 
 template void launch_subtree_factor<float>(const DevPlan&, const DevNum<float>&, const int4*, int, const int32_t*,
-                                           int*, int, int, double, int, cudaStream_t);
+                                           const int32_t*, int*, int, int, double, int, cudaStream_t);
 template void launch_subtree_factor<double>(const DevPlan&, const DevNum<double>&, const int4*, int, const int32_t*,
-                                            int*, int, int, double, int, cudaStream_t);
+                                            const int32_t*, int*, int, int, double, int, cudaStream_t);
 
 template void launch_factor_small<float>(const DevPlan&, const DevNum<float>&, const int32_t*, int, int, double,
                                          int, cudaStream_t);

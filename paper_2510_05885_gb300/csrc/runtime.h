@@ -206,7 +206,7 @@ void launch_gemm_simt(const DevPlan& P, const DevNum<T>& N, const GemmProb* prob
 int small_front_smem(int nrow, int ncp, int esz);
 int subtree_front_smem(int nrow, int ncp, int esz);
 template <typename T>
-void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes,
+void launch_subtree_factor(const DevPlan& P, const DevNum<T>& N, const int4* items, int count, const int32_t* nodes, const int32_t* bounds,
                            int* counter, int smem, int nsm, double eps, int policy, cudaStream_t st);
 void launch_macro_panel(const DevPlan& P, const DevNum<float>& N, const int4* items, int count, int* sync, int* err,
                         double eps, int policy, long long wait, cudaStream_t st);
