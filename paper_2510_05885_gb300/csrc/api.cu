@@ -438,6 +438,7 @@ void build_schedule(ncl_kkt_s* h) {
   hs.sn_Soff.assign(P.ns, -1);
   hs.sn_flags.assign(P.ns, 0);
   hs.asm_cptr.assign(1, 0);
+  std::vector<int> asm_pos;   // per child of a front: its rows dealt out to assembly items so far
   // problems of one launch are pushed consecutively; each launch's tiles map
   // to its problems through a contiguous run of the per-tile index arrays
   auto push_gemm = [&](GemmProb g, int64_t prob_base, int64_t& tiles, Cost& c) {
@@ -528,8 +529,11 @@ void build_schedule(ncl_kkt_s* h) {
           const int32_t c = P.child_list[k2];
           const int32_t* rel = P.relmap.data() + P.relmap_off[c];
           const int nbc = P.sn_nrow[c] - P.sn_ncol[c];
-          const int alo = (int)(std::lower_bound(rel, rel + nbc, r0) - rel);
-          const int ahi = (int)(std::lower_bound(rel, rel + nbc, r1) - rel);
+          const int alo = r0 == 0 ? 0 : asm_pos[k2 - P.child_ptr[s]];   // where the item before ended
+          int ahi = alo;
+          while (ahi < nbc && rel[ahi] < r1) ahi++;
+          if (r0 == 0 && k2 == P.child_ptr[s]) asm_pos.assign(P.child_ptr[s + 1] - P.child_ptr[s], 0);
+          asm_pos[k2 - P.child_ptr[s]] = ahi;
           if (ahi > alo) hs.asm_cran.push_back(AsmChild{P.sn_Uoff[c], P.relmap_off[c], nbc, alo, ahi, c});
         }
         hs.asm_cptr.push_back((int32_t)hs.asm_cran.size());
