@@ -129,7 +129,7 @@ typedef struct {
     int64_t max_device_bytes; /* 0 = no limit */
     int64_t wait_cycles;      /* bound, in SM clock cycles, of every wait of one CTA
                                  on another inside a kernel (the panel factorisation's
-                                 rows waiting for the diagonal block, the chained
+                                 rows waiting for the diagonal block, the FP64 chained
                                  triangular sweeps, the tensor-core pipeline); past it
                                  the kernel sets an error flag, finishes without the
                                  awaited data and the call returns NCL_ERR_TIMEOUT.
@@ -139,17 +139,20 @@ typedef struct {
                                  and trailing-update tile tasks from a
                                  dependency-ordered list; 0 (default): one launch
                                  per 128-column panel step plus one per trailing
-                                 update (measured a few percent faster on every
-                                 workload of the autotuner's classes) */
+                                 update (FP64: one per 32-column panel, with the
+                                 previous panel's update in it).  Which is faster
+                                 depends on the size class, within a few percent in
+                                 FP32; FP64 is up to twice as fast with 0 */
     double ir_switch;         /* single-instance handles with use_fgmres: Richardson
                                  hands over to FGMRES as soon as a step reduces the
                                  backward error by less than this factor (default
                                  0.5; values outside (0, 1] select it) */
     int32_t subtree_sweeps;   /* 1 (default): every maximal subtree of supernodes with
                                  at most 32 pivots (and a front that fits the
-                                 shared-memory front) is factored by one CTA and, in
-                                 the triangular sweeps, swept by one warp (one launch
-                                 each for all of them, largest subtrees first); 0:
+                                 front of at most 16 KB) is factored by one CTA and, in
+                                 the triangular sweeps, swept by one CTA, a warp to a
+                                 supernode, level by level (one launch each for all of
+                                 them, largest subtrees first); 0:
                                  those supernodes go through the per-level launches
                                  like the others */
     int32_t tc_min_pivots;    /* FP32_IR: large fronts with at least this many pivots
@@ -552,7 +555,8 @@ ncl_status ncl_kkt_selftest_tensor_update(int32_t rows, int32_t ld, int32_t K, c
  *              supernode with more than one block-row (needs a factored
  *              handle); its ticket counter starts past block-row 0, so that
  *              block-row's flag is never published and the next one's CTA
- *              waits for it;
+ *              waits for it (the FP64 sweeps use this kernel; the FP32 ones
+ *              have no waits, and the kernel is there for this test);
  *   which = 1: the first macro panel with rows below it; its ticket counter
  *              starts past the diagonal role, so the row CTAs wait for
  *              sub-block flags that are never published.  The handle's

@@ -6,8 +6,8 @@ of every candidate setting of
 
   persistent_fronts   one persistent launch per level for the large fronts,
                       or one launch per 128-column panel step
-  subtree_sweeps      the small subtrees factored and swept by one CTA /
-                      warp each, or level launches for every supernode
+  subtree_sweeps      the small subtrees factored and swept by one CTA
+                      each, or level launches for every supernode
   tc_min_pivots       the front size from which the FP32 path uses the
                       tensor cores (split TF32) for the dense updates
 

@@ -1,15 +1,17 @@
 // Device roles of the dense front factorisation (internal), shared by the
-// per-step macro-panel kernel (panel.cu) and the persistent front kernel
-// (front_dag.cu): the 32-column sub-block LDL^T, the blocked substitution,
-// the diagonal role and the row role of a 128-column macro panel.
+// per-step macro-panel kernel (panel.cu, FP32; FP64 panels are in panel64.cuh)
+// and the persistent front kernel (front_dag.cu, both precisions): the
+// 32-column sub-block LDL^T, the blocked substitution, the diagonal role and the
+// row role of a 128-column macro panel.
 //
 // The pivot columns of a large front are processed NB = 128 at a time
 // (right-looking blocked LDL^T with D diagonal and static pivoting, Section
 // 3.1).  For macro panel [q0, qe) one launch (k_macro_panel) runs, for every
 // large front of the level:
-//   the diagonal role  one CTA: the w x w diagonal block (w <= 128) is
-//                      factored in shared memory by 32-column sub-blocks,
-//                      each published as soon as it is done;
+//   the diagonal role  one CTA: the w x w diagonal block (w <= 128), FP32
+//                      eight columns at a time with the rest in registers, FP64
+//                      in shared memory by 32-column sub-blocks; each 32
+//                      columns are published as soon as they are done;
 //   the row role       one CTA per 64 rows below the panel: as the
 //                      sub-blocks appear, the blocked forward substitution
 //                      L21 = F21 L11^-T D1^-1; for a tensor-core front also

@@ -32,10 +32,12 @@
 // front row, factor entries as 16-byte vectors with several in flight), and
 // a level's launch overlaps the end of the one before it.  Measured against
 // chained 128-row block-rows with a launch each for the pivot blocks and the
-// rows below: a refined solve of the stabilized 93 x 107 grid 2.54 -> 1.12 ms,
-// of the condensed 300 x 300 grid with 8 right-hand sides 37.3 -> 15.6 ms; the
-// small subtrees' sweep 0.68 -> 0.46 (forward) and 0.71 -> 0.34 ms (backward)
-// at 700 x 700, where one warp used to walk a subtree supernode by supernode.
+// rows below: a refined solve of the stabilized 93 x 107 grid 2.54 -> 0.66 ms,
+// of the condensed 300 x 300 grid with 8 right-hand sides 37.3 -> 10.8 ms (with
+// one role per size of front and interleaved vectors in shared memory: 1.12 and
+// 15.6 ms); the small subtrees' sweep 0.68 -> 0.41 (forward) and 0.71 -> 0.34 ms
+// (backward) at 700 x 700, where one warp used to walk a subtree supernode by
+// supernode.
 #include "runtime.h"
 
 #include <algorithm>
