@@ -275,7 +275,7 @@ template <typename T>
 void launch_assemble(const DevPlan& P, const DevNum<T>& N, const int4* items, const int32_t* cptr,
                      const AsmChild* cran, int count, int smem, cudaStream_t st) {
   if (count <= 0) return;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k_assemble<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static_assert(ASM_SMEM <= 48 * 1024, "no opt-in needed");
   k_assemble<T><<<count, 256, smem, st>>>(P, N, items, cptr, cran);
 }
 

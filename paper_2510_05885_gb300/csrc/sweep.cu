@@ -1255,10 +1255,16 @@ static void by_nrhs(int nrhs, F&& f) {
 
 // a launch that may start before the previous kernel of the stream has ended
 // (the kernel waits itself, see wait_previous); overlap = false: after a
-// memset, an ordinary launch
-template <typename... KA, typename... A>
+// memset, an ordinary launch.  The limit on a kernel's dynamic shared memory
+// belongs to the kernel and the device, not to the launch or the handle: every
+// launch asks for the same one, the most that any launch of the kernel takes,
+// so that threads with a handle each cannot lower it for one another between
+// the request and the launch.  (Errors of either call stay with the thread
+// until the sweeps' cudaGetLastError.)
+template <int SMEM_MAX, typename... KA, typename... A>
 static void launch_overlapped(bool overlap, void (*k)(KA...), int grid, int block, int smem, cudaStream_t st, A... args) {
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static_assert(SMEM_MAX <= 227 * 1024, "a CTA's shared memory");
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1274,13 +1280,20 @@ static void launch_overlapped(bool overlap, void (*k)(KA...), int grid, int bloc
 
 static int level_blocks(const SweepItems& I) { return (I.nnarrow + 7) / 8 + I.nblock + I.nstrips; }
 
-// dynamic shared memory (in values per right-hand side) of a level launch:
-// the roles' needs, the staged vector of `vec` entries at most a chunk
-static int level_smem(const SweepItems& I, int nr, int esz, bool bwd) {
-  int v = I.nnarrow ? 8 * NARROW_SMEM(nr, NARROW_K(nr)) / nr : 0;
-  if (I.nblock) v = std::max(v, (bwd ? 128 + 256 * (16 / esz) : 256) + I.block_below);
-  if (I.nstrips) v = std::max(v, std::min((I.vec + 3) & ~3, SWEEP_CHUNK_BYTES / (nr * esz)) + (bwd ? 8 * 16 : 0));
+// dynamic shared memory of a level launch: the roles' needs, the staged vector
+// of `vec` entries at most a chunk
+static constexpr int level_smem(bool narrow, bool block, bool strips, int block_below, int vec, int nr, int esz, bool bwd) {
+  int v = narrow ? 8 * NARROW_SMEM(nr, NARROW_K(nr)) / nr : 0;   // values per right-hand side
+  if (block) v = std::max(v, (bwd ? 128 + 256 * (16 / esz) : 256) + block_below);
+  if (strips) v = std::max(v, std::min((vec + 3) & ~3, SWEEP_CHUNK_BYTES / (nr * esz)) + (bwd ? 8 * 16 : 0));
   return v * nr * esz;
+}
+static int level_smem(const SweepItems& I, int nr, int esz, bool bwd) {
+  return level_smem(I.nnarrow > 0, I.nblock > 0, I.nstrips > 0, I.block_below, I.vec, nr, esz, bwd);
+}
+// the most a launch takes: every role, a full chunk
+static constexpr int level_smem_max(int nr, int esz, bool bwd) {
+  return level_smem(true, true, true, SWEEP_BLOCK_BELOW, SWEEP_CHUNK_BYTES, nr, esz, bwd);
 }
 
 template <typename T>
@@ -1291,7 +1304,7 @@ void launch_fwd_level(const DevPlan& P, const DevNum<T>& N, const SweepItems& I,
   by_nrhs(nrhs, [&](auto nr) {
     constexpr int NR = decltype(nr)::value;
     const int smem = level_smem(I, NR, sizeof(T), false);
-    launch_overlapped(overlap, k_fwd_level<T, NR>, grid, 256, smem, st, P, N, I, xp, yv, W, nrhs);
+    launch_overlapped<level_smem_max(NR, sizeof(T), false)>(overlap, k_fwd_level<T, NR>, grid, 256, smem, st, P, N, I, xp, yv, W, nrhs);
   });
 }
 
@@ -1303,8 +1316,9 @@ void launch_bwd_level(const DevPlan& P, const DevNum<T>& N, const SweepItems& I,
   by_nrhs(nrhs, [&](auto nr) {
     constexpr int NR = decltype(nr)::value;
     const int smem = level_smem(I, NR, sizeof(T), true);
-    if (piv) launch_overlapped(true, k_bwd_level<T, NR, true>, grid, 256, smem, st, P, N, I, xp, yv, nrhs);
-    else launch_overlapped(true, k_bwd_level<T, NR, false>, grid, 256, smem, st, P, N, I, xp, yv, nrhs);
+    constexpr int most = level_smem_max(NR, sizeof(T), true);
+    if (piv) launch_overlapped<most>(true, k_bwd_level<T, NR, true>, grid, 256, smem, st, P, N, I, xp, yv, nrhs);
+    else launch_overlapped<most>(true, k_bwd_level<T, NR, false>, grid, 256, smem, st, P, N, I, xp, yv, nrhs);
   });
 }
 
