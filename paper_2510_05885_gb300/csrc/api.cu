@@ -1432,6 +1432,41 @@ Cost scaled(Cost c, double f) {
   return c;
 }
 
+// A capture on the handle's private stream, from its begin to end() or, where
+// the captured work throws, to the end of the scope: left open, it would bar
+// this thread from allocating and the handle from capturing again.  Launches
+// counted while it records are taken back (they have not run).
+struct Capture {
+  ncl_kkt_s* h;
+  const int64_t launches0 = g_kernel_launches.load();
+  bool open = false;
+  explicit Capture(ncl_kkt_s* handle) : h(handle) {
+    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+    open = h->capturing = true;
+  }
+  // the recorded graph and its number of this library's launches
+  cudaGraph_t end(int64_t* nodes) {
+    cudaGraph_t g = nullptr;
+    const cudaError_t e = close(&g, nodes);
+    CK(e);
+    return g;
+  }
+  cudaError_t close(cudaGraph_t* g, int64_t* nodes) {
+    open = h->capturing = false;
+    *nodes = g_kernel_launches.load() - launches0;
+    g_kernel_launches.fetch_sub(*nodes);
+    return cudaStreamEndCapture(h->cap_stream, g);
+  }
+  ~Capture() {
+    if (!open) return;
+    cudaGraph_t g = nullptr;
+    int64_t nodes;
+    close(&g, &nodes);
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();   // (the abandoned capture's own)
+  }
+};
+
 // Run `body(stream)` directly, or as a captured graph replayed on `st`.
 // The first call of a kind runs directly (it also loads the kernels), the
 // second captures on the handle's private stream, later calls replay.
@@ -1444,15 +1479,9 @@ void run_graphed(ncl_kkt_s* h, cudaGraphExec_t* exec, int64_t* nodes, int* calls
   }
   if (!*exec && *calls >= 1) {
     // capturing records the work without running it; the graph then runs on st
-    cudaGraph_t g = nullptr;
-    const int64_t l0 = g_kernel_launches.load();
-    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    h->capturing = true;
+    Capture rec(h);
     body(h->cap_stream);
-    h->capturing = false;
-    CK(cudaStreamEndCapture(h->cap_stream, &g));
-    *nodes = g_kernel_launches.load() - l0;
-    g_kernel_launches.fetch_sub(*nodes);
+    const cudaGraph_t g = rec.end(nodes);
     cudaError_t ie = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     CK(ie);
