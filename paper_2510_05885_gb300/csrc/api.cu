@@ -353,6 +353,7 @@ void build_schedule(ncl_kkt_s* h) {
   hs.dag_counters = (int64_t)P.nlevels;   // one queue head per level first
   hs.inv64.clear();
   hs.inv128.clear();
+  hs.inv_cost = hs.merge_cost = Cost{};
   hs.inreg.assign(P.ns, 0);
   hs.regnodes.clear();
   hs.regitems.clear();
@@ -591,10 +592,12 @@ void build_schedule(ncl_kkt_s* h) {
         cb.flops += 2.0 * nb * ncol;
         // inverses: the fronts kept in shared memory with one sub-block have theirs
         if (ncol > 1 && !(is_small && ncol <= 32)) {
-          for (int b = 0; b < ncol; b += CHAIN_ROWS) (ncol <= 64 ? hs.inv64 : hs.inv128).push_back(make_int2(s, b));
-          const double w = std::min(ncol, CHAIN_ROWS), q = (ncol + CHAIN_ROWS - 1) / CHAIN_ROWS;
-          hs.inv_cost.flops += q * w * w * w / 3.0;
-          hs.inv_cost.bytes += q * esz * w * w;
+          for (int b = 0; b < ncol; b += CHAIN_ROWS) {
+            (ncol <= 64 ? hs.inv64 : hs.inv128).push_back(make_int2(s, b));
+            const double w = std::min(ncol - b, CHAIN_ROWS);
+            hs.inv_cost.flops += w * w * w / 3.0;
+            hs.inv_cost.bytes += esz * w * w;
+          }
         }
       }
     }
@@ -864,7 +867,6 @@ void build_schedule(ncl_kkt_s* h) {
   // FP32: merges of the inverted diagonal blocks of 128, 256, ... columns
   hs.mergev.clear();
   hs.merges.clear();
-  hs.inv_cost = hs.merge_cost = Cost{};
   if (is_fp32(h))
     for (int w = CHAIN_ROWS; w < P.max_pivots; w *= 2) {
       HostSched::Merge M{w, (int64_t)hs.mergev.size(), 0};
