@@ -1627,7 +1627,7 @@ void run_sweeps(ncl_kkt_s* h, DevNum<T>& N, int nrhs, cudaStream_t st) {
     klaunch(h, st, f32 ? (L.multi ? "fwd_chain_multi_f32" : "fwd_chain_f32") : "fwd_chain_f64",
             L.narrow_cnt + L.fblock_cnt + L.prow.cnt, scaled(sum(L.one_cost, L.diag_cost), nrhs),
             [&] { launch_fwd_level<T>(P, N, items(L, L.prow, true, true), xp, yv, W, nrhs, f32 || nb == 0, st); });
-    if (!f32)
+    if constexpr (!f32)
       klaunch(h, st, "fwd_chain_multi_f64", L.chain_cnt, scaled(L.diag_cost, nrhs), [&] {
         launch_fwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, W, nrhs, tk_f, fl_f, serr,
                             h->opt.wait_cycles, st);
@@ -1643,9 +1643,9 @@ void run_sweeps(ncl_kkt_s* h, DevNum<T>& N, int nrhs, cudaStream_t st) {
     klaunch(h, st, f32 ? (L.multi ? "bwd_chain_multi_f32" : "bwd_chain_f32") : "bwd_chain_f64", L.pcol.cnt,
             scaled(L.diag_cost, nrhs),
             [&] { launch_bwd_level<T>(P, N, items(L, L.pcol, false, false), true, xp, yv, nrhs, st); });
-    if (!f32)
+    if constexpr (!f32)
       klaunch(h, st, "bwd_chain_multi_f64", L.chain_cnt, scaled(L.diag_cost, nrhs), [&] {
-        launch_bwd_chain<T>(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, nrhs, tk_b, fl_b, serr,
+        launch_bwd_chain(P, N, h->d_chain + L.chain_off, L.chain_cnt, xp, yv, nrhs, tk_b, fl_b, serr,
                             h->opt.wait_cycles, st);
       });
   }

@@ -239,28 +239,6 @@ __device__ __forceinline__ void block_trsm32(T* R, int ldr, int nrows, int ncols
   }
 }
 
-// Copy a tile from shared memory back to global memory (stores where
-// keep(r, c)), 8 shared loads in flight per thread before the stores.
-template <typename T, typename Keep>
-__device__ __forceinline__ void store_tile(T* dst, int64_t ldd, const T* src, int lds, int rows, int cols, Keep keep) {
-  const int n = rows * cols;
-  for (int base = threadIdx.x; base < n; base += 8 * blockDim.x) {
-    T v[8];
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const int idx = min(base + k * blockDim.x, n - 1);
-      const int r = idx / cols, c = idx - r * cols;
-      v[k] = src[r * lds + c];
-    }
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const int idx = base + k * blockDim.x;
-      const int r = idx / cols, c = idx - r * cols;
-      if (idx < n && keep(r, c)) dst[(int64_t)r * ldd + c] = v[k];
-    }
-  }
-}
-
 __device__ __forceinline__ int ld_acquire_i32(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");

@@ -10,7 +10,6 @@ namespace ncl {
 // Tile/chunk constants shared by the launch planner and the kernels.
 constexpr int ASM_ROWS = 32;      // front rows per assembly CTA, at most
 constexpr int ASM_SMEM = 32 * 1024;   // and their bytes
-constexpr int PANEL_NB = 32;      // pivot columns of a diagonal sub-block
 constexpr int MACRO_NB = 128;     // pivot columns per panel of a large front
 constexpr int MACRO_ROWS = 64;    // rows below the macro panel per CTA
 // FP64 panels: 32 columns, 32 rows per row CTA (panel64.cuh says why)
@@ -258,9 +257,8 @@ void launch_region_bwd(const DevPlan& P, const DevNum<T>& N, const int4* items, 
 template <typename T>
 void launch_fwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const T* xp, T* yv,
                       const T* W, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st);
-template <typename T>
-void launch_bwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, T* xp, const T* yv, int nrhs,
-                      int* tickets, int* flags, int* err, long long wait, cudaStream_t st);
+void launch_bwd_chain(const DevPlan& P, const DevNum<double>& N, const int2* items, int count, double* xp,
+                      const double* yv, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st);
 
 // launchers (solve.cu)
 void launch_residual(const DevPlan& P, const double* Kf, const double* B, int64_t ldb, const double* X,

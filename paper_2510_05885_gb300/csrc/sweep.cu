@@ -1340,23 +1340,26 @@ void launch_region_bwd(const DevPlan& P, const DevNum<T>& N, const int4* items, 
   });
 }
 
+// FP32 sweeps have no chains; the FP32 kernel is there for the self-test of a
+// wait that runs out, which has one right-hand side
 template <typename T>
 void launch_fwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, const T* xp, T* yv,
                       const T* W, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st) {
   if (count <= 0) return;
-  by_nrhs(nrhs, [&](auto nr) {
+  auto go = [&](auto nr) {
     k_fwd_chain<T, decltype(nr)::value><<<count, CHAIN_THREADS, 0, st>>>(P, N, items, xp, yv, W, nrhs, tickets, flags,
                                                                          err, wait);
-  });
+  };
+  if constexpr (sizeof(T) == 8) by_nrhs(nrhs, go);
+  else go(std::integral_constant<int, 1>{});
 }
 
-template <typename T>
-void launch_bwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, int count, T* xp, const T* yv, int nrhs,
-                      int* tickets, int* flags, int* err, long long wait, cudaStream_t st) {
+void launch_bwd_chain(const DevPlan& P, const DevNum<double>& N, const int2* items, int count, double* xp,
+                      const double* yv, int nrhs, int* tickets, int* flags, int* err, long long wait, cudaStream_t st) {
   if (count <= 0) return;
   by_nrhs(nrhs, [&](auto nr) {
-    k_bwd_chain<T, decltype(nr)::value><<<count, CHAIN_THREADS, 0, st>>>(P, N, items, xp, yv, nrhs, tickets, flags,
-                                                                         err, wait);
+    k_bwd_chain<double, decltype(nr)::value><<<count, CHAIN_THREADS, 0, st>>>(P, N, items, xp, yv, nrhs, tickets, flags,
+                                                                              err, wait);
   });
 }
 
@@ -1372,9 +1375,7 @@ void launch_bwd_chain(const DevPlan& P, const DevNum<T>& N, const int2* items, i
   template void launch_region_bwd<T>(const DevPlan&, const DevNum<T>&, const int4*, int, const int32_t*,          \
                                      const int32_t*, T*, const T*, int, cudaStream_t);                            \
   template void launch_fwd_chain<T>(const DevPlan&, const DevNum<T>&, const int2*, int, const T*, T*, const T*,   \
-                                    int, int*, int*, int*, long long, cudaStream_t);                              \
-  template void launch_bwd_chain<T>(const DevPlan&, const DevNum<T>&, const int2*, int, T*, const T*, int, int*,  \
-                                    int*, int*, long long, cudaStream_t);
+                                    int, int*, int*, int*, long long, cudaStream_t);
 NCL_INST(float)
 NCL_INST(double)
 #undef NCL_INST
