@@ -148,8 +148,8 @@ typedef struct {
                                  backward error by less than this factor (default
                                  0.5; values outside (0, 1] select it) */
     int32_t subtree_sweeps;   /* 1 (default): every maximal subtree of supernodes with
-                                 at most 32 pivots (and a front that fits the
-                                 front of at most 16 KB) is factored by one CTA and, in
+                                 at most 32 pivots and a front of at most 512 rows
+                                 and 16 KB is factored by one CTA and, in
                                  the triangular sweeps, swept by one CTA, a warp to a
                                  supernode, level by level (one launch each for all of
                                  them, largest subtrees first); 0:
@@ -349,6 +349,13 @@ const char* ncl_kkt_last_error(void);
  * Sigma (n[i] each) and right-hand sides (dim_i rows each, so B is the
  * concatenated dim x nrhs column-major block).  delta and rho are host
  * arrays with one entry per instance.
+ *
+ * Sums have a fixed order, so equal calls on a handle give equal bits as long
+ * as they take the same number of refinement steps and the same precision.  An
+ * instance alone and the same instance in a batch agree to rounding only: how
+ * the sweeps split a supernode, and so the order of their sums, follows the
+ * work of the whole level, and all instances take as many refinement steps as
+ * the one that needs most.
  * ------------------------------------------------------------------------ */
 
 ncl_status ncl_kkt_batch_analyze(int32_t count, int32_t form, const int32_t* n, const int32_t* m,

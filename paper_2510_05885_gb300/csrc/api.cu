@@ -26,8 +26,9 @@ void launch_adjoint_scalars(const DevPlan& P, const int64_t* inst_n, const int64
 using namespace ncl;
 
 namespace {
-constexpr int N_SM = 152;   // multiprocessors that the schedules are laid out for
-
+// multiprocessors that the schedules are laid out for: GB300's, and the same
+// where a handle is analysed without a device
+constexpr int N_SM = 152;
 
 thread_local std::string g_last_error;
 
@@ -1227,7 +1228,8 @@ void build_device(ncl_kkt_s* h) {
     d.wm = h->upload(wm);
     d.wm_list = h->upload(list);
   }
-  // (the no-alloc entry point's size rule counts partial sums per 64 rows below)
+  // (for the no-alloc entry point's documented size rule, which counts partial
+  // sums per 64 rows below; the sweeps have none)
   d.Ptot = 0;
   for (int32_t s = 0; s < P.ns; s++)
     d.Ptot += (int64_t)((P.sn_nrow[s] - P.sn_ncol[s] + SOLVE_ROWS - 1) / SOLVE_ROWS) * P.sn_ncol[s];

@@ -13,9 +13,14 @@
 // (The pivot blocks of at most 32 columns of the fronts kept in shared memory
 // are inverted where they are factored.)  The factorisation itself uses
 // substitution throughout; an error of the inverse only enters the solve's
-// preconditioner, which the FP64 refinement corrects: the backward errors
-// after each refinement step are the same as with substitution in the sweeps
-// (condensed and stabilized grids, penalties 1e4 to 1e7).
+// preconditioner, which the FP64 refinement corrects.  A product with an inverse
+// leaves a larger residual than substitution where L11 is badly conditioned:
+// against block-rows substituted with 32-column inverses, over condensed and
+// stabilized grids and penalties 1e2 to 1e6 (12 to 20 draws each, both
+// precisions), the error of an unrefined solution is 0.8 to 1.25 times as large
+// (geometric means), its backward error 0.65 to 1.5 times, at the condensed
+// form's penalty 1e5 2.2 to 2.6 times (at most 8); 775 refinement steps in all
+// instead of 767.
 #include "runtime.h"
 
 namespace ncl {

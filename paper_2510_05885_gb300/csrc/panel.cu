@@ -199,9 +199,11 @@ void launch_factor_small(const DevPlan& P, const DevNum<T>& N, const int32_t* li
 //
 // The fronts of the small-subtree region (at most 32 pivots, small enough
 // for the shared-memory front, and only such fronts below them) are
-// factored by one CTA per maximal subtree, front by front in postorder, in
-// one launch for the whole region; the level launches of the assembly, the
-// small-front factorisation and the update blocks skip them.  Per front:
+// factored by one CTA per maximal subtree, in one launch for the whole region;
+// the level launches of the assembly, the small-front factorisation and the
+// update blocks skip them.  A subtree's fronts are listed level by level: the
+// leaves that fit a warp's share of the shared memory first, a warp each (see
+// below), then the others one after the other by the whole CTA.  Per front:
 //   the front is assembled straight into shared memory (original entries,
 //   then the children's update blocks child by child; a child's entries
 //   that land below the pivot columns go to this front's update block in
